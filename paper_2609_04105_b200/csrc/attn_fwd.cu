@@ -60,7 +60,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   constexpr uint64_t kDescV = (uint64_t)(16 >> 4) << 16 | (uint64_t)(512 >> 4) << 32 | 1ull << 46 | kSwz64 << 61;
   auto at = [](uint64_t tmpl, uint32_t addr) { return tmpl | (uint64_t)((addr & 0x3FFFFu) >> 4); };
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int qtiles = p.N / BM;
 
   if (threadIdx.x == 0) {
@@ -100,7 +100,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     // ===================================================================== TMA producer
     // The whole warp runs the loop (addresses and waits stay warp-uniform); one elected lane issues.
     int s = 0, ph = 0;
-    uint32_t gs = 0;                                            // stages issued so far (all items)
     uint32_t st = sbase + C::OFF_STAGE;
     bool ok = true;
     int i = 0;
@@ -108,7 +107,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       const WorkItem wi = decode_item<CAUSAL>(item, p, qtiles);
       const int T2 = wi.T2;
       const int qb = i & 1;
-      if (i >= 2) ok = __all_sync(0xffffffffu, mbar_wait(bar(BAR_QFREE0 + qb), ((i >> 1) - 1) & 1, abortf));
+      if (i >= 2) ok = mbar_wait(bar(BAR_QFREE0 + qb), ((i >> 1) - 1) & 1, abortf);
       if (!ok) break;
       if (elect_one()) {
         mbar_arrive_expect_tx(bar(BAR_QFULL0 + qb), C::Q_BYTES + C::QSF_BYTES);
@@ -118,9 +117,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       const uint8_t* ksf = p.k_sf + (size_t)wi.kvh * qtiles * C::KSF_BYTES;
       const uint8_t* vsf = p.v_sf + (size_t)wi.kvh * qtiles * C::VSF_BYTES;
       const int krow0 = wi.kvh * p.N, vrow0 = wi.kvh * D;
-      for (int s2 = 0; s2 < T2; ++s2, ++gs) {
-        if (gs >= (uint32_t)C::NST) ok = __all_sync(0xffffffffu, mbar_wait(bar_empty(s), ph ^ 1, abortf));
-        if (!ok) break;
+      for (int s2 = 0; s2 < T2; ++s2) {
+        if (!mbar_wait(bar_empty(s), ph ^ 1, abortf)) { ok = false; break; }   // (a fresh barrier passes)
         const uint32_t fb = bar_full(s);
         if (elect_one()) {
           mbar_arrive_expect_tx(fb, C::K_BYTES + C::V_BYTES + C::KSF_BYTES + C::VSF_BYTES);
@@ -152,7 +150,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     for (int item = blockIdx.x; ok && item < p.n_items; item += gridDim.x, ++i) {
       const int T2 = decode_item<CAUSAL>(item, p, qtiles).T2;
       const int qb = i & 1;
-      ok = __all_sync(0xffffffffu, mbar_wait(bar(BAR_QFULL0 + qb), (i >> 1) & 1, abortf));
+      ok = mbar_wait(bar(BAR_QFULL0 + qb), (i >> 1) & 1, abortf);
       if (!ok) break;
       tc_fence_after();
       const uint32_t tSFQ = tmem + kColSFQ + 8 * qb;
@@ -164,8 +162,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       for (int s2 = 0; s2 < T2; ++s2, ++g) {
         const int pr = g & 1;
         const uint32_t m = g >> 1;
-        ok = __all_sync(0xffffffffu, mbar_wait(bar_full(sq), phq, abortf));
-        if (ok && m > 0) ok = __all_sync(0xffffffffu, mbar_wait(bar(BAR_SEMPTY0 + pr), (m - 1) & 1, abortf));   // both teams have read the pair
+        ok = mbar_wait(bar_full(sq), phq, abortf);
+        if (ok) ok = mbar_wait(bar(BAR_SEMPTY0 + pr), (m & 1) ^ 1, abortf);   // both teams have read the pair (a fresh barrier passes)
         if (!ok) break;
         tc_fence_after();
         const uint32_t tSFK = tmem + kColSFK + 8 * pr;
@@ -210,13 +208,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     int i = 0;
     for (int item = blockIdx.x; ok && item < p.n_items; item += gridDim.x, ++i) {
       const int T2 = decode_item<CAUSAL>(item, p, qtiles).T2;
-      if (i >= 1) ok = __all_sync(0xffffffffu, mbar_wait(bar(BAR_OFREE), (i - 1) & 1, abortf));   // epilogue has read O
+      if (i >= 1) ok = mbar_wait(bar(BAR_OFREE), (i - 1) & 1, abortf);   // epilogue has read O
       for (int s2 = 0; ok && s2 < T2; ++s2, ++g) {
         const int pr = g & 1;
         const uint32_t m = g >> 1;
         // codes of both tiles are in tensor memory, their scale bytes in shared memory (written by the correction
         // warps, or with a fixed reference by the teams themselves)
-        ok = __all_sync(0xffffffffu, mbar_wait(bar((FIXREF ? BAR_SMDONE0 : BAR_PFULL0) + pr), m & 1, abortf));
+        ok = mbar_wait(bar((FIXREF ? BAR_SMDONE0 : BAR_PFULL0) + pr), m & 1, abortf);
         if (!ok) break;
         tc_fence_after();
         const uint32_t tSFP = tmem + kColSFP + 4 * pr, tSFV = tmem + kColSFV + 8 * pr;
@@ -271,7 +269,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       for (uint32_t g = FIXREF ? g0 + (uint32_t)T2 : g0 + (first_served ? 1u : 0u); g < g0 + (uint32_t)T2; ++g) {
         const bool first_of_item = g == g0;
         const int pr = g & 1;
-        ok = __all_sync(0xffffffffu, mbar_wait(bar(BAR_SMDONE0 + pr), (g >> 1) & 1, abortf));
+        ok = mbar_wait(bar(BAR_SMDONE0 + pr), (g >> 1) & 1, abortf);
         if (!ok) break;
         const int4 me = *reinterpret_cast<const int4*>(sgen + C::OFF_META + C::META_BYTES * pr + row * 16);
         const int Emax = max(max(me.x, me.y), max(me.z, me.w));
@@ -293,7 +291,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             // O holds the item's earlier stages once their PV has landed (an item's first stage never
             // touches O: it may still belong to the previous item)
             const uint32_t gprev = g - 1;
-            ok = __all_sync(0xffffffffu, mbar_wait(bar(BAR_PFREE0 + (gprev & 1)), (gprev >> 1) & 1, abortf));
+            ok = mbar_wait(bar(BAR_PFREE0 + (gprev & 1)), (gprev >> 1) & 1, abortf);
             if (!ok) break;
             tc_fence_after();
 #pragma unroll 1
@@ -321,7 +319,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       if (!ok) break;
       first_served = false;
       // ---- epilogue: with L_hw = column d of the accumulator, O = O_hw / (6 L_hw), LSE = ln2 (mu + log2(L_hw / 6))
-      ok = __all_sync(0xffffffffu, mbar_wait(bar(BAR_OFULL), i & 1, abortf));
+      ok = mbar_wait(bar(BAR_OFULL), i & 1, abortf);
       if (!ok) break;
       tc_fence_after();
       float Lhw;
@@ -377,7 +375,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // sequences either way and serves the stage in its own loop, after the epilogue.)
         const uint32_t g = g0 + (uint32_t)T2;
         const int pr = g & 1;
-        ok = __all_sync(0xffffffffu, mbar_wait(bar(BAR_SMDONE0 + pr), (g >> 1) & 1, abortf));
+        ok = mbar_wait(bar(BAR_SMDONE0 + pr), (g >> 1) & 1, abortf);
         if (!ok) break;
         const int4 me = *reinterpret_cast<const int4*>(sgen + C::OFF_META + C::META_BYTES * pr + row * 16);
         mu_next = max(max(me.x, me.y), max(me.z, me.w)) + kRefHeadroom;
@@ -430,9 +428,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           c32 = __fdiv_rn(p.c_base, __fmul_rn(__ldg(p.q_G + wi.bh), __ldg(p.k_G + wi.kvh)));
       }
       for (uint32_t g = g0 + ((g0 & 1) != (uint32_t)pr); g < g0 + T2; g += 2) {   // this team's stages of the item
-        const uint32_t m = g >> 1;
-        ok = __all_sync(0xffffffffu, mbar_wait(sfull, m & 1, abortf));
-        if (!ok) break;
+        const uint32_t par = (g >> 1) & 1;
+        if (!mbar_wait(sfull, par, abortf)) { ok = false; break; }
         tc_fence_after();
         uint32_t sraw[32], w0[4], w1[4];
         int E0, E1;
@@ -457,8 +454,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           if (lane == 0) mbar_arrive(sempty);
           direct_p_block<PMAP, true, THR16>(sraw, c32, p.aff_a, p.aff_b, v0 - 32, E1, w1);
         }
-        if (m > 0) ok = __all_sync(0xffffffffu, mbar_wait(pfree, (m - 1) & 1, abortf));   // PV of the pair's previous stage is done
-        if (!ok) break;
+        if (!mbar_wait(pfree, par ^ 1, abortf)) { ok = false; break; }   // PV of the pair's previous stage is done (a fresh barrier passes)
         // fixed reference: E8M0 bytes of the two blocks against the constant; below the range a zero block (no codes,
         // so that a row without any live block shows as a zero row sum), above it an error
         const int b0 = FIXREF ? E0 - p.ref_fixed + 127 : 0, b1 = FIXREF ? E1 - p.ref_fixed + 127 : 0;
