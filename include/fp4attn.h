@@ -290,12 +290,11 @@ typedef struct {
  * causal = 1 and with grouped K/V heads.
  *
  * What FP4ATTN_PMAP_IDEAL guarantees.  x is one fused multiply-add in float32, x = fma(S, c, fl32(log2 6 - E_B)).
- * Of the 16 element pairs (keys 2k, 2k+1) of a block, pairs 0, 5, 10 and 15 evaluate 2^x by a degree-6
- * polynomial through the seven points where a code can change (after clamping x at -2.75, below which the
- * code is 0 either way), the other twelve by ex2.approx; the pattern is fixed in this build of the library.
- * Both are monotone there, so the codes equal Q_E2M1(2^x) except for x within about three float32 spacings of
- * a rounding boundary log2(t), t in {1/4, 3/4, 5/4, 7/4, 5/2, 7/2, 5}, where either neighbouring code may come
- * out.  FP4ATTN_PMAP_AFFINE has no such band: its arithmetic is exact float32 as written above.
+ * Of the 32 keys of a block, keys 0..7 and 24..31 evaluate 2^x by ex2.approx; for keys 8..23 the code is counted as the
+ * number of boundaries log2(t) below x, by three float32 affine functions of x whose E2M1 codes add up to it.  Both are
+ * monotone, so the codes equal Q_E2M1(2^x) except for x within about three float32 spacings of a rounding boundary
+ * log2(t), t in {1/4, 3/4, 5/4, 7/4, 5/2, 7/2, 5}, where either neighbouring code may come out.  FP4ATTN_PMAP_AFFINE
+ * has no such band: its arithmetic is exact float32 as written above.
  *
  * O_bf16 [B,H,N,d]; LSE [B,H,N] (may be NULL); device_status (may be NULL) receives
  * FP4ATTN_ERR_TIMEOUT if a bounded in-kernel wait ran out (or FP4ATTN_ERR_RANGE, see above), and is otherwise left
@@ -380,7 +379,8 @@ int fp4attn_mma_peak_probe(int iters, unsigned long long* cycles_out, fp4attn_st
  * Arithmetic ceiling of the softmax warps on the current device, measured: on every SM, sixteen warps (four per
  * scheduler, as in the attention kernel) each run the score -> code arithmetic of Algorithm "direct-p-pack" -
  * block maximum, block exponent (ceiling rule), the code map (`p_map` and `exact_pairs` as in
- * fp4attn_operands; other values: FP4ATTN_ERR_INVALID_ARG), E2M1 conversion and packing - on `iters`
+ * fp4attn_operands; other values: FP4ATTN_ERR_INVALID_ARG; of the ideal map's 16 pairs twelve on ex2.approx, so that the
+ * special-function unit is the bound, where the attention kernel has eight), E2M1 conversion and packing - on `iters`
  * (1 .. 2^20) blocks of 32 rows x 32 scores held in shared memory, with no tensor product, tensor-memory
  * access or hand-off around it.  Enqueues one kernel; cycles_out (device, TWO 64-bit words, the second is scratch)
  * receives in its first word the slowest warp's clock count, so that cycles / (4 * iters) is the clocks one

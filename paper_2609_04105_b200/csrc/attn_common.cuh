@@ -70,6 +70,7 @@ struct AttnParams {
   int N, stages;           // keys, N / 128
   int n_items;             // B * H * N / 128
   float c_base;            // fl32(log2(e) * softmax_scale)
+  unsigned long long c_mx2, ca_mx2;            // MXFP4 Q, K: {c, c} with c = fl32(c_base / 36), and {A c, A c}: packed multiply-add operands
   float aff_a, aff_b;      // affine classifier u = max(0, A x + B) (only read by the affine variant)
   int thr16;               // block exponent rule: 0 = ceil(max y), 1 = floor(max y + log2 1.6)
   int causal;              // 1: query row i sees keys 0..i
@@ -157,45 +158,46 @@ __device__ __forceinline__ float max32(const uint32_t* r) {
   const float a = max3(t[0], t[1], t[2]), b = max3(t[3], t[4], t[5]), c = max3(t[6], t[7], t[8]), d = max3(t[9], t[10], t[11]);
   return fmaxf(max3(a, b, c), d);
 }
-// two fused multiply-adds in one instruction: {x0, x1} = {s0, s1} * {c, c} + {b, b}
-__device__ __forceinline__ void fma2(float s0, float s1, float c, float b, float& x0, float& x1) {
-  asm("{\n\t.reg .b64 s, cc, bb, d;\n\t"
-      "mov.b64 s, {%2, %3};\n\tmov.b64 cc, {%4, %4};\n\tmov.b64 bb, {%5, %5};\n\t"
-      "fma.rn.f32x2 d, s, cc, bb;\n\t"
-      "mov.b64 {%0, %1}, d;\n\t}"
-      : "=f"(x0), "=f"(x1) : "f"(s0), "f"(s1), "f"(c), "f"(b));
-}
-// ---- 2^x on the FMA pipe for a share of the elements (the SFU's 16 ex2/clk/SM is the tightest unit).
-// Only the E2M1 code of 2^x matters, and it changes only where 2^x crosses 0.25, 0.75, 1.25, 1.75, 2.5,
-// 3.5 or 5.  2^x is therefore replaced by the degree-6 polynomial through the seven points (log2 b, b):
-// equal to 2^x at every point where a code can change and monotone on [-2.75, 3.3], so the codes are
-// those of the exact exponential (a 4-million-point sweep plus dense sweeps around the seven boundaries
-// differ only within three fp32 ulps of x at a boundary - the same class as ex2.approx).  No range
-// reduction: x is at most log2(9.6) by construction of the block exponent, and below -2.75 it is clamped
-// (there the polynomial stays inside (0.18, 0.25), i.e. code 0 like 2^x).
-#ifndef FP4ATTN_POLY_MASK
-#define FP4ATTN_POLY_MASK 0x8421u      // which of a block's 16 element pairs take the polynomial path
-#endif
-// The header states which pairs take which evaluation (fp4attn.h, FP4ATTN_PMAP_IDEAL); a build with another
-// pattern would change codes within rounding distance of a boundary, so it has to change that text as well.
-static_assert(FP4ATTN_POLY_MASK == 0x8421u, "the pattern of polynomial pairs is part of the documented behaviour");
 __device__ __forceinline__ uint64_t pack2(float a, float b) {
   uint64_t r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
   return r;
 }
-__device__ __forceinline__ void exp2_poly6(float x0, float x1, float& p0, float& p1) {
-  const uint64_t x = pack2(fmaxf(x0, -2.75f), fmaxf(x1, -2.75f));
-  uint64_t q;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(pack2(0.0002452842309139669f, 0.0002452842309139669f)), "l"(x),
-      "l"(pack2(0.0012840019771829247f, 0.0012840019771829247f)));
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(q), "l"(x), "l"(pack2(0.009303540922701359f, 0.009303540922701359f)));
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(q), "l"(x), "l"(pack2(0.05597471818327904f, 0.05597471818327904f)));
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(q), "l"(x), "l"(pack2(0.2401072233915329f, 0.2401072233915329f)));
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(q), "l"(x), "l"(pack2(0.6930626630783081f, 0.6930626630783081f)));
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(q) : "l"(q), "l"(x), "l"(pack2(1.0000272989273071f, 1.0000272989273071f)));
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(p0), "=f"(p1) : "l"(q));
+__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
 }
+// {x0, x1} = {s0, s1} * {c, c} + {b, b}
+__device__ __forceinline__ void fma2(float s0, float s1, float c, float b, float& x0, float& x1) {
+  unpack2(fma2(pack2(s0, s1), pack2(c, c), pack2(b, b)), x0, x1);
+}
+// ---- the code of 2^x without 2^x.
+// A code is the number of boundaries log2(b), b in {1/4, 3/4, 5/4, 7/4, 5/2, 7/2, 5}, below x.  The conversion to E2M1
+// counts the boundaries {1/4, 3/4, 5/4, 7/4, ...} below its own argument, so three conversions of affine functions of x
+// count all seven, each exactly once:
+//   u0 = x/2 + k0     crosses 1/4, 3/4, 5/4 at log2 5/4, log2 5/2, log2 5
+//   u1 = a1 x + k1    crosses 1/4, 3/4      at log2 1/4, log2 7/4
+//   u2 = a2 x + k2    crosses 1/4, 3/4      at log2 3/4, log2 7/2
+// The next crossing of each lies above 3.32, and x never exceeds log2 7.5 = 2.91 (log2 6 under the ceiling rule) by
+// construction of the block exponent, which leaves room for its rounding up to |y| = 2^21; negative arguments are clamped to code 0 by the conversion.  The three counts never sum to more than 7, so the packed
+// words of eight codes simply add.  The arguments are float32, so the codes are those of the exact exponential up to the
+// rounding of x at a boundary, as with ex2.approx (2-million-score sweeps at |y| up to 2000: no mismatch further than
+// 0.3 spacings of y from a boundary for either).
+//
+// What it is for: ex2.approx costs 8 clocks per warp instruction and scheduler, so 32 of them per block would alone take
+// 256.  Half the pairs on this route leave 128, and it takes less of everything else than a polynomial does: of its
+// four multiply-adds three read one register pair (x; slope and offset are literals).  Register operands are what the
+// dispatch is short of (about two 32-bit operands per clock and scheduler: a packed multiply-add with three register
+// pairs takes 4 clocks, with two 2, a three-input maximum 2).  Clocks per 32 x 32 block and scheduler, four warps, scores
+// from tensor memory: all pairs on ex2 272, 12 of 16 and a degree-6 polynomial for the rest 220, 12 / 10 / 8 / 6 / 0 of 16
+// and this route for the rest 211 / 192 / 178 / 186 / 233.
+constexpr float kCodeA1 = 0.1781035935540111f;                   // 1/2 / (log2 7/4 - log2 1/4)
+constexpr float kCodeA2 = 0.22498276865942612f;                  // 1/2 / (log2 7/2 - log2 3/4)
+constexpr float kCodeK0 = 0.0890359525563188f;                   // 1/4 - 1/2 log2 5/4
+constexpr float kCodeK1 = 0.6062071871080222f;                   // 1/4 + 2 a1
+constexpr float kCodeK2 = 0.34337628568523887f;                  // 1/4 - a2 log2 3/4
 
 // One N32 score fragment of one row: E_B = ceil(max y) and the codes.  Nothing here depends on the
 // row reference.
@@ -208,22 +210,27 @@ __device__ __forceinline__ void exp2_poly6(float x0, float x1, float& p0, float&
 __host__ __device__ constexpr uint32_t exact_pairs_of(int pmap) {
   return pmap == 0 ? 0xFFFFu : pmap == 1 ? 0x0000u : pmap == 2 ? 0x1111u : pmap == 3 ? 0x5555u : 0x7777u;
 }
+// Words (of eight keys) whose exact pairs take the conversion count instead of ex2.approx: so many that the special-function
+// unit stops being the bound (8 of 16 pairs are left to it, 9 with 12 of 16 exact; with 8 or fewer exact it never is).  The
+// two middle words rather than the first two: 889 against 903 us at N = 8192 (903: words 0 and 1, 934: one word).
+__host__ __device__ constexpr uint32_t counted_words_of(int pmap) { return pmap == 0 ? 0x6u : pmap == 4 ? 0x1u : 0x0u; }
 // RULE: block exponent from the block maximum - 0 ceiling, 1 threshold rule, 2 the better of ceiling and ceiling - 1 by
 // squared error of the 32 represented values (ideal map only; see direct_p_block_mse)
-template <bool MASKED>
-__device__ __forceinline__ void direct_p_block_mse(uint32_t* sraw, float c32, int visible, int& E, uint32_t* words);
+__device__ __forceinline__ void direct_p_block_mse(const uint32_t* sraw, float c32, int& E, uint32_t* words);
+// keys from `visible` on (causal mask, padding) get -inf: they never raise a block maximum and always code to 0
+__device__ __forceinline__ void mask_scores(uint32_t* sraw, int visible) {
+#pragma unroll
+  for (int i = 0; i < 32; ++i) sraw[i] = (i < visible) ? sraw[i] : 0xFF800000u;
+}
 
-template <int PMAP, bool MASKED, int RULE>
-__device__ __forceinline__ void direct_p_block(uint32_t* sraw, float c32, float A, float B, int visible, int& E,
-                                               uint32_t* words) {
-  if (RULE == 2) { direct_p_block_mse<MASKED>(sraw, c32, visible, E, words); return; }
+// c2 = {c, c}, ca2 = {fl32(A c), fl32(A c)}: 64-bit so that they can stay in uniform registers (kernel parameters)
+template <int PMAP, int RULE, uint32_t COUNTED = counted_words_of(PMAP)>
+__device__ __forceinline__ void direct_p_block(const uint32_t* sraw, uint64_t c2, uint64_t ca2, float A, float B, int& E, uint32_t* words) {
+  const float c32 = __uint_as_float((uint32_t)c2);
+  if (RULE == 2) { direct_p_block_mse(sraw, c32, E, words); return; }
   constexpr bool THR16 = RULE == 1;
   constexpr uint32_t kExact = exact_pairs_of(PMAP);
   const float LOG2_6 = 2.5849625007211560f;
-  if (MASKED) {                                                 // keys the row does not see (causal mask, padding) get -inf
-#pragma unroll
-    for (int i = 0; i < 32; ++i) sraw[i] = (i < visible) ? sraw[i] : 0xFF800000u;
-  }
   // y is clamped to +-2^21 (scores beyond that are outside any softmax's range; a fully masked block,
   // max = -inf, lands on the lower clamp and becomes a zero block)
   const float ymax = fminf(fmaxf(__fmul_rn(max32(sraw), c32), -2097152.0f), 2097152.0f);
@@ -235,44 +242,45 @@ __device__ __forceinline__ void direct_p_block(uint32_t* sraw, float c32, float 
   const float t = THR16 ? __fadd_rd(__fadd_rn(ymax, 0.6780719161033630f), M) : __fadd_ru(ymax, M);
   E = (int)(__float_as_uint(t) - 0x4B400000u);
   const float bB = __fsub_rn(LOG2_6, __fsub_rn(t, M));          // t - M = (float)E, exact
-  const float cA = __fmul_rn(A, c32), bA = __fmaf_rn(A, bB, B);  // affine pairs only
+  const float bA = __fmaf_rn(A, bB, B);                          // affine pairs only
+  static_assert(COUNTED == 0u || kExact == 0xFFFFu || kExact == 0x7777u, "a counted word has its first three pairs exact, or all four");
 #pragma unroll
   for (int w = 0; w < 4; ++w) {
-    float pv[8];
+    const bool counted = (COUNTED >> w) & 1u;
+    float pv[8], q1[8], q2[8];
 #pragma unroll
     for (int i = 0; i < 8; i += 2) {
-      const int pair = 4 * w + i / 2;
-      if ((kExact >> pair) & 1u) {
-        float x0, x1;
-        fma2(__uint_as_float(sraw[8 * w + i]), __uint_as_float(sraw[8 * w + i + 1]), c32, bB, x0, x1);
-        if ((FP4ATTN_POLY_MASK >> pair) & 1u) {
-          exp2_poly6(x0, x1, pv[i], pv[i + 1]);
+      const float s0 = __uint_as_float(sraw[8 * w + i]), s1 = __uint_as_float(sraw[8 * w + i + 1]);
+      if ((kExact >> (4 * w + i / 2)) & 1u) {
+        const uint64_t x = fma2(pack2(s0, s1), c2, pack2(bB, bB));
+        if (counted) {
+          unpack2(fma2(x, pack2(0.5f, 0.5f), pack2(kCodeK0, kCodeK0)), pv[i], pv[i + 1]);
+          unpack2(fma2(x, pack2(kCodeA1, kCodeA1), pack2(kCodeK1, kCodeK1)), q1[i], q1[i + 1]);
+          unpack2(fma2(x, pack2(kCodeA2, kCodeA2), pack2(kCodeK2, kCodeK2)), q2[i], q2[i + 1]);
         } else {
+          float x0, x1;
+          unpack2(x, x0, x1);
           pv[i] = ex2_approx(x0);
           pv[i + 1] = ex2_approx(x1);
         }
       } else {
-        fma2(__uint_as_float(sraw[8 * w + i]), __uint_as_float(sraw[8 * w + i + 1]), cA, bA, pv[i], pv[i + 1]);
+        unpack2(fma2(pack2(s0, s1), ca2, pack2(bA, bA)), pv[i], pv[i + 1]);
       }
     }
-    // the conversion clamps negative inputs to +0 (affine pairs; exact pairs are positive anyway)
-    words[w] = kExact == 0xFFFFu ? cvt_e2m1x8(pv) : cvt_e2m1x8_relu(pv);
+    // the conversion clamps negative inputs to +0 (affine and counted pairs; an exponential is positive anyway)
+    words[w] = (kExact == 0xFFFFu && !counted) ? cvt_e2m1x8(pv) : cvt_e2m1x8_relu(pv);
+    if (counted) words[w] += kExact == 0xFFFFu ? cvt_e2m1x8_relu(q1) + cvt_e2m1x8_relu(q2) : cvt_e2m1x6_relu(q1) + cvt_e2m1x6_relu(q2);
   }
 }
 
 // Eq. "mx-scale" names both powers of two next to a block maximum.  Here every block takes, of E_c = ceil(max y) and
 // E_c - 1, the one with the smaller squared error of its 32 represented probabilities.  Under E_c the code units are
-// v = 6 * 2^(y - E_c) (every v through ex2.approx: the boundary polynomial is exact only where codes change); under
+// v = 6 * 2^(y - E_c) (every v through ex2.approx: the conversion count gives codes, not values); under
 // E_c - 1 they are 2v, saturating at 6, in units half as large: the floor wins iff
 //   sum (2v - q(2v))^2 < 4 sum (v - q(v))^2      (strictly; a block whose maximum is an integer has one candidate).
 // Error sums in fp32: eight consecutive keys left to right, the four group sums as (g0 + g1) + (g2 + g3).
-template <bool MASKED>
-__device__ __forceinline__ void direct_p_block_mse(uint32_t* sraw, float c32, int visible, int& E, uint32_t* words) {
+__device__ __forceinline__ void direct_p_block_mse(const uint32_t* sraw, float c32, int& E, uint32_t* words) {
   const float LOG2_6 = 2.5849625007211560f;
-  if (MASKED) {
-#pragma unroll
-    for (int i = 0; i < 32; ++i) sraw[i] = (i < visible) ? sraw[i] : 0xFF800000u;
-  }
   const float ymax = fminf(fmaxf(__fmul_rn(max32(sraw), c32), -2097152.0f), 2097152.0f);
   const float M = 12582912.0f;
   const float t = __fadd_ru(ymax, M);

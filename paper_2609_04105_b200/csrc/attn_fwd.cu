@@ -408,9 +408,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     const uint32_t smdone = bar(BAR_SMDONE0 + pr), pfree = bar(BAR_PFREE0 + pr);
     const uint32_t tP = tmem + ((uint32_t)(quarter * 32) << 16) + kColP + 8 * team;
     int2* meta = reinterpret_cast<int2*>(sgen + C::OFF_META + C::META_BYTES * pr + row * 16 + 8 * (team & 1));
-    float c32;
-    if (NV) c32 = __fdiv_rn(p.c_base, __fmul_rn(__ldg(p.q_G), __ldg(p.k_G)));
-    else    c32 = __fdiv_rn(p.c_base, 36.0f);
+    uint64_t c2 = p.c_mx2, ca2 = p.ca_mx2;
+    if (NV) {
+      const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldg(p.q_G), __ldg(p.k_G)));
+      c2 = pack2(c, c);
+      ca2 = pack2(__fmul_rn(p.aff_a, c), __fmul_rn(p.aff_a, c));
+    }
     uint32_t g0 = 0;
     bool ok = true;
     int T2 = 0;
@@ -424,48 +427,39 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // causal: keys 0..i of row i = qt * 128 + row; padded sequence: keys 0..len-1; both: the fewer
         const int seen = (CAUSAL && p.causal) ? min(wi.len, wi.qt * BM + row + 1) : wi.len;
         vis = seen - (T2 - 1) * BS;
-        if (NV == 2)                                            // this unit's own pair of encode factors
-          c32 = __fdiv_rn(p.c_base, __fmul_rn(__ldg(p.q_G + wi.bh), __ldg(p.k_G + wi.kvh)));
+        if (NV == 2) {                                          // this unit's own pair of encode factors
+          const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldg(p.q_G + wi.bh), __ldg(p.k_G + wi.kvh)));
+          c2 = pack2(c, c);
+          ca2 = pack2(__fmul_rn(p.aff_a, c), __fmul_rn(p.aff_a, c));
+        }
       }
       for (uint32_t g = g0 + ((g0 & 1) != (uint32_t)pr); g < g0 + T2; g += 2) {   // this team's stages of the item
         const uint32_t par = (g >> 1) & 1;
         if (!mbar_wait(sfull, par, abortf)) { ok = false; break; }
         tc_fence_after();
-        uint32_t sraw[32], w0[4], w1[4];
+        uint32_t sraw[32], pw[8];
         int E0, E1;
         tmem_ld_32x32b_x32(tS, sraw);
         tmem_wait_ld();
-        if (!CAUSAL || g != gdiag) {
-          direct_p_block<PMAP, false, THR16>(sraw, c32, p.aff_a, p.aff_b, 32, E0, w0);
-          tmem_ld_32x32b_x32(tS + 32, sraw);
-          tmem_wait_ld();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(sempty);                   // pair may take the stage after next
-          direct_p_block<PMAP, false, THR16>(sraw, c32, p.aff_a, p.aff_b, 32, E1, w1);
-        } else {
-          // masked stage: this row sees the first `vis` keys of the stage; the team's tile starts at key 64*(team&1)
-          const int v0 = vis - 64 * (team & 1);
-          direct_p_block<PMAP, true, THR16>(sraw, c32, p.aff_a, p.aff_b, v0, E0, w0);
-          tmem_ld_32x32b_x32(tS + 32, sraw);
-          tmem_wait_ld();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(sempty);
-          direct_p_block<PMAP, true, THR16>(sraw, c32, p.aff_a, p.aff_b, v0 - 32, E1, w1);
-        }
+        // masked stage: this row sees the first `vis` keys of the stage; the team's tile starts at key 64*(team&1)
+        if (CAUSAL && g == gdiag) mask_scores(sraw, vis - 64 * (team & 1));
+        direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E0, pw);
+        tmem_ld_32x32b_x32(tS + 32, sraw);
+        tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sempty);                     // pair may take the stage after next
+        if (CAUSAL && g == gdiag) mask_scores(sraw, vis - 64 * (team & 1) - 32);
+        direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E1, pw + 4);
         if (!mbar_wait(pfree, par ^ 1, abortf)) { ok = false; break; }   // PV of the pair's previous stage is done (a fresh barrier passes)
         // fixed reference: E8M0 bytes of the two blocks against the constant; below the range a zero block (no codes,
         // so that a row without any live block shows as a zero row sum), above it an error
         const int b0 = FIXREF ? E0 - p.ref_fixed + 127 : 0, b1 = FIXREF ? E1 - p.ref_fixed + 127 : 0;
         if (FIXREF && __any_sync(0xffffffffu, min(b0, b1) < 1)) {    // rare: some row of the warp has a block below the range
-          if (b0 < 1) w0[0] = w0[1] = w0[2] = w0[3] = 0u;
-          if (b1 < 1) w1[0] = w1[1] = w1[2] = w1[3] = 0u;
+          if (b0 < 1) pw[0] = pw[1] = pw[2] = pw[3] = 0u;
+          if (b1 < 1) pw[4] = pw[5] = pw[6] = pw[7] = 0u;
         }
-        {
-          const uint32_t pw[8] = {w0[0], w0[1], w0[2], w0[3], w1[0], w1[1], w1[2], w1[3]};
-          tmem_st_32x32b_x8(tP, pw);
-        }
+        tmem_st_32x32b_x8(tP, pw);
         if (FIXREF) {
           if (max(b0, b1) > 254 && p.status) *p.status = FP4ATTN_ERR_RANGE;      // (the byte written below is then meaningless)
           const uint32_t u0 = (uint32_t)max(b0, 0) & 0xFFu, u1 = (uint32_t)max(b1, 0) & 0xFFu;
@@ -710,6 +704,10 @@ extern "C" int fp4attn_fwd(const fp4attn_operands* ops, int B, int H, int N, int
   const bool nv = ops->qk_fmt == FP4ATTN_FMT_NVFP4;
   prm.aff_a = ops->affine_a != 0.f ? ops->affine_a : 1.5f;         // the paper's generic `fast` fit
   prm.aff_b = ops->affine_a != 0.f ? ops->affine_b : 1.2f;
+  auto twice = [](float f) { uint32_t u; memcpy(&u, &f, 4); return (unsigned long long)u << 32 | u; };
+  const float c_mx = prm.c_base / 36.0f;                           // IEEE division and products, as on the device
+  prm.c_mx2 = twice(c_mx);
+  prm.ca_mx2 = twice(prm.aff_a * c_mx);
   prm.thr16 = ops->p_scale_rule == FP4ATTN_PSCALE_THR16;
   if (ops->schedule != FP4ATTN_SCHEDULE_ONE_QUERY && ops->schedule != FP4ATTN_SCHEDULE_TWO_QUERY) return FP4ATTN_ERR_INVALID_ARG;
   if (ops->pv_fmt != FP4ATTN_PV_MXFP4 && ops->pv_fmt != FP4ATTN_PV_E4M3) return FP4ATTN_ERR_INVALID_ARG;

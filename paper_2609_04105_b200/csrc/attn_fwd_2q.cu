@@ -365,9 +365,12 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const uint32_t smdone = bar(B2_SMDONE0 + q), pfree = bar(B2_PFREE0 + q);
     const uint32_t tP = tmem + ((uint32_t)(quarter * 32) << 16) + k2ColP + 8 * team;
     int2* meta = reinterpret_cast<int2*>(sgen + C2::OFF_META + C::META_BYTES * q + row * 16 + 8 * (team & 1));
-    float c32;
-    if (NV) c32 = __fdiv_rn(p.c_base, __fmul_rn(__ldg(p.q_G), __ldg(p.k_G)));
-    else    c32 = __fdiv_rn(p.c_base, 36.0f);
+    uint64_t c2 = p.c_mx2, ca2 = p.ca_mx2;
+    if (NV) {
+      const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldg(p.q_G), __ldg(p.k_G)));
+      c2 = pack2(c, c);
+      ca2 = pack2(__fmul_rn(p.aff_a, c), __fmul_rn(p.aff_a, c));
+    }
     bool ok = true;
     uint32_t ms = 0;
     for (int item = blockIdx.x; ok && item < p.n_items; item += gridDim.x) {
@@ -379,13 +382,13 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         int E0, E1;
         tmem_ld_32x32b_x32(tS, sraw);
         tmem_wait_ld();
-        direct_p_block<PMAP, false, THR16>(sraw, c32, p.aff_a, p.aff_b, 32, E0, w0);
+        direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E0, w0);
         tmem_ld_32x32b_x32(tS + 32, sraw);
         tmem_wait_ld();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(sempty);                     // S_q may take the next stage
-        direct_p_block<PMAP, false, THR16>(sraw, c32, p.aff_a, p.aff_b, 32, E1, w1);
+        direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E1, w1);
         if (ms > 0) ok = mbar_wait(pfree, (ms - 1) & 1, abortf);   // PV of the query's previous stage is done
         if (!ok) break;
         {

@@ -5,6 +5,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <string.h>
+
 #include <atomic>
 #include <mutex>
 
@@ -37,6 +39,19 @@ __device__ __forceinline__ uint32_t cvt_e2m1x8_relu(const float* v) {
       "mov.b32 %0, {t0, t1, t2, t3};\n\t}"
       : "=r"(w)
       : "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]));
+  return w;
+}
+
+// the first six of eight elements; the last two get code 0
+__device__ __forceinline__ uint32_t cvt_e2m1x6_relu(const float* v) {
+  uint32_t w;
+  asm("{\n\t.reg .b8 t0, t1, t2, t3;\n\tmov.b32 {t3, _, _, _}, 0;\n\t"
+      "cvt.rn.satfinite.relu.e2m1x2.f32 t0, %2, %1;\n\t"
+      "cvt.rn.satfinite.relu.e2m1x2.f32 t1, %4, %3;\n\t"
+      "cvt.rn.satfinite.relu.e2m1x2.f32 t2, %6, %5;\n\t"
+      "mov.b32 %0, {t0, t1, t2, t3};\n\t}"
+      : "=r"(w)
+      : "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]));
   return w;
 }
 
