@@ -1,11 +1,14 @@
-"""Thin ctypes binding over libfp4attn.so: argument marshalling only.
+"""Thin binding over libfp4attn.so: argument marshalling only.
 
-PyTorch appears here for device memory and streams; every step of the path runs inside the
-library's CUDA kernels.  Importing this module fails loudly when the library is missing.
+The calls of a step (the quantizers and the forward) are marshalled by the native module _fp4attn_native.so, the others by
+ctypes.  PyTorch appears here for device memory and streams; every step of the path runs inside the library's CUDA kernels.
+The first call fails loudly when the library or the module is missing.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import Optional, Tuple
@@ -24,6 +27,7 @@ QSCALE_CEIL, QSCALE_THR16, QSCALE_FLOOR, QSCALE_MSE = 0, 1, 2, 3
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libfp4attn.so")
+NATIVE_PATH = os.path.join(_HERE, "_fp4attn_native.so")
 
 EXPORTS = [
     "fp4attn_status_string", "fp4attn_version", "fp4attn_packed_bytes", "fp4attn_scale_bytes",
@@ -97,7 +101,26 @@ def _load() -> ctypes.CDLL:
     return lib
 
 
+# the functions the native module calls, in the order it takes their addresses
+_NATIVE_CALLS = ["fp4attn_status_string", "fp4attn_packed_bytes", "fp4attn_scale_bytes", "fp4attn_quantize_workspace_bytes",
+                 "fp4attn_quantize", "fp4attn_quantize_mxfp4_rule", "fp4attn_quantize_nvfp4_per_head_workspace_bytes",
+                 "fp4attn_quantize_nvfp4_per_head", "fp4attn_quantize_v_e4m3_workspace_bytes", "fp4attn_quantize_v_e4m3",
+                 "fp4attn_fwd"]
+
+
+def _load_native(lib_: ctypes.CDLL):
+    if not os.path.exists(NATIVE_PATH):
+        raise Fp4AttnError(f"{NATIVE_PATH} is missing: build it with `python -m paper_2609_04105_b200.build` "
+                           "(there is no fallback path)")
+    loader = importlib.machinery.ExtensionFileLoader("_fp4attn_native", NATIVE_PATH)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_fp4attn_native", loader))
+    loader.exec_module(module)
+    module.init(Fp4AttnError, *[ctypes.cast(getattr(lib_, n), ctypes.c_void_p).value for n in _NATIVE_CALLS])
+    return module
+
+
 _lib: Optional[ctypes.CDLL] = None
+_native_module = None
 
 
 def lib() -> ctypes.CDLL:
@@ -105,6 +128,13 @@ def lib() -> ctypes.CDLL:
     if _lib is None:
         _lib = _load()
     return _lib
+
+
+def _native():
+    global _native_module
+    if _native_module is None:
+        _native_module = _load_native(lib())
+    return _native_module
 
 
 def _check(rc: int, what: str) -> None:
@@ -133,64 +163,20 @@ class QuantizedOperand:
 
 def fp4attn_quantize(x: torch.Tensor, fmt: int, role: int, workspace: Optional[torch.Tensor] = None) -> QuantizedOperand:
     """x: CUDA bf16 [B,H,N,d] contiguous -> packed E2M1 + scale factors (see include/fp4attn.h)."""
-    assert x.is_cuda and x.dtype == torch.bfloat16 and x.is_contiguous() and x.dim() == 4
-    B, H, N, d = x.shape
-    L = lib()
-    nb = L.fp4attn_packed_bytes(B, H, N, d)
-    ns = L.fp4attn_scale_bytes(fmt, role, B, H, N, d)
-    if nb == 0 or ns == 0:
-        _check(L.fp4attn_quantize(x.data_ptr(), fmt, role, B, H, N, d, 1, 1, None, None, 0, _stream()), "fp4attn_quantize")
-        raise Fp4AttnError("fp4attn_quantize: unsupported arguments")
-    packed = torch.empty(nb, dtype=torch.uint8, device=x.device)
-    scales = torch.empty(ns, dtype=torch.uint8, device=x.device)
-    G = torch.empty(1, dtype=torch.float32, device=x.device) if fmt == FMT_NVFP4 else None
-    nw = L.fp4attn_quantize_workspace_bytes(fmt, role, B, H, N, d)
-    if nw and workspace is None:
-        workspace = torch.empty(nw, dtype=torch.uint8, device=x.device)
-    _check(L.fp4attn_quantize(x.data_ptr(), fmt, role, B, H, N, d, packed.data_ptr(), scales.data_ptr(),
-                              _ptr(G), _ptr(workspace), 0 if workspace is None else workspace.numel(), _stream()),
-           "fp4attn_quantize")
-    return QuantizedOperand(packed, scales, G, fmt, role, (B, H, N, d))
+    packed, scales, G, shape = (_native_module or _native()).quantize(x, fmt, role, workspace)
+    return QuantizedOperand(packed, scales, G, fmt, role, shape)
 
 
 def fp4attn_quantize_mxfp4_rule(x: torch.Tensor, role: int, scale_rule: int) -> QuantizedOperand:
     """MXFP4 quantizer with a selectable amplitude rule (QSCALE_CEIL / QSCALE_THR16 / QSCALE_FLOOR)."""
-    assert x.is_cuda and x.dtype == torch.bfloat16 and x.is_contiguous() and x.dim() == 4
-    B, H, N, d = x.shape
-    L = lib()
-    nb = L.fp4attn_packed_bytes(B, H, N, d)
-    ns = L.fp4attn_scale_bytes(FMT_MXFP4, role, B, H, N, d)
-    if nb == 0 or ns == 0:
-        _check(L.fp4attn_quantize_mxfp4_rule(x.data_ptr(), role, scale_rule, B, H, N, d, 1, 1, _stream()),
-               "fp4attn_quantize_mxfp4_rule")
-        raise Fp4AttnError("fp4attn_quantize_mxfp4_rule: unsupported arguments")
-    packed = torch.empty(nb, dtype=torch.uint8, device=x.device)
-    scales = torch.empty(ns, dtype=torch.uint8, device=x.device)
-    _check(L.fp4attn_quantize_mxfp4_rule(x.data_ptr(), role, scale_rule, B, H, N, d, packed.data_ptr(),
-                                         scales.data_ptr(), _stream()), "fp4attn_quantize_mxfp4_rule")
-    return QuantizedOperand(packed, scales, None, FMT_MXFP4, role, (B, H, N, d))
+    packed, scales, _, shape = (_native_module or _native()).quantize_mxfp4_rule(x, role, scale_rule)
+    return QuantizedOperand(packed, scales, None, FMT_MXFP4, role, shape)
 
 
 def fp4attn_quantize_nvfp4_per_head(x: torch.Tensor, role: int) -> QuantizedOperand:
     """NVFP4 quantizer with one encode factor per (batch, head) unit; G comes back as fp32 [B*H]."""
-    assert x.is_cuda and x.dtype == torch.bfloat16 and x.is_contiguous() and x.dim() == 4
-    B, H, N, d = x.shape
-    L = lib()
-    nb = L.fp4attn_packed_bytes(B, H, N, d)
-    ns = L.fp4attn_scale_bytes(FMT_NVFP4, role, B, H, N, d)
-    nw = L.fp4attn_quantize_nvfp4_per_head_workspace_bytes(B, H, N, d)
-    if nb == 0 or ns == 0 or nw == 0:
-        _check(L.fp4attn_quantize_nvfp4_per_head(x.data_ptr(), role, B, H, N, d, 1, 1, 1, None, 0, _stream()),
-               "fp4attn_quantize_nvfp4_per_head")
-        raise Fp4AttnError("fp4attn_quantize_nvfp4_per_head: unsupported arguments")
-    packed = torch.empty(nb, dtype=torch.uint8, device=x.device)
-    scales = torch.empty(ns, dtype=torch.uint8, device=x.device)
-    G = torch.empty(B * H, dtype=torch.float32, device=x.device)
-    ws = torch.empty(nw, dtype=torch.uint8, device=x.device)
-    _check(L.fp4attn_quantize_nvfp4_per_head(x.data_ptr(), role, B, H, N, d, packed.data_ptr(), scales.data_ptr(),
-                                             G.data_ptr(), ws.data_ptr(), ws.numel(), _stream()),
-           "fp4attn_quantize_nvfp4_per_head")
-    return QuantizedOperand(packed, scales, G, FMT_NVFP4, role, (B, H, N, d), True)
+    packed, scales, G, shape = (_native_module or _native()).quantize_nvfp4_per_head(x, role)
+    return QuantizedOperand(packed, scales, G, FMT_NVFP4, role, shape, True)
 
 
 def fp4attn_quantize_nvfp4_noalloc(x: torch.Tensor, role: int, packed: torch.Tensor, scales: torch.Tensor,
@@ -209,19 +195,8 @@ FMT_E4M3 = 2          # QuantizedOperand.fmt of an E4M3 V (fp4attn_quantize_v_e4
 
 def fp4attn_quantize_v_e4m3(x: torch.Tensor) -> QuantizedOperand:
     """E4M3 bytes of V^T [B,H,d,N] with one encode factor per (batch, head) unit (G fp32 [B*H]); `scales` is empty."""
-    assert x.is_cuda and x.dtype == torch.bfloat16 and x.is_contiguous() and x.dim() == 4
-    B, H, N, d = x.shape
-    L = lib()
-    nw = L.fp4attn_quantize_v_e4m3_workspace_bytes(B, H, N, d)
-    if nw == 0:
-        _check(L.fp4attn_quantize_v_e4m3(x.data_ptr(), B, H, N, d, 1, 1, None, 0, _stream()), "fp4attn_quantize_v_e4m3")
-        raise Fp4AttnError("fp4attn_quantize_v_e4m3: unsupported arguments")
-    out = torch.empty(B * H * d * N, dtype=torch.uint8, device=x.device)
-    G = torch.empty(B * H, dtype=torch.float32, device=x.device)
-    ws = torch.empty(nw, dtype=torch.uint8, device=x.device)
-    _check(L.fp4attn_quantize_v_e4m3(x.data_ptr(), B, H, N, d, out.data_ptr(), G.data_ptr(), ws.data_ptr(), ws.numel(), _stream()),
-           "fp4attn_quantize_v_e4m3")
-    return QuantizedOperand(out, torch.empty(0, dtype=torch.uint8, device=x.device), G, FMT_E4M3, ROLE_V, (B, H, N, d), True)
+    out, scales, G, shape = (_native_module or _native()).quantize_v_e4m3(x)
+    return QuantizedOperand(out, scales, G, FMT_E4M3, ROLE_V, shape, True)
 
 
 def fp4attn_fwd(q: QuantizedOperand, k: QuantizedOperand, v: QuantizedOperand, softmax_scale: float = 0.0,
@@ -234,25 +209,8 @@ def fp4attn_fwd(q: QuantizedOperand, k: QuantizedOperand, v: QuantizedOperand, s
     p_map selects the exact code map or the affine classifier (affine_a = 0: A = 1.5, B = 1.2).
     seq_len: optional CUDA int32 tensor [B], the token count of every batch entry (padded to N).
     fixed_reference: None - running row reference; an integer - that constant row reference (the shiftless path)."""
-    B, H, N, d = q.shape
-    Hkv = k.shape[1]                                   # grouped-query attention when Hkv < H
-    assert k.shape == v.shape and k.shape == (B, Hkv, N, d) and H % Hkv == 0 and q.fmt == k.fmt and v.fmt in (FMT_MXFP4, FMT_E4M3)
-    fp8 = v.fmt == FMT_E4M3
-    assert q.per_head == k.per_head, "Q and K must both carry per-head factors, or neither"
-    assert seq_len is None or (seq_len.is_cuda and seq_len.dtype == torch.int32 and seq_len.numel() == B and seq_len.is_contiguous())
-    dev = q.packed.device
-    if out is None:
-        out = torch.empty((B, H, N, d), dtype=torch.bfloat16, device=dev)
-    if lse is None:
-        lse = torch.empty((B, H, N), dtype=torch.float32, device=dev)
-    ops = _Operands(q.packed.data_ptr(), k.packed.data_ptr(), v.packed.data_ptr(),
-                    q.scales.data_ptr(), k.scales.data_ptr(), None if fp8 else v.scales.data_ptr(),
-                    _ptr(q.G), _ptr(k.G), q.fmt, float(softmax_scale), int(p_map), float(affine_a), float(affine_b), int(p_scale_rule), int(bool(causal)), int(Hkv),
-                    int(exact_pairs), int(q.per_head), int(schedule), PV_E4M3 if fp8 else PV_MXFP4, _ptr(v.G) if fp8 else None,
-                    0 if fixed_reference is None else 1, 0 if fixed_reference is None else int(fixed_reference), _ptr(seq_len))
-    _check(lib().fp4attn_fwd(ctypes.byref(ops), B, H, N, d, out.data_ptr(), lse.data_ptr(), _ptr(status), _stream()),
-           "fp4attn_fwd")
-    return out, lse
+    return (_native_module or _native()).fwd(q, k, v, softmax_scale, out, lse, status, p_map, affine_a, affine_b, p_scale_rule, causal,
+                                             exact_pairs, schedule, seq_len, fixed_reference)
 
 
 def fp4attn_attention_host_workspace_bytes(qk_fmt: int, B: int, H: int, N: int, d: int) -> int:
