@@ -124,7 +124,7 @@ __device__ __forceinline__ WorkItem decode_item(int item, const AttnParams& p, i
   w.T2 = p.stages;
   if (MASKED) {
     if (p.seq_len) {
-      const int len = __ldg(p.seq_len + fast_div(bh, p.recip_h));
+      const int len = __ldcg(p.seq_len + fast_div(bh, p.recip_h));
       w.len = len < 1 ? 1 : (len > p.N ? p.N : len);
       w.T2 = w.qt * BM < w.len ? (w.len + BS - 1) / BS : 1;   // a query tile beyond the length: one stage, results unused
     }

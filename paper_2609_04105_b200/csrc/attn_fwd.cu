@@ -94,6 +94,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  wait_prior_grids();                                           // everything above is this block's own set-up
   const uint32_t tmem = *tslot;
 
   if (warp == 0) {
@@ -410,7 +411,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     int2* meta = reinterpret_cast<int2*>(sgen + C::OFF_META + C::META_BYTES * pr + row * 16 + 8 * (team & 1));
     uint64_t c2 = p.c_mx2, ca2 = p.ca_mx2;
     if (NV) {
-      const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldg(p.q_G), __ldg(p.k_G)));
+      const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldcg(p.q_G), __ldcg(p.k_G)));
       c2 = pack2(c, c);
       ca2 = pack2(__fmul_rn(p.aff_a, c), __fmul_rn(p.aff_a, c));
     }
@@ -428,7 +429,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const int seen = (CAUSAL && p.causal) ? min(wi.len, wi.qt * BM + row + 1) : wi.len;
         vis = seen - (T2 - 1) * BS;
         if (NV == 2) {                                          // this unit's own pair of encode factors
-          const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldg(p.q_G + wi.bh), __ldg(p.k_G + wi.kvh)));
+          const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldcg(p.q_G + wi.bh), __ldcg(p.k_G + wi.kvh)));
           c2 = pack2(c, c);
           ca2 = pack2(__fmul_rn(p.aff_a, c), __fmul_rn(p.aff_a, c));
         }
@@ -640,7 +641,7 @@ static int launch_attn(const fp4attn_operands* ops, int B, int H, int N, AttnPar
   const CUtensorMap* tm = tensor_maps<D>(ops, prm.O, B, H, Hkv, N);
   if (!tm) return FP4ATTN_ERR_CUDA;
   const unsigned grid = (unsigned)(prm.n_items < sms ? prm.n_items : sms);     // persistent: one CTA per SM
-  attn_fwd_kernel<D, NV, PMAP, CAUSAL, THR16, FIXREF><<<grid, kAttnThreads, C::SMEM_BYTES, st>>>(tm[0], tm[1], tm[2], tm[3], prm);
+  launch_overlapped(attn_fwd_kernel<D, NV, PMAP, CAUSAL, THR16, FIXREF>, dim3(grid), kAttnThreads, C::SMEM_BYTES, st, tm[0], tm[1], tm[2], tm[3], prm);
   return cudaGetLastError() == cudaSuccess ? FP4ATTN_OK : FP4ATTN_ERR_CUDA;
 }
 

@@ -118,6 +118,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  wait_prior_grids();                                           // everything above is this block's own set-up
   const uint32_t tmem = *tslot;
 
   if (warp == 0) {
@@ -367,7 +368,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     int2* meta = reinterpret_cast<int2*>(sgen + C2::OFF_META + C::META_BYTES * q + row * 16 + 8 * (team & 1));
     uint64_t c2 = p.c_mx2, ca2 = p.ca_mx2;
     if (NV) {
-      const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldg(p.q_G), __ldg(p.k_G)));
+      const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldcg(p.q_G), __ldcg(p.k_G)));
       c2 = pack2(c, c);
       ca2 = pack2(__fmul_rn(p.aff_a, c), __fmul_rn(p.aff_a, c));
     }
@@ -433,7 +434,7 @@ static int launch_2q(const fp4attn_operands* ops, int B, int H, int N, AttnParam
   const CUtensorMap* tm = attention_tensor_maps(64, ops, prm.O, B, H, prm.Hkv, N);
   if (!tm) return FP4ATTN_ERR_CUDA;
   const unsigned grid = (unsigned)(prm.n_items < sms ? prm.n_items : sms);
-  attn_fwd_2q_kernel<NV, PMAP, THR16><<<grid, kAttnThreads, C2::SMEM_BYTES, st>>>(tm[0], tm[1], tm[2], tm[3], prm);
+  launch_overlapped(attn_fwd_2q_kernel<NV, PMAP, THR16>, dim3(grid), kAttnThreads, C2::SMEM_BYTES, st, tm[0], tm[1], tm[2], tm[3], prm);
   return cudaGetLastError() == cudaSuccess ? FP4ATTN_OK : FP4ATTN_ERR_CUDA;
 }
 

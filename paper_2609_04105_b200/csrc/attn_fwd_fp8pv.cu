@@ -159,6 +159,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  wait_prior_grids();                                           // everything above is this block's own set-up
   const uint32_t tmem = *tslot;
 
   // Every role walks the same schedule.  Phase ph (0 .. n_my) carries the first sweep ("A": scores -> row maxima) of
@@ -341,7 +342,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         tmem_wait_ld();
         Lhw = __uint_as_float(r16[0]);
       }
-      const float inv = __frcp_rn(Lhw * __ldg(pp.v_G + wi.kvh));
+      const float inv = __frcp_rn(Lhw * __ldcg(pp.v_G + wi.kvh));
       if (lane == 0) bulk_wait_read_all();
       __syncwarp();
 #pragma unroll
@@ -389,7 +390,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const uint32_t smdone = bar(B8_SMDONE0 + pr), pfree = bar(B8_PFREE0 + pr);
     const uint32_t tP = tmem + ((uint32_t)(quarter * 32) << 16) + k8ColP + 32 * pr + 16 * h;
     float c32;
-    if (NV) c32 = __fdiv_rn(p.c_base, __fmul_rn(__ldg(p.q_G), __ldg(p.k_G)));
+    if (NV) c32 = __fdiv_rn(p.c_base, __fmul_rn(__ldcg(p.q_G), __ldcg(p.k_G)));
     else    c32 = __fdiv_rn(p.c_base, 36.0f);
     bool ok = true;
     uint32_t g = 0;                                             // steps so far (both kinds, all pairs)
@@ -514,7 +515,7 @@ static int launch_fp8(const fp4attn_operands* ops, int B, int H, int N, const Fp
   const CUtensorMap* tm = attention_tensor_maps_fp8v(D, ops, prm.a.O, B, H, prm.a.Hkv, N);
   if (!tm) return FP4ATTN_ERR_CUDA;
   const unsigned grid = (unsigned)(prm.a.n_items < sms ? prm.a.n_items : sms);
-  attn_fwd_fp8pv_kernel<D, NV, CAUSAL><<<grid, kAttnThreads, C8::SMEM_BYTES, st>>>(tm[0], tm[1], tm[2], tm[3], prm);
+  launch_overlapped(attn_fwd_fp8pv_kernel<D, NV, CAUSAL>, dim3(grid), kAttnThreads, C8::SMEM_BYTES, st, tm[0], tm[1], tm[2], tm[3], prm);
   return cudaGetLastError() == cudaSuccess ? FP4ATTN_OK : FP4ATTN_ERR_CUDA;
 }
 

@@ -86,6 +86,30 @@ __device__ __forceinline__ float mx_inv_amplitude(uint32_t u) {
   return __uint_as_float(u == 254u ? 0x00400000u : ((254u - u) << 23));
 }
 
+// Programmatic dependent launch.  Every quantizer kernel lets its successor start when its own last blocks have
+// (launch_dependents in each block's first instructions), and every kernel of the path touches global memory only after wait_prior_grids, which
+// returns when all earlier kernels of the stream are complete and their writes visible.  What overlaps is a kernel's launch
+// and its set-up with the tail of the one before: the 1.5-2.5 us between two kernels of a step (B=1, H=16, N=4096, affine map,
+// whole step: 73.7 -> 64.0 us).  The attention kernels wait but do not announce: the next step's quantizer blocks, resident
+// beside an attention block and waiting, cost it up to 3 % (B=32, H=16, N=1024: 242 against 228 us a step).
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_prior_grids() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... Params, class... Args>
+cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 constexpr int kMaxDevices = 64;      // per-device host-side caches are arrays of this length
 
 int check_device_sm100();            // FP4ATTN_OK or FP4ATTN_ERR_UNSUPPORTED_ARCH / _CUDA

@@ -1,22 +1,20 @@
 // Operand quantizers: bf16 -> packed E2M1 + scale bytes in the 128x4 atom order.
-// HBM-bound: 128-bit loads, block amax by lane shuffles, 32-bit / 128-bit stores.
+// HBM-bound: 128-bit loads, block amax by lane shuffles, 32-bit / 128-bit stores.  Loads are ld.global.cg: a kernel may have
+// started before its inputs were written (programmatic dependent launch), which rules out the non-coherent path.
 #include "common.cuh"
 
 namespace fp4attn {
 
 constexpr int kThreads = 256;
-constexpr int kGroupsPerThread = 4;          // 16-byte loads in flight per thread
-constexpr int kGroupsPerCta = kThreads * kGroupsPerThread;
+constexpr int kGroupsPerCta = 1024;          // 16-byte groups (eight elements) of a chunk: what a CTA takes at a time
+constexpr int kLoads = kGroupsPerCta / 2 / kThreads;   // 32-byte loads of a thread and chunk
+constexpr int kRowsCtas = 4;                  // CTAs of the rows kernels per SM
 constexpr int kMaxPartials = 1024;           // NVFP4 amax pass: one partial maximum per block
 constexpr int kPartialsPerHead = 32;         // the same, per (batch, head) unit, for per-head factors
 
 // ---------------------------------------------------------------- MXFP4, blocks along d (Q, K)
 // |bf16| bit patterns order like the magnitudes, so the block maximum is taken on packed 16-bit
 // integers; 6 v / alpha = v * (1.5 * 2^(129-u)) is one exact fp32 multiply.
-__device__ __forceinline__ uint32_t absmax_bf16x8(const uint4& r) {
-  const uint32_t m = __vmaxu2(__vmaxu2(r.x & 0x7FFF7FFFu, r.y & 0x7FFF7FFFu), __vmaxu2(r.z & 0x7FFF7FFFu, r.w & 0x7FFF7FFFu));
-  return max(m & 0xFFFFu, m >> 16);
-}
 // E8M0 byte from the bf16 bit pattern of the block maximum a = (1 + m/128) 2^(e-127): the biased exponent
 // e, plus one where the rule rounds the amplitude up (Eq. "mx-scale" allows either neighbouring power of
 // two): ceiling - whenever a is not a power of two; threshold - alpha = 2^floor(log2(1.6 a)), i.e. when
@@ -28,15 +26,19 @@ __device__ __forceinline__ uint32_t mx_scale_byte_bf16(uint32_t a16) {
   const uint32_t up = RULE == FP4ATTN_QSCALE_CEIL ? (m != 0) : RULE == FP4ATTN_QSCALE_THR16 ? (m >= 32u) : 0u;
   return min(max((a16 >> 7) + up, 1u), 254u);
 }
+// two products per instruction
+template <int N_>
+__device__ __forceinline__ void scale_values(float* v, float f) {
+#pragma unroll
+  for (int i = 0; i < N_; i += 2)
+    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %4};\n\tmul.rn.f32x2 c, a, b;\n\tmov.b64 {%0, %1}, c;\n\t}"
+        : "=f"(v[i]), "=f"(v[i + 1]) : "f"(v[i]), "f"(v[i + 1]), "f"(f));
+}
 // v[i] <- 6 v[i] / alpha for the amplitude of byte u: exact in fp32 (one multiply by 1.5 * 2^k)
 template <int N_>
 __device__ __forceinline__ void mx_scale_values(float* v, uint32_t u) {
   if (u >= 2u) {
-    const float s6 = __uint_as_float(((256u - u) << 23) | 0x400000u);   // 1.5 * 2^(129-u) = 6 / alpha
-#pragma unroll
-    for (int i = 0; i < N_; i += 2)                                       // two exact products per instruction
-      asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %4};\n\tmul.rn.f32x2 c, a, b;\n\tmov.b64 {%0, %1}, c;\n\t}"
-          : "=f"(v[i]), "=f"(v[i + 1]) : "f"(v[i]), "f"(v[i + 1]), "f"(s6));
+    scale_values<N_>(v, __uint_as_float(((256u - u) << 23) | 0x400000u));   // 1.5 * 2^(129-u) = 6 / alpha
   } else {                                                              // alpha = 2^-126: 6/alpha overflows fp32
     const float inv = mx_inv_amplitude(u);
 #pragma unroll
@@ -49,72 +51,119 @@ __device__ __forceinline__ uint32_t mx_codes_x8(const uint4& raw, uint32_t u) {
   mx_scale_values<8>(v, u);
   return cvt_e2m1x8(v);
 }
-// MSE rule, blocks along d: the four eight-element groups of a block sit in four adjacent lanes, so the
-// group sums meet as (g0 + g1) + (g2 + g3) in every lane.  The floor's error is in units four times
+// MSE rule, blocks along d: two eight-element groups of a block sit in a lane, the other two in its neighbour, so the
+// group sums meet as (g0 + g1) + (g2 + g3) in both.  The floor's error is in units four times
 // smaller than the ceiling's, hence the factor; the floor wins only if strictly better.  Returns the
 // chosen byte, `word` gets this lane's codes under it.
-__device__ __forceinline__ uint32_t mx_choose_mse_rows(const uint4& raw, uint32_t a16, uint32_t& word) {
+__device__ __forceinline__ uint32_t mx_choose_mse_rows(const uint32_t* raw, uint32_t a16, uint32_t* words) {
   const uint32_t uf = mx_scale_byte_bf16<FP4ATTN_QSCALE_FLOOR>(a16), uc = mx_scale_byte_bf16<FP4ATTN_QSCALE_CEIL>(a16);
-  float tf[8], tc[8];
-  bf16x8_to_f32(raw, tf);
+  uint32_t wf[2], wc[2];
+  float ef[2], ec[2];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) tc[i] = tf[i];
-  mx_scale_values<8>(tf, uf);
-  mx_scale_values<8>(tc, uc);
-  const uint32_t wf = cvt_e2m1x8(tf), wc = cvt_e2m1x8(tc);
-  float ef = mx_error_x8(tf, wf), ec = mx_error_x8(tc, wc);
-  ef = __fadd_rn(ef, __shfl_xor_sync(0xffffffffu, ef, 1));
-  ec = __fadd_rn(ec, __shfl_xor_sync(0xffffffffu, ec, 1));
-  ef = __fadd_rn(ef, __shfl_xor_sync(0xffffffffu, ef, 2));
-  ec = __fadd_rn(ec, __shfl_xor_sync(0xffffffffu, ec, 2));
-  const bool take_f = (uf != uc) && (ef < __fmul_rn(4.0f, ec));
-  word = take_f ? wf : wc;
+  for (int h = 0; h < 2; ++h) {
+    float tf[8], tc[8];
+    bf16x8_to_f32(make_uint4(raw[4 * h], raw[4 * h + 1], raw[4 * h + 2], raw[4 * h + 3]), tf);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) tc[i] = tf[i];
+    mx_scale_values<8>(tf, uf);
+    mx_scale_values<8>(tc, uc);
+    wf[h] = cvt_e2m1x8(tf);
+    wc[h] = cvt_e2m1x8(tc);
+    ef[h] = mx_error_x8(tf, wf[h]);
+    ec[h] = mx_error_x8(tc, wc[h]);
+  }
+  float f = __fadd_rn(ef[0], ef[1]), c = __fadd_rn(ec[0], ec[1]);
+  f = __fadd_rn(f, __shfl_xor_sync(0xffffffffu, f, 1));
+  c = __fadd_rn(c, __shfl_xor_sync(0xffffffffu, c, 1));
+  const bool take_f = (uf != uc) && (f < __fmul_rn(4.0f, c));
+  words[0] = take_f ? wf[0] : wc[0];
+  words[1] = take_f ? wf[1] : wc[1];
   return take_f ? uf : uc;
 }
 
-// grid (N * D/8 / kGroupsPerCta, B*H)
-template <int D, int RULE>
-__global__ void __launch_bounds__(kThreads)
-quant_mx_rows_kernel(const uint4* __restrict__ x, uint32_t* __restrict__ packed,
-                     uint8_t* __restrict__ sf, int N) {
-  constexpr int GPR = D / 8;                       // 8-element groups per row
-  const uint32_t bh = blockIdx.y;
-  const uint32_t gl = blockIdx.x * kGroupsPerCta + threadIdx.x;
-  const size_t gbase = (size_t)bh * N * GPR;
-  uint8_t* sfb = sf + (size_t)bh * (N / 128) * 512;
-  uint4 raw[kGroupsPerThread];
+// 32 bytes in one load (64 a thread and chunk, and the next chunk's in flight while this one is converted): sixteen elements
+// of a row, so that half a 32-block, or a whole 16-block, needs no lane exchange and its scale is formed once, not twice.
+// W32: the tensor starts on a 32-byte boundary; one that only starts on a 16-byte boundary takes two loads.
+template <bool W32>
+__device__ __forceinline__ void load_16(uint32_t* r, const uint4* p) {
+  if (W32) {
+    asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "l"(p) : "memory");
+  } else {
+    const uint4 lo = __ldcg(p), hi = __ldcg(p + 1);
+    r[0] = lo.x; r[1] = lo.y; r[2] = lo.z; r[3] = lo.w;
+    r[4] = hi.x; r[5] = hi.y; r[6] = hi.z; r[7] = hi.w;
+  }
+}
+__device__ __forceinline__ uint32_t absmax_bf16x16(const uint32_t* r) {
+  uint32_t m = r[0] & 0x7FFF7FFFu;
 #pragma unroll
-  for (int k = 0; k < kGroupsPerThread; ++k) raw[k] = __ldg(x + gbase + gl + k * kThreads);
+  for (int i = 1; i < 8; ++i) m = __vmaxu2(m, r[i] & 0x7FFF7FFFu);
+  return max(m & 0xFFFFu, m >> 16);
+}
+
+// Bound by HBM.  67 M elements back to back on one stream: 26.7 us, 6.37 TB/s (one CTA per chunk, 16-byte loads, byte stores
+// of the scales, a plain launch: 30.8); 3 / 4 / 5 CTAs per SM 27.5 / 26.7 / 27.6.
+// The rows of all units are one list (a unit is a whole number of 128-row atoms), cut into chunks of kGroupsPerCta groups.
+// grid rows_grid(): persistent CTAs that walk the chunks
+template <int D, int RULE, bool W32>
+__global__ void __launch_bounds__(kThreads, RULE == FP4ATTN_QSCALE_MSE ? 3 : kRowsCtas)
+quant_mx_rows_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, uint8_t* __restrict__ sf, uint32_t n_chunks) {
+  constexpr uint32_t LPR = D / 16;                 // lanes per row
+  launch_dependents();
+  wait_prior_grids();
+  const uint32_t seg = threadIdx.x % LPR;
+  uint32_t chunk = blockIdx.x, raw[kLoads][8];
 #pragma unroll
-  for (int k = 0; k < kGroupsPerThread; ++k) {
-    const uint32_t g = gl + k * kThreads;
-    uint32_t a = absmax_bf16x8(raw[k]);
-    a = max(a, __shfl_xor_sync(0xffffffffu, a, 1));
-    a = max(a, __shfl_xor_sync(0xffffffffu, a, 2));
-    uint32_t u, word;
-    if (RULE == FP4ATTN_QSCALE_MSE) {
-      u = mx_choose_mse_rows(raw[k], a, word);
-    } else {
-      u = mx_scale_byte_bf16<RULE>(a);
-      word = mx_codes_x8(raw[k], u);
+  for (int k = 0; k < kLoads; ++k) load_16<W32>(raw[k], x + (size_t)chunk * kGroupsPerCta + 2 * (threadIdx.x + k * kThreads));
+  while (true) {
+    const uint32_t next = chunk + gridDim.x;
+    uint32_t ahead[kLoads][8];
+    if (next < n_chunks) {
+#pragma unroll
+      for (int k = 0; k < kLoads; ++k) load_16<W32>(ahead[k], x + (size_t)next * kGroupsPerCta + 2 * (threadIdx.x + k * kThreads));
     }
-    packed[gbase + g] = word;
-    const uint32_t row = g / GPR, seg = g % GPR;
-    uint8_t* p = sfb + (row >> 7) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4;
-    if ((seg & 3) == 0) p[seg >> 2] = (uint8_t)u;                    // one lane per 32-block
-    if (D == 64 && (seg & 3) == 1) p[2 + (seg >> 2)] = 0;            // padding columns
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k) {
+      uint32_t a = absmax_bf16x16(raw[k]);
+      a = max(a, __shfl_xor_sync(0xffffffffu, a, 1));
+      uint32_t u, w[2];
+      if (RULE == FP4ATTN_QSCALE_MSE) {
+        u = mx_choose_mse_rows(raw[k], a, w);
+      } else {
+        u = mx_scale_byte_bf16<RULE>(a);
+        w[0] = mx_codes_x8(make_uint4(raw[k][0], raw[k][1], raw[k][2], raw[k][3]), u);
+        w[1] = mx_codes_x8(make_uint4(raw[k][4], raw[k][5], raw[k][6], raw[k][7]), u);
+      }
+      packed[(size_t)chunk * (kGroupsPerCta / 2) + threadIdx.x + k * kThreads] = make_uint2(w[0], w[1]);
+      // the row's scale bytes as one word, from the lanes of its blocks (d = 64: two of them, and two columns of padding)
+      u |= __shfl_xor_sync(0xffffffffu, u, 2) << 8;
+      if (D == 128) u |= __shfl_xor_sync(0xffffffffu, u, 4) << 16;
+      const uint32_t row = chunk * (kGroupsPerCta / 2 / LPR) + (threadIdx.x + k * kThreads) / LPR;
+      if (seg == 0) *reinterpret_cast<uint32_t*>(sf + (size_t)(row >> 7) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4) = u;
+    }
+    if (next >= n_chunks) return;
+    chunk = next;
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) raw[k][i] = ahead[k][i];
   }
 }
 
 // ---------------------------------------------------------------- MXFP4, blocks along keys (V), transposed out
 // A [128 keys x D] tile (contiguous in memory) goes through shared memory; a thread owns two adjacent head-dim
-// columns and one 32-key block, reads them as bf16x2 words (conflict-free) and writes two 16-byte code groups.
+// columns and one 32-key block, reads them as bf16x2 words and writes two 16-byte code groups.  A warp owns eight column
+// pairs of all four key blocks, so that a column's four code groups leave as 64 contiguous bytes (two whole sectors) and its
+// four scale bytes meet by lane exchange; 16-byte chunk c of a tile row sits at c ^ 2 (key block), which keeps the reads of
+// the four blocks in different banks.  (One warp per key block, with half-sector stores and the scale bytes meeting in shared
+// memory: 29.5 us for 67 M elements at d = 128; this way 29.0.)
 // Persistent CTAs walk the tiles with two tile buffers: the asynchronous copies (cp.async, 16 bytes per thread
 // and copy, no registers in between) of the next tile are in flight while the current one is converted, so the
 // memory system always has work although each tile passes through a load -> barrier -> convert sequence.
-// grid min(tiles, CTAs that fit) , 2*D threads, dynamic shared memory kVSmem<D>
+// grid min(tiles, CTAs that fit) , 2*D threads, dynamic shared memory two tiles
 template <int D> constexpr int kVTileBytes = 128 * D * 2;
-template <int D> constexpr int kVSmem = 2 * kVTileBytes<D> + 512;
+template <int D> __device__ __forceinline__ uint32_t v_swizzle(uint32_t key) { return 2 * ((key >> 5) & 3); }   // on the chunk index
 __device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -128,24 +177,26 @@ quant_mx_v_kernel(const uint4* __restrict__ x, uint4* __restrict__ packed, uint8
   constexpr int T = 2 * D;                         // threads: D/2 column pairs x 4 key blocks
   constexpr int LOADS = 128 * D / 8 / T;           // 16-byte copies per thread and tile: 8
   extern __shared__ __align__(16) uint8_t vsm[];
-  uint8_t* sfb = vsm + 2 * kVTileBytes<D>;
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(vsm);
   const int tiles_per_head = N / 128;
-  const int cp = threadIdx.x % (D / 2);            // column pair: columns 2cp, 2cp+1
-  const int kb = threadIdx.x / (D / 2);            // key block 0..3
+  const int cp = (threadIdx.x >> 5) * 8 + (threadIdx.x & 7);   // column pair: columns 2cp, 2cp+1
+  const int kb = (threadIdx.x >> 3) & 3;           // key block 0..3
   auto issue = [&](int t, int buf) {               // tile t is contiguous: 128 keys x D bf16 starting at key 128 t of the flat [B*H*N] key space
     const uint4* src = x + (size_t)t * (128 * D / 8);
 #pragma unroll
-    for (int k = 0; k < LOADS; ++k)
-      cp_async_16(sbase + buf * kVTileBytes<D> + (threadIdx.x + k * T) * 16, src + threadIdx.x + k * T);
+    for (int k = 0; k < LOADS; ++k) {
+      const uint32_t j = threadIdx.x + k * T;      // 16-byte chunk of the tile, in row j / (D / 8)
+      cp_async_16(sbase + buf * kVTileBytes<D> + (j ^ v_swizzle<D>(j / (D / 8))) * 16, src + j);
+    }
     cp_async_commit();
   };
   int t = blockIdx.x, i = 0;
+  launch_dependents();
+  wait_prior_grids();
   if (t < n_tiles) issue(t, 0);
   for (; t < n_tiles; t += gridDim.x, ++i) {
     const int tn = t + gridDim.x;
     if (tn < n_tiles) { issue(tn, (i + 1) & 1); cp_async_wait<1>(); } else { cp_async_wait<0>(); }
-    if (threadIdx.x < 128) reinterpret_cast<uint32_t*>(sfb)[threadIdx.x] = 0;
     __syncthreads();
     const uint32_t* tile = reinterpret_cast<const uint32_t*>(vsm + (i & 1) * kVTileBytes<D>);
     const size_t bh = t / tiles_per_head;
@@ -154,7 +205,7 @@ quant_mx_v_kernel(const uint4* __restrict__ x, uint4* __restrict__ packed, uint8
     uint32_t m = 0;
 #pragma unroll
     for (int r = 0; r < 32; ++r) {
-      w[r] = tile[(kb * 32 + r) * (D / 2) + cp];
+      w[r] = tile[(kb * 32 + r) * (D / 2) + (cp ^ (8 * kb))];
       m = __vmaxu2(m, w[r] & 0x7FFF7FFFu);
     }
 #pragma unroll
@@ -196,16 +247,38 @@ quant_mx_v_kernel(const uint4* __restrict__ x, uint4* __restrict__ packed, uint8
       }
       const int col = 2 * cp + c;
       packed[((bh * D + col) * (size_t)(N / 2) + (size_t)kt * 64 + kb * 16) / 16] = out;
-      sfb[col * 4 + kb] = (uint8_t)u;
+      u |= __shfl_xor_sync(0xffffffffu, u, 8) << 8;  // kb 0: bytes of blocks 0, 1 (kb 2: of 2, 3)
+      u |= __shfl_xor_sync(0xffffffffu, u, 16) << 16;
+      uint32_t* atom = reinterpret_cast<uint32_t*>(sf + (size_t)t * 512);   // row r at word (r % 32) * 4 + r / 32
+      if (kb == 0) atom[(col & 31) * 4 + (col >> 5)] = u;
+      if (D == 64 && kb == 1) atom[(col & 31) * 4 + 2 + (col >> 5)] = 0;    // rows from 64 on are padding
     }
-    __syncthreads();
-    if (threadIdx.x < 128) {
-      const int r = threadIdx.x;                     // head-dim row; rows >= D are zero padding
-      uint8_t* p = sf + (bh * (size_t)tiles_per_head + kt) * 512 + (r & 31) * 16 + (r >> 5) * 4;
-      *reinterpret_cast<uint32_t*>(p) = reinterpret_cast<const uint32_t*>(sfb)[r];
-    }
-    __syncthreads();                                 // the tile buffer and the scale staging are free again
+    __syncthreads();                                 // the tile buffer is free again
   }
+}
+
+// Encode factor of a tensor or unit from its partial maxima: fl32(top / max), 1 for an all-zero one.  Each kernel that needs
+// the factor takes it so (at most 1024 partials, in L2) instead of waiting for a kernel of its own to form it.
+// encode_factor_warp: every warp by itself, at most 32 partials; encode_factor_block: the whole block, with a barrier.
+__device__ __forceinline__ float encode_factor_of(float amax, float top) { return amax == 0.f ? 1.0f : __fdiv_rn(top, amax); }
+__device__ __forceinline__ float encode_factor_warp(const float* partials, int n_partials, float top) {
+  const int lane = threadIdx.x & 31;
+  float a = lane < n_partials ? __ldcg(partials + lane) : 0.f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
+  return encode_factor_of(a, top);
+}
+__device__ __forceinline__ float encode_factor_block(const float* partials, int n_partials, float top) {
+  __shared__ float wmax[kThreads / 32];
+  float a = 0.f;
+  for (int i = threadIdx.x; i < n_partials; i += kThreads) a = fmaxf(a, __ldcg(partials + i));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
+  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = a;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kThreads / 32; ++i) a = fmaxf(a, wmax[i]);
+  return encode_factor_of(a, top);
 }
 
 // ---------------------------------------------------------------- E4M3 V (FP8 P/V route), transposed out
@@ -222,34 +295,40 @@ __device__ __forceinline__ uint32_t cvt_e4m3x4(float a, float b, float c, float 
 }
 template <int D>
 __global__ void __launch_bounds__(2 * D, D == 128 ? 3 : 6)
-quant_e4m3_v_kernel(const uint4* __restrict__ x, uint4* __restrict__ bytes_out, const float* __restrict__ G_in, int N, int n_tiles) {
+quant_e4m3_v_kernel(const uint4* __restrict__ x, uint4* __restrict__ bytes_out, const float* __restrict__ partials, int n_partials,
+                    float* __restrict__ G_out, int N, int n_tiles) {
   constexpr int T = 2 * D;
   constexpr int LOADS = 128 * D / 8 / T;
   extern __shared__ __align__(16) uint8_t vsm[];
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(vsm);
   const int tiles_per_head = N / 128;
-  const int cp = threadIdx.x % (D / 2);
-  const int kb = threadIdx.x / (D / 2);
+  const int cp = (threadIdx.x >> 5) * 8 + (threadIdx.x & 7);
+  const int kb = (threadIdx.x >> 3) & 3;
   auto issue = [&](int t, int buf) {
     const uint4* src = x + (size_t)t * (128 * D / 8);
 #pragma unroll
-    for (int k = 0; k < LOADS; ++k)
-      cp_async_16(sbase + buf * kVTileBytes<D> + (threadIdx.x + k * T) * 16, src + threadIdx.x + k * T);
+    for (int k = 0; k < LOADS; ++k) {
+      const uint32_t j = threadIdx.x + k * T;      // 16-byte chunk of the tile, in row j / (D / 8)
+      cp_async_16(sbase + buf * kVTileBytes<D> + (j ^ v_swizzle<D>(j / (D / 8))) * 16, src + j);
+    }
     cp_async_commit();
   };
-  int t = blockIdx.x, i = 0;
-  if (t < n_tiles) issue(t, 0);
-  for (; t < n_tiles; t += gridDim.x, ++i) {
-    const int tn = t + gridDim.x;
-    if (tn < n_tiles) { issue(tn, (i + 1) & 1); cp_async_wait<1>(); } else { cp_async_wait<0>(); }
+  int t = n_tiles - 1 - (int)blockIdx.x, i = 0;    // from the end of the tensor: the amax pass has read that last
+  launch_dependents();
+  wait_prior_grids();
+  if (t >= 0) issue(t, 0);
+  for (; t >= 0; t -= gridDim.x, ++i) {
+    const int tn = t - (int)gridDim.x;
+    if (tn >= 0) { issue(tn, (i + 1) & 1); cp_async_wait<1>(); } else { cp_async_wait<0>(); }
     __syncthreads();
     const uint32_t* tile = reinterpret_cast<const uint32_t*>(vsm + (i & 1) * kVTileBytes<D>);
     const size_t bh = t / tiles_per_head;
     const int kt = t - (int)bh * tiles_per_head;
-    const float G = __ldg(G_in + bh);
+    const float G = encode_factor_warp(partials + bh * n_partials, n_partials, 448.0f);
+    if (kt == 0 && threadIdx.x == 0) G_out[bh] = G;
     uint32_t w[32];
 #pragma unroll
-    for (int r = 0; r < 32; ++r) w[r] = tile[(kb * 32 + r) * (D / 2) + cp];
+    for (int r = 0; r < 32; ++r) w[r] = tile[(kb * 32 + r) * (D / 2) + (cp ^ (8 * kb))];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       uint32_t o[8];
@@ -270,39 +349,33 @@ quant_e4m3_v_kernel(const uint4* __restrict__ x, uint4* __restrict__ bytes_out, 
   }
 }
 
-// One block per unit: G = fl32(448 / max of the unit's partial maxima) (1 for an all-zero unit)
-__global__ void __launch_bounds__(kThreads)
-e4m3_encode_factor_kernel(const float* __restrict__ partials, int n_partials, float* __restrict__ G_out) {
-  partials += (size_t)blockIdx.x * n_partials;
-  float a = 0.f;
-  for (int i = threadIdx.x; i < n_partials; i += kThreads) a = fmaxf(a, partials[i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
-  __shared__ float wmax[kThreads / 32];
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = a;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = 1; i < kThreads / 32; ++i) a = fmaxf(a, wmax[i]);
-    G_out[blockIdx.x] = (a == 0.f) ? 1.0f : __fdiv_rn(448.0f, a);
-  }
-}
-
 // ---------------------------------------------------------------- NVFP4 pass 1: amax partials
 // grid (P, U): U = 1 for the tensor-wide maximum, U = B*H for one maximum per (batch, head) unit; row y of
 // the grid covers groups [y * n_groups, (y + 1) * n_groups) and writes partials[y * P .. y * P + P)
+template <bool W32>
 __global__ void __launch_bounds__(kThreads)
 amax_partials_kernel(const uint4* __restrict__ x, size_t n_groups, float* __restrict__ partials) {
   x += (size_t)blockIdx.y * n_groups;
   partials += (size_t)blockIdx.y * gridDim.x;
-  // |bf16| bit patterns order like the magnitudes: packed 16-bit maxima, four independent loads per trip
+  launch_dependents();
+  wait_prior_grids();
+  // |bf16| bit patterns order like the magnitudes: packed 16-bit maxima, four independent 32-byte loads per trip
   uint32_t m = 0;
   const size_t stride = (size_t)gridDim.x * kThreads;
   size_t g = (size_t)blockIdx.x * kThreads + threadIdx.x;
+  n_groups /= 2;                                   // 32 bytes each
   for (; g + 3 * stride < n_groups; g += 4 * stride) {
-    const uint4 r0 = __ldg(x + g), r1 = __ldg(x + g + stride), r2 = __ldg(x + g + 2 * stride), r3 = __ldg(x + g + 3 * stride);
-    m = max(max(m, absmax_bf16x8(r0)), max(absmax_bf16x8(r1), max(absmax_bf16x8(r2), absmax_bf16x8(r3))));
+    uint32_t r[4][8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) load_16<W32>(r[k], x + 2 * (g + k * stride));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m = max(m, absmax_bf16x16(r[k]));
   }
-  for (; g < n_groups; g += stride) m = max(m, absmax_bf16x8(__ldg(x + g)));
+  for (; g < n_groups; g += stride) {
+    uint32_t r[8];
+    load_16<W32>(r, x + 2 * g);
+    m = max(m, absmax_bf16x16(r));
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
   __shared__ uint32_t wmax[kThreads / 32];
@@ -311,24 +384,6 @@ amax_partials_kernel(const uint4* __restrict__ x, size_t n_groups, float* __rest
   if (threadIdx.x == 0) {
     for (int i = 1; i < kThreads / 32; ++i) m = max(m, wmax[i]);
     partials[blockIdx.x] = __uint_as_float(m << 16);
-  }
-}
-
-// One block per encode factor: G = fl32(2688 / max of its partial maxima) (1 for an all-zero tensor or unit).
-// grid (U): block y reads partials[y * n_partials ..) and writes G_out[y]
-__global__ void __launch_bounds__(kThreads)
-nv_encode_factor_kernel(const float* __restrict__ partials, int n_partials, float* __restrict__ G_out) {
-  partials += (size_t)blockIdx.x * n_partials;
-  float a = 0.f;
-  for (int i = threadIdx.x; i < n_partials; i += kThreads) a = fmaxf(a, partials[i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
-  __shared__ float wmax[kThreads / 32];
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = a;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = 1; i < kThreads / 32; ++i) a = fmaxf(a, wmax[i]);
-    G_out[blockIdx.x] = (a == 0.f) ? 1.0f : __fdiv_rn(2688.0f, a);
   }
 }
 
@@ -343,42 +398,69 @@ __device__ __forceinline__ float e4m3_byte_to_f32(uint32_t b) {
   return __half2float(__ushort_as_half((unsigned short)(h2 & 0xFFFFu)));
 }
 
-// ---------------------------------------------------------------- NVFP4 pass 3, blocks of 16 along d (Q, K)
-// grid (N * D/8 / kGroupsPerCta, B*H)
-template <int D>
-__global__ void __launch_bounds__(kThreads)
-quant_nv_rows_kernel(const uint4* __restrict__ x, uint32_t* __restrict__ packed, uint8_t* __restrict__ sf,
-                     const float* __restrict__ G_in, int N, int per_head) {
-  constexpr int GPR = D / 8;
-  constexpr int CT = (D / 16 + 3) / 4;
-  const float G = __ldg(G_in + (per_head ? blockIdx.y : 0));    // this block's (batch, head) unit, or the tensor's
-  const uint32_t bh = blockIdx.y;
-  const uint32_t gl = blockIdx.x * kGroupsPerCta + threadIdx.x;
-  const size_t gbase = (size_t)bh * N * GPR;
-  uint8_t* sfb = sf + (size_t)bh * (N / 128) * CT * 512;
-  uint4 raw[kGroupsPerThread];
+// ---------------------------------------------------------------- NVFP4 pass 2, blocks of 16 along d (Q, K)
+// Bound by HBM (twice over the tensor, less what is left of it in L2) and by the two IEEE divisions per block.  67 M elements,
+// both passes: 50.6 us; with a kernel of its own for the factor, a block's scale formed in two lanes and plain launches 61.6.
+// The chunks and the grid of quant_mx_rows_kernel, walked from the tensor's end (the amax pass has read that last).  A chunk
+// lies within one unit; `chunks_per_unit` is 0 when the tensor has one factor, else a CTA forms its unit's for every chunk.
+template <int D, bool W32>
+__global__ void __launch_bounds__(kThreads, kRowsCtas)
+quant_nv_rows_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, uint8_t* __restrict__ sf,
+                     const float* __restrict__ partials, int n_partials, float* __restrict__ G_out, uint32_t n_chunks,
+                     uint32_t chunks_per_unit) {
+  constexpr uint32_t LPR = D / 16;
+  constexpr uint32_t CT = (D / 16 + 3) / 4;
+  launch_dependents();
+  wait_prior_grids();
+  const uint32_t seg = threadIdx.x % LPR;
+  uint32_t i = blockIdx.x, raw[kLoads][8];
 #pragma unroll
-  for (int k = 0; k < kGroupsPerThread; ++k) raw[k] = __ldg(x + gbase + gl + k * kThreads);
+  for (int k = 0; k < kLoads; ++k) load_16<W32>(raw[k], x + (size_t)(n_chunks - 1 - i) * kGroupsPerCta + 2 * (threadIdx.x + k * kThreads));
+  float G = 0.f;
+  if (!chunks_per_unit) {
+    G = encode_factor_block(partials, n_partials, 2688.0f);
+    if (blockIdx.x == 0 && threadIdx.x == 0) G_out[0] = G;
+  }
+  while (true) {
+    const uint32_t chunk = n_chunks - 1 - i;
+    i += gridDim.x;
+    uint32_t ahead[kLoads][8];
+    if (i < n_chunks) {
 #pragma unroll
-  for (int k = 0; k < kGroupsPerThread; ++k) {
-    const uint32_t g = gl + k * kThreads;
-    uint32_t a16 = absmax_bf16x8(raw[k]);
-    a16 = max(a16, __shfl_xor_sync(0xffffffffu, a16, 1));
-    const float a = __uint_as_float(a16 << 16);
-    const float t = __fdiv_rn(__fmul_rn(a, G), 6.0f);
-    const uint32_t sb = cvt_e4m3_byte(t);
-    const float S = e4m3_byte_to_f32(sb);
-    const float r = (S > 0.f) ? __fdiv_rn(G, S) : 0.f;
-    float v[8];
-    bf16x8_to_f32(raw[k], v);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __fmul_rn(v[i], r);       // sign rides along; 0*r = 0 for zero blocks
-    packed[gbase + g] = cvt_e2m1x8(v);
-    const uint32_t row = g / GPR, seg = g % GPR;
-    if ((seg & 1) == 0) {                                        // one lane per 16-block
-      const uint32_t c = seg >> 1;                               // scale column
-      sfb[((row >> 7) * CT + (c >> 2)) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4 + (c & 3)] = (uint8_t)sb;
+      for (int k = 0; k < kLoads; ++k) load_16<W32>(ahead[k], x + (size_t)(n_chunks - 1 - i) * kGroupsPerCta + 2 * (threadIdx.x + k * kThreads));
     }
+    if (chunks_per_unit) {
+      const uint32_t unit = chunk / chunks_per_unit;
+      G = encode_factor_warp(partials + (size_t)unit * n_partials, n_partials, 2688.0f);
+      if (threadIdx.x == 0 && unit * chunks_per_unit == chunk) G_out[unit] = G;
+    }
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k) {
+      const float a = __uint_as_float(absmax_bf16x16(raw[k]) << 16);
+      const float t = __fdiv_rn(__fmul_rn(a, G), 6.0f);
+      uint32_t sb = cvt_e4m3_byte(t);
+      const float S = e4m3_byte_to_f32(sb);
+      const float r = (S > 0.f) ? __fdiv_rn(G, S) : 0.f;
+      uint32_t w[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float v[8];
+        bf16x8_to_f32(make_uint4(raw[k][4 * h], raw[k][4 * h + 1], raw[k][4 * h + 2], raw[k][4 * h + 3]), v);
+        scale_values<8>(v, r);                                     // sign rides along; 0*r = 0 for zero blocks
+        w[h] = cvt_e2m1x8(v);
+      }
+      packed[(size_t)chunk * (kGroupsPerCta / 2) + threadIdx.x + k * kThreads] = make_uint2(w[0], w[1]);
+      sb |= __shfl_xor_sync(0xffffffffu, sb, 1) << 8;              // four columns' bytes as one word
+      sb |= __shfl_xor_sync(0xffffffffu, sb, 2) << 16;
+      const uint32_t row = chunk * (kGroupsPerCta / 2 / LPR) + (threadIdx.x + k * kThreads) / LPR;
+      if ((seg & 3) == 0)
+        *reinterpret_cast<uint32_t*>(sf + ((size_t)(row >> 7) * CT + (seg >> 2)) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4) = sb;
+    }
+    if (i >= n_chunks) return;
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) raw[k][j] = ahead[k][j];
   }
 }
 
@@ -423,23 +505,42 @@ static void launch_mx_v(const uint4* xs, int n_tiles, int N, void* packed, void*
   int grid = ctas[dev].load(std::memory_order_acquire);
   if (!grid) {
     int sms = 0, per_sm = 0;
-    if (cudaFuncSetAttribute(quant_mx_v_kernel<D, RULE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kVSmem<D>) != cudaSuccess ||
+    if (cudaFuncSetAttribute(quant_mx_v_kernel<D, RULE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kVTileBytes<D>) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quant_mx_v_kernel<D, RULE>, 2 * D, kVSmem<D>) != cudaSuccess || per_sm < 1)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quant_mx_v_kernel<D, RULE>, 2 * D, 2 * kVTileBytes<D>) != cudaSuccess || per_sm < 1)
       return;
     grid = sms * per_sm;
     ctas[dev].store(grid, std::memory_order_release);
   }
-  quant_mx_v_kernel<D, RULE><<<n_tiles < grid ? n_tiles : grid, 2 * D, kVSmem<D>, st>>>(xs, (uint4*)packed, (uint8_t*)scales, N, n_tiles);
+  launch_overlapped(quant_mx_v_kernel<D, RULE>, dim3(n_tiles < grid ? n_tiles : grid), 2 * D, 2 * kVTileBytes<D>, st, xs, (uint4*)packed,
+                    (uint8_t*)scales, N, n_tiles);
+}
+
+// Persistent CTAs of the rows kernels: at most what the device holds at once, each with the same number of chunks (within
+// one).  One CTA per chunk would pay a CTA's start - its launch, the wait for the kernels before, the encode factor - every
+// 16 KB.
+static unsigned rows_grid(size_t n_chunks) {
+  static std::atomic<int> sm_count[kMaxDevices];
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return (unsigned)n_chunks;
+  sms = sm_count[dev].load(std::memory_order_acquire);
+  if (!sms) {
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return (unsigned)n_chunks;
+    sm_count[dev].store(sms, std::memory_order_release);
+  }
+  const size_t resident = (size_t)kRowsCtas * sms, rounds = (n_chunks + resident - 1) / resident;
+  return (unsigned)((n_chunks + rounds - 1) / rounds);
 }
 
 // Shared by fp4attn_quantize and the variants that bring their own scratch.
 template <int RULE>
 static void launch_mx(const uint4* xs, int role, int B, int H, int N, int d, void* packed, void* scales, cudaStream_t st) {
   if (role != FP4ATTN_ROLE_V) {
-    const dim3 grid2((unsigned)((size_t)N * d / 8 / kGroupsPerCta), (unsigned)(B * H));   // N % 128 == 0 makes this exact
-    if (d == 128) quant_mx_rows_kernel<128, RULE><<<grid2, kThreads, 0, st>>>(xs, (uint32_t*)packed, (uint8_t*)scales, N);
-    else          quant_mx_rows_kernel<64, RULE><<<grid2, kThreads, 0, st>>>(xs, (uint32_t*)packed, (uint8_t*)scales, N);
+    const size_t n_chunks = (size_t)B * H * N * d / 8 / kGroupsPerCta;                     // N % 128 == 0 makes this exact
+    const bool w32 = ((uintptr_t)xs & 31) == 0;
+    launch_overlapped(d == 128 ? (w32 ? quant_mx_rows_kernel<128, RULE, true> : quant_mx_rows_kernel<128, RULE, false>)
+                               : (w32 ? quant_mx_rows_kernel<64, RULE, true> : quant_mx_rows_kernel<64, RULE, false>), dim3(rows_grid(n_chunks)), kThreads, 0,
+                      st, xs, (uint2*)packed, (uint8_t*)scales, (uint32_t)n_chunks);
   } else if (d == 128) {
     launch_mx_v<128, RULE>(xs, B * H * (N / 128), N, packed, scales, st);
   } else {
@@ -450,8 +551,7 @@ static void launch_mx(const uint4* xs, int role, int B, int H, int N, int d, voi
 int launch_quantize(const void* x, int fmt, int role, int B, int H, int N, int d, void* packed, void* scales,
                     float* G_out, float* partials, cudaStream_t st, int mx_rule, bool per_head = false) {
   const size_t n_groups = (size_t)B * H * N * d / 8;
-  const unsigned grid = (unsigned)(n_groups / kGroupsPerCta);
-  const dim3 grid2((unsigned)((size_t)N * d / 8 / kGroupsPerCta), (unsigned)(B * H));   // N % 128 == 0 makes this exact
+  const size_t n_chunks = n_groups / kGroupsPerCta, unit_chunks = (size_t)N * d / 8 / kGroupsPerCta;   // N % 128 == 0 makes these exact
   const uint4* xs = reinterpret_cast<const uint4*>(x);
   if (fmt == FP4ATTN_FMT_MXFP4) {
     if (mx_rule == FP4ATTN_QSCALE_THR16)      launch_mx<FP4ATTN_QSCALE_THR16>(xs, role, B, H, N, d, packed, scales, st);
@@ -459,17 +559,16 @@ int launch_quantize(const void* x, int fmt, int role, int B, int H, int N, int d
     else if (mx_rule == FP4ATTN_QSCALE_MSE)   launch_mx<FP4ATTN_QSCALE_MSE>(xs, role, B, H, N, d, packed, scales, st);
     else                                      launch_mx<FP4ATTN_QSCALE_CEIL>(xs, role, B, H, N, d, packed, scales, st);
   } else {
-    int n_partials;
-    if (per_head) {
-      n_partials = (int)(grid2.x < (unsigned)kPartialsPerHead ? grid2.x : kPartialsPerHead);
-      amax_partials_kernel<<<dim3(n_partials, B * H), kThreads, 0, st>>>(xs, n_groups / ((size_t)B * H), partials);
-    } else {
-      n_partials = (int)(grid < (unsigned)kMaxPartials ? grid : kMaxPartials);
-      amax_partials_kernel<<<n_partials, kThreads, 0, st>>>(xs, n_groups, partials);
-    }
-    nv_encode_factor_kernel<<<per_head ? B * H : 1, kThreads, 0, st>>>(partials, n_partials, G_out);
-    if (d == 128) quant_nv_rows_kernel<128><<<grid2, kThreads, 0, st>>>(xs, (uint32_t*)packed, (uint8_t*)scales, G_out, N, per_head);
-    else          quant_nv_rows_kernel<64><<<grid2, kThreads, 0, st>>>(xs, (uint32_t*)packed, (uint8_t*)scales, G_out, N, per_head);
+    const unsigned most = per_head ? (unsigned)kPartialsPerHead : (unsigned)kMaxPartials;
+    const size_t want = per_head ? unit_chunks : n_chunks;
+    const int n_partials = (int)(want < most ? want : most);
+    const bool w32 = ((uintptr_t)xs & 31) == 0;
+    launch_overlapped(w32 ? amax_partials_kernel<true> : amax_partials_kernel<false>, per_head ? dim3(n_partials, B * H) : dim3(n_partials), kThreads, 0, st, xs,
+                      per_head ? n_groups / ((size_t)B * H) : n_groups, partials);
+    launch_overlapped(d == 128 ? (w32 ? quant_nv_rows_kernel<128, true> : quant_nv_rows_kernel<128, false>)
+                               : (w32 ? quant_nv_rows_kernel<64, true> : quant_nv_rows_kernel<64, false>), dim3(rows_grid(n_chunks)), kThreads, 0, st, xs,
+                      (uint2*)packed, (uint8_t*)scales, (const float*)partials, n_partials, G_out, (uint32_t)n_chunks,
+                      (uint32_t)(per_head ? unit_chunks : 0));
   }
   return cudaGetLastError() == cudaSuccess ? FP4ATTN_OK : FP4ATTN_ERR_CUDA;
 }
@@ -568,7 +667,7 @@ extern "C" size_t fp4attn_quantize_v_e4m3_workspace_bytes(int B, int H, int N, i
 }
 
 template <int D>
-static int launch_e4m3_v(const uint4* xs, int BH, int N, void* bytes_out, const float* G, cudaStream_t st) {
+static int launch_e4m3_v(const uint4* xs, int BH, int N, void* bytes_out, const float* partials, int n_partials, float* G, cudaStream_t st) {
   static std::atomic<int> ctas[kMaxDevices];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return FP4ATTN_ERR_CUDA;
@@ -583,7 +682,8 @@ static int launch_e4m3_v(const uint4* xs, int BH, int N, void* bytes_out, const 
     ctas[dev].store(grid, std::memory_order_release);
   }
   const int n_tiles = BH * (N / 128);
-  quant_e4m3_v_kernel<D><<<n_tiles < grid ? n_tiles : grid, 2 * D, 2 * kVTileBytes<D>, st>>>(xs, (uint4*)bytes_out, G, N, n_tiles);
+  launch_overlapped(quant_e4m3_v_kernel<D>, dim3(n_tiles < grid ? n_tiles : grid), 2 * D, 2 * kVTileBytes<D>, st, xs, (uint4*)bytes_out,
+                    partials, n_partials, G, N, n_tiles);
   return FP4ATTN_OK;
 }
 
@@ -603,9 +703,10 @@ extern "C" int fp4attn_quantize_v_e4m3(const void* x, int B, int H, int N, int d
   const size_t groups_per_unit = (size_t)N * d / 8;
   const unsigned gx = (unsigned)(groups_per_unit / kGroupsPerCta);
   const int n_partials = (int)(gx < (unsigned)kPartialsPerHead ? gx : kPartialsPerHead);
-  amax_partials_kernel<<<dim3(n_partials, B * H), kThreads, 0, st>>>(xs, groups_per_unit, (float*)workspace);
-  e4m3_encode_factor_kernel<<<B * H, kThreads, 0, st>>>((const float*)workspace, n_partials, G_out);
-  rc = d == 128 ? launch_e4m3_v<128>(xs, B * H, N, bytes_out, G_out, st) : launch_e4m3_v<64>(xs, B * H, N, bytes_out, G_out, st);
+  launch_overlapped(((uintptr_t)xs & 31) == 0 ? amax_partials_kernel<true> : amax_partials_kernel<false>, dim3(n_partials, B * H), kThreads, 0, st, xs, groups_per_unit, (float*)workspace);
+  const float* partials = (const float*)workspace;
+  rc = d == 128 ? launch_e4m3_v<128>(xs, B * H, N, bytes_out, partials, n_partials, G_out, st)
+                : launch_e4m3_v<64>(xs, B * H, N, bytes_out, partials, n_partials, G_out, st);
   if (rc != FP4ATTN_OK) return rc;
   return cudaGetLastError() == cudaSuccess ? FP4ATTN_OK : FP4ATTN_ERR_CUDA;
 }

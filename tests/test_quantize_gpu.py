@@ -194,6 +194,32 @@ def test_nvfp4_per_head_factors_match_oracle(kw):
         assert got.per_head
 
 
+@pytest.mark.parametrize("offset", [0, 8])          # elements: a tensor on a 32-byte boundary, and on a 16-byte one only
+@pytest.mark.parametrize("B,H,N,d", [(1, 1, 128, 64),       # one 16 KB chunk of the rows kernels
+                                     (1, 1, 128, 128),      # two
+                                     (3, 29, 896, 128),     # 1218 chunks: more than the persistent CTAs, the last ones with one less
+                                     (2, 7, 6144, 64)])     # 672 chunks, 672 tiles of V
+def test_quantizers_at_chunk_edges_and_alignments(B, H, N, d, offset):
+    from paper_2609_04105_b200 import binding as Bd
+    w = I.shrink(I.WORKLOADS["cfg3"], B=B, H=H, N=N, d=d)
+    bits = I.make_qkv(w)[0]
+    buf = torch.empty(bits.size + offset, dtype=torch.bfloat16, device="cuda")
+    x = buf[offset:].view(B, H, N, d)
+    x.copy_(_dev(bits))
+    assert x.data_ptr() % 32 == 2 * offset
+    _check_operand(Bd.fp4attn_quantize(x, Bd.FMT_MXFP4, Bd.ROLE_Q), Qz.quantize_qk(bits, "mx"), Bd.ROLE_Q)
+    _check_operand(Bd.fp4attn_quantize(x, Bd.FMT_NVFP4, Bd.ROLE_K), Qz.quantize_qk(bits, "nv"), Bd.ROLE_K)
+    got, want = Bd.fp4attn_quantize_nvfp4_per_head(x, Bd.ROLE_Q), Qz.quantize_qk(bits, "nv", per_head=True)
+    G = want.pop("G")
+    _check_operand(got, {**want, "G": None}, Bd.ROLE_Q)
+    assert np.array_equal(got.G.cpu().numpy(), G.reshape(-1))
+    _check_operand(Bd.fp4attn_quantize(x, Bd.FMT_MXFP4, Bd.ROLE_V), Qz.quantize_v(bits), Bd.ROLE_V)
+    e, want = Bd.fp4attn_quantize_v_e4m3(x), Qz.quantize_v_e4m3(bits)
+    strip = lambda b: np.where((b & 0x7F) == 0, 0, b)
+    assert np.array_equal(strip(e.packed.cpu().numpy().reshape(want["byte"].shape)), strip(want["byte"]))
+    assert np.array_equal(e.G.cpu().numpy().reshape(B, H), want["G"])
+
+
 def test_nvfp4_per_head_rejects_v_and_missing_workspace():
     from paper_2609_04105_b200 import binding as Bd
     x = torch.zeros((1, 2, 128, 64), dtype=torch.bfloat16, device="cuda")
