@@ -282,7 +282,7 @@ typedef struct {
  * Padded sequences.  With seq_len != NULL, batch entry b holds a sequence of L = seq_len[b] tokens (1 <= L <= N) in
  * buffers laid out for N: keys L..N-1 are removed from every row of that entry exactly as a causal row's invisible
  * keys are (a block's maximum, hence its exponent, is taken over the keys that exist), key tiles that lie entirely
- * beyond L are neither loaded nor multiplied, query tiles that lie entirely beyond L walk one key tile only, and rows
+ * beyond L are neither loaded nor multiplied, query tiles that lie entirely beyond L walk one key tile at most, and rows
  * L..N-1 of O and LSE receive unspecified finite values.  The quantizers see the padded buffers: MXFP4 rows of Q and K
  * are quantized one by one, so their padding rows only have to be finite; a 32-key block of V that straddles L takes its
  * scale from all 32 keys, and an NVFP4 encode factor from the maximum over the whole tensor (or unit), so V's padding

@@ -55,7 +55,8 @@ struct Cfg {
   static constexpr int OFF_OUT = (OFF_STAGE + NST * STAGE_BYTES + 1023) / 1024 * 1024; // bf16 O tile staged for TMA stores: D/64 halves of [128 rows][128 B]
   static constexpr int OUT_BYTES = (D / 64) * BM * 128;
   static constexpr int OFF_BAR = OFF_OUT + OUT_BYTES;
-  static constexpr int SMEM_BYTES = OFF_BAR + 1024 + 1024;      // barriers + alignment slack
+  static constexpr int OFF_SEQ = OFF_BAR + 1024;                // SeqTable
+  static constexpr int SMEM_BYTES = OFF_SEQ + 1536 + 1024;      // + alignment slack
   static constexpr uint64_t SWZ_QK = (ROW_BYTES == 64) ? kSwz64 : kSwz32;
   static_assert(STAGE_BYTES % 512 == 0 && OFF_STAGE % 1024 == 0 && OFF_OUT % 1024 == 0, "stage alignment");
   static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
@@ -80,6 +81,8 @@ struct AttnParams {
   int ref_fixed;           // the constant row reference of the FIXREF instances (octaves)
   const int* seq_len;      // NULL, or B token counts: batch entry b is seq_len[b] tokens padded to N (masked kernels only)
   unsigned long long recip_h;                  // ceil(2^64 / H); 0 for H = 1
+  int B;
+  int sorted;              // seq_len given and B <= kSeqTableMax: the work items come from a SeqTable
 };
 
 // One work item = one 128-row query tile of one (batch, query head).
@@ -92,6 +95,83 @@ struct WorkItem {
   int T2;                  // 128-key stages to walk (causal: up to and including the diagonal; padded: those with a key)
   int len;                 // keys that exist for this unit (N unless the batch entry is a padded sequence)
 };
+// ---- which work items a CTA takes, and in which order (masked kernels)
+// The items of a causal mask or of sequences of unlike lengths differ in cost (stages).  They are numbered from the most
+// expensive down and dealt to the persistent CTAs in rounds of alternating direction: dealt in one direction only, the first
+// CTA gets the dearest item of every round (causal, 64 heads, N = 4096: 269 stages against 254, with a mean of 253).
+template <bool MASKED>
+__device__ __forceinline__ int item_at(int i) {
+  return i * (int)gridDim.x + (MASKED && (i & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x);
+}
+template <bool MASKED>
+__device__ __forceinline__ int items_of_cta(int n_items) {
+  const int rounds = n_items / (int)gridDim.x;
+  return rounds + (item_at<MASKED>(rounds) < n_items ? 1 : 0);
+}
+// Padded sequences: the entries ordered by length, longest first (rank r is entry b[r] with len[r] tokens in T[r] tiles), and
+// the items numbered accordingly, query tiles beyond a length left out (they are only filled with zeros, fill_skipped).
+// Built by every CTA from the token counts.  Without a causal mask rank r has H * T[r] items of T[r] stages each; with it,
+// tile qt costs qt + 1 stages wherever it exists, so the items go tile level by tile level, from T[0] - 1 down, and the
+// levels from T[r] - 1 to T[r + 1] have (r + 1) * H items each.  first[r]: number of the first item of segment r; skipped[r]:
+// of the first left-out tile of rank r.  Both end with the total at [B] and the largest int beyond.
+// (B = 6, H = 12, N = 2176, 436 ... 2176 tokens, d = 64, whole step: 100 -> 77 us; in batch order one CTA had 163 stages
+// and item boundaries where the mean is 111.)
+constexpr int kSeqTableMax = 64;
+struct SeqTable {
+  int first[kSeqTableMax + 1], skipped[kSeqTableMax + 1], T[kSeqTableMax + 1], b[kSeqTableMax], len[kSeqTableMax];
+};
+static_assert(sizeof(SeqTable) <= 1536, "the space behind the barriers");
+// all threads; ends with a barrier
+__device__ __forceinline__ void build_seq_table(SeqTable* st, const AttnParams& p, int qtiles) {
+  const int t = threadIdx.x;
+  int len = 0, rank = 0;
+  if (t < p.B) {
+    len = min(max(__ldcg(p.seq_len + t), 1), p.N);
+    st->first[t] = len;                                          // for the comparison below
+  }
+  __syncthreads();
+  if (t < p.B)
+    for (int k = 0; k < p.B; ++k) {
+      const int T = (st->first[k] + BS - 1) / BS, Tt = (len + BS - 1) / BS;
+      rank += T > Tt || (T == Tt && k < t);
+    }
+  __syncthreads();
+  if (t < p.B) {
+    st->b[rank] = t;
+    st->len[rank] = len;
+    st->T[rank] = (len + BS - 1) / BS;
+  }
+  if (t == p.B) st->T[t] = 0;
+  __syncthreads();
+  if (t <= kSeqTableMax) {
+    int items = 0, left_out = 0;
+    for (int k = 0; k < min(t, p.B); ++k) {
+      items += p.causal ? (st->T[k] - st->T[k + 1]) * (k + 1) : st->T[k];
+      left_out += qtiles - st->T[k];
+    }
+    st->first[t] = t <= p.B ? items * p.H : 0x7FFFFFFF;
+    st->skipped[t] = t <= p.B ? left_out * p.H : 0x7FFFFFFF;
+  }
+  __syncthreads();
+}
+// r with start[r] <= n < start[r + 1]; the whole warp, n the same in every lane
+__device__ __forceinline__ int seq_segment(const int* start, int n) {
+  const int lane = threadIdx.x & 31;
+  return __popc(__ballot_sync(0xffffffffu, start[1 + lane] <= n)) + __popc(__ballot_sync(0xffffffffu, start[33 + lane] <= n));
+}
+// Zeros for O and LSE in the query tiles that no token occupies.  All threads of all CTAs.
+template <int D>
+__device__ __forceinline__ void fill_skipped(const SeqTable* st, const AttnParams& p, int qtiles) {
+  const int total = st->skipped[p.B];
+  for (int j = blockIdx.x; j < total; j += gridDim.x) {
+    const int r = seq_segment(st->skipped, j), n = qtiles - st->T[r], rem = j - st->skipped[r], h = rem / n;
+    const size_t row0 = ((size_t)st->b[r] * p.H + h) * p.N + (size_t)(st->T[r] + rem - h * n) * BM;
+    uint4* o = reinterpret_cast<uint4*>(p.O + row0 * D);
+    for (int k = threadIdx.x; k < BM * D / 8; k += kAttnThreads) o[k] = make_uint4(0u, 0u, 0u, 0u);
+    if (p.LSE && threadIdx.x < BM) p.LSE[row0 + threadIdx.x] = 0.f;
+  }
+}
+
 // floor(n / d) for n < 2^31 through the precomputed reciprocal ceil(2^64 / d) (0 stands for d = 1): the
 // roles decode a work item on their critical path, and a 32-bit division costs some fifty instructions
 __device__ __forceinline__ int fast_div(int n, unsigned long long recip) {
@@ -100,10 +180,32 @@ __device__ __forceinline__ int fast_div(int n, unsigned long long recip) {
 // MASKED: the kernels that mask the last stage of an item - the causal mask (p.causal), padded sequences
 // (p.seq_len), or both.  The unmasked kernels ignore both fields.
 template <bool MASKED>
-__device__ __forceinline__ WorkItem decode_item(int item, const AttnParams& p, int qtiles) {
+__device__ __forceinline__ WorkItem decode_item(int item, const AttnParams& p, int qtiles, const SeqTable* st) {
   constexpr bool CAUSAL = MASKED;
   WorkItem w;
   int bh;
+  if (MASKED && p.sorted) {
+    int r = seq_segment(st->first, item), h;
+    const int rem = item - st->first[r];
+    w.T2 = st->T[r];
+    if (p.causal) {
+      const int width = (r + 1) * p.H, level = rem / width, k = rem - level * width;
+      w.qt = w.T2 - 1 - level;
+      w.T2 = w.qt + 1;
+      r = k / p.H;
+      h = k - r * p.H;
+    } else {
+      h = rem / w.T2;
+      w.qt = rem - h * w.T2;
+    }
+    const int b = st->b[r];
+    w.len = st->len[r];
+    w.bh = b * p.H + h;
+    w.qrow0 = w.bh * p.N + w.qt * BM;
+    w.qtile_lin = w.bh * qtiles + w.qt;
+    w.kvh = p.H != p.Hkv ? b * p.Hkv + h / (p.H / p.Hkv) : w.bh;
+    return w;
+  }
   if (CAUSAL) {             // longest items first, so the persistent CTAs finish together
     const int r = fast_div(item, p.recip_bh);
     w.qt = qtiles - 1 - r;

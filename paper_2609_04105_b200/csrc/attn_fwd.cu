@@ -96,6 +96,16 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   tc_fence_after();
   wait_prior_grids();                                           // everything above is this block's own set-up
   const uint32_t tmem = *tslot;
+  SeqTable* const seq = reinterpret_cast<SeqTable*>(sgen + C::OFF_SEQ);
+  if (CAUSAL && p.sorted) {
+    build_seq_table(seq, p, qtiles);
+    fill_skipped<D>(seq, p, qtiles);
+  }
+  // this CTA's items.  Masked: item_at(0 .. n_my - 1).  Unmasked: blockIdx.x, blockIdx.x + gridDim.x, ... (every role counting
+  // rounds instead of items costs these kernels registers: -1.6 % at d = 64)
+  const int n_my = CAUSAL ? items_of_cta<CAUSAL>(p.sorted ? seq->first[p.B] : p.n_items) : 0;
+  auto mine = [&](int i, int item) { return CAUSAL ? i < n_my : item < p.n_items; };
+  auto work = [&](int i, int item) { return decode_item<CAUSAL>(CAUSAL ? item_at<true>(i) : item, p, qtiles, seq); };
 
   if (warp == 0) {
     // ===================================================================== TMA producer
@@ -104,8 +114,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     uint32_t st = sbase + C::OFF_STAGE;
     bool ok = true;
     int i = 0;
-    for (int item = blockIdx.x; ok && item < p.n_items; item += gridDim.x, ++i) {
-      const WorkItem wi = decode_item<CAUSAL>(item, p, qtiles);
+    for (int item = blockIdx.x; ok && mine(i, item); ++i, item += gridDim.x) {
+      const WorkItem wi = work(i, item);
       const int T2 = wi.T2;
       const int qb = i & 1;
       if (i >= 2) ok = mbar_wait(bar(BAR_QFREE0 + qb), ((i >> 1) - 1) & 1, abortf);
@@ -148,8 +158,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     uint32_t g = 0;                                             // stages issued so far (all items)
     bool ok = true;
     int i = 0;
-    for (int item = blockIdx.x; ok && item < p.n_items; item += gridDim.x, ++i) {
-      const int T2 = decode_item<CAUSAL>(item, p, qtiles).T2;
+    for (int item = blockIdx.x; ok && mine(i, item); ++i, item += gridDim.x) {
+      const int T2 = work(i, item).T2;
       const int qb = i & 1;
       ok = mbar_wait(bar(BAR_QFULL0 + qb), (i >> 1) & 1, abortf);
       if (!ok) break;
@@ -207,8 +217,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     uint32_t g = 0;
     bool ok = true;
     int i = 0;
-    for (int item = blockIdx.x; ok && item < p.n_items; item += gridDim.x, ++i) {
-      const int T2 = decode_item<CAUSAL>(item, p, qtiles).T2;
+    for (int item = blockIdx.x; ok && mine(i, item); ++i, item += gridDim.x) {
+      const int T2 = work(i, item).T2;
       if (i >= 1) ok = mbar_wait(bar(BAR_OFREE), (i - 1) & 1, abortf);   // epilogue has read O
       for (int s2 = 0; ok && s2 < T2; ++s2, ++g) {
         const int pr = g & 1;
@@ -255,14 +265,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     const uint32_t tO = tmem + ((uint32_t)(quarter * 32) << 16) + kColO;
     uint32_t g0 = 0;                                            // stages completed in earlier items
     bool ok = true;
-    int i = 0;
     int T2 = 0;
     int mu_next = -(1 << 28);                                   // reference of the item whose first stage was served ahead
     bool first_served = false;
-    for (int item = blockIdx.x; ok && item < p.n_items; item += gridDim.x, ++i, g0 += T2) {
-      const WorkItem wi = decode_item<CAUSAL>(item, p, qtiles);
+    int i = 0;
+    for (int item = blockIdx.x; ok && mine(i, item); ++i, item += gridDim.x, g0 += T2) {
+      const WorkItem wi = work(i, item);
       T2 = wi.T2;
-      const bool has_next = item + (int)gridDim.x < p.n_items;
+      const bool has_next = mine(i + 1, item + (int)gridDim.x);
       int mu = FIXREF ? p.ref_fixed : (first_served ? mu_next : -(1 << 28));
       int runmax = first_served ? mu_next - kRefHeadroom : -(1 << 28);   // largest block exponent of the row so far
       // One pass per 128-key stage (both of its tiles).  The item's first stage may already have been served
@@ -418,11 +428,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     uint32_t g0 = 0;
     bool ok = true;
     int T2 = 0;
-    for (int item = blockIdx.x; ok && item < p.n_items; item += gridDim.x, g0 += T2) {
+    int i = 0;
+    for (int item = blockIdx.x; ok && mine(i, item); ++i, item += gridDim.x, g0 += T2) {
       uint32_t gdiag;                                           // global index of the item's masked stage, its last (none: ~0)
       int vis;                                                  // keys of that stage this row sees
       {
-        const WorkItem wi = decode_item<CAUSAL>(item, p, qtiles);
+        const WorkItem wi = work(i, item);
         T2 = wi.T2;
         gdiag = CAUSAL ? g0 + (uint32_t)(T2 - 1) : 0xFFFFFFFFu;
         // causal: keys 0..i of row i = qt * 128 + row; padded sequence: keys 0..len-1; both: the fewer
@@ -691,6 +702,8 @@ extern "C" int fp4attn_fwd(const fp4attn_operands* ops, int B, int H, int N, int
   prm.O = (__nv_bfloat16*)O; prm.LSE = LSE; prm.status = device_status;
   prm.N = N; prm.stages = N / BS; prm.n_items = B * H * (N / BM);
   prm.BH = B * H;
+  prm.B = B;
+  prm.sorted = ops->seq_len && B <= kSeqTableMax;
   prm.recip_qtiles = (N / BM) > 1 ? ~0ull / (unsigned long long)(N / BM) + 1 : 0;
   prm.recip_bh = prm.BH > 1 ? ~0ull / (unsigned long long)prm.BH + 1 : 0;
   prm.causal = ops->causal ? 1 : 0;

@@ -48,7 +48,8 @@ struct Cfg8 {
   static constexpr int OFF_STAGE = (OFF_MU + 2 * BM * 4 + 1023) / 1024 * 1024;
   static constexpr int OFF_OUT = OFF_STAGE + NST * STAGE_BYTES;
   static constexpr int OFF_BAR = OFF_OUT + C1::OUT_BYTES;
-  static constexpr int SMEM_BYTES = OFF_BAR + 1024 + 1024;
+  static constexpr int OFF_SEQ = OFF_BAR + 1024;                      // SeqTable
+  static constexpr int SMEM_BYTES = OFF_SEQ + 1536 + 1024;
   static_assert(OFF_STAGE % 1024 == 0 && OFF_OUT % 1024 == 0 && SMEM_BYTES <= 227 * 1024, "shared memory");
 };
 
@@ -126,10 +127,6 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int qtiles = p.N / BM;
-  // this CTA's work items are item(k) = blockIdx.x + k * gridDim.x, k = 0 .. n_my - 1
-  const int n_my = p.n_items > (int)blockIdx.x ? (p.n_items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-  auto item_of = [&](int k) { return (int)blockIdx.x + k * (int)gridDim.x; };
-
   if (threadIdx.x == 0) {
     for (int b = 0; b < 2; ++b) {
       mbar_init(bar(B8_QFULL0 + b), 1);
@@ -161,6 +158,12 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   tc_fence_after();
   wait_prior_grids();                                           // everything above is this block's own set-up
   const uint32_t tmem = *tslot;
+  SeqTable* const seq = reinterpret_cast<SeqTable*>(sgen + C8::OFF_SEQ);
+  if (CAUSAL && p.sorted) {
+    build_seq_table(seq, p, qtiles);
+    fill_skipped<D>(seq, p, qtiles);
+  }
+  const int n_my = items_of_cta<CAUSAL>(CAUSAL && p.sorted ? seq->first[p.B] : p.n_items);   // this CTA's items: item_at(0 .. n_my - 1)
 
   // Every role walks the same schedule.  Phase ph (0 .. n_my) carries the first sweep ("A": scores -> row maxima) of
   // item ph and the second sweep ("B": scores -> bytes -> PV) of item ph - 1, stage by stage, in the order
@@ -177,8 +180,8 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     for (int phs = 0; ok && phs <= n_my; ++phs) {
       WorkItem wa = {}, wb = {};
       int TA = 0, TB = 0;
-      if (phs < n_my) { wa = decode_item<CAUSAL>(item_of(phs), p, qtiles); TA = wa.T2; }
-      if (phs >= 1) { wb = decode_item<CAUSAL>(item_of(phs - 1), p, qtiles); TB = wb.T2; }
+      if (phs < n_my) { wa = decode_item<CAUSAL>(item_at<CAUSAL>(phs), p, qtiles, seq); TA = wa.T2; }
+      if (phs >= 1) { wb = decode_item<CAUSAL>(item_at<CAUSAL>(phs - 1), p, qtiles, seq); TB = wb.T2; }
       if (phs < n_my) {
         const int qb = phs & 1;
         if (phs >= 2) ok = mbar_wait(bar(B8_QFREE0 + qb), ((phs >> 1) - 1) & 1, abortf);
@@ -226,8 +229,8 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     bool ok = true;
     for (int phs = 0; ok && phs <= n_my; ++phs) {
       int TA = 0, TB = 0;
-      if (phs < n_my) TA = decode_item<CAUSAL>(item_of(phs), p, qtiles).T2;
-      if (phs >= 1) TB = decode_item<CAUSAL>(item_of(phs - 1), p, qtiles).T2;
+      if (phs < n_my) TA = decode_item<CAUSAL>(item_at<CAUSAL>(phs), p, qtiles, seq).T2;
+      if (phs >= 1) TB = decode_item<CAUSAL>(item_at<CAUSAL>(phs - 1), p, qtiles, seq).T2;
       if (phs < n_my) {
         const int qb = phs & 1;
         ok = mbar_wait(bar(B8_QFULL0 + qb), (phs >> 1) & 1, abortf);
@@ -290,8 +293,8 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     bool ok = true;
     for (int phs = 0; ok && phs <= n_my; ++phs) {
       int TA = 0, TB = 0;
-      if (phs < n_my) TA = decode_item<CAUSAL>(item_of(phs), p, qtiles).T2;
-      if (phs >= 1) TB = decode_item<CAUSAL>(item_of(phs - 1), p, qtiles).T2;
+      if (phs < n_my) TA = decode_item<CAUSAL>(item_at<CAUSAL>(phs), p, qtiles, seq).T2;
+      if (phs >= 1) TB = decode_item<CAUSAL>(item_at<CAUSAL>(phs - 1), p, qtiles, seq).T2;
       if (phs >= 2) ok = mbar_wait(bar(B8_OFREE), (phs - 2) & 1, abortf);   // epilogue of item phs - 2 has read O
       const int TM = TA > TB ? TA : TB;
       for (int s2 = 0; ok && s2 < TM; ++s2) {
@@ -330,7 +333,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const uint32_t tO = tmem + ((uint32_t)(quarter * 32) << 16) + kColO;
     bool ok = true;
     for (int k = 0; ok && k < n_my; ++k) {
-      const WorkItem wi = decode_item<CAUSAL>(item_of(k), p, qtiles);
+      const WorkItem wi = decode_item<CAUSAL>(item_at<CAUSAL>(k), p, qtiles, seq);
       ok = mbar_wait(bar(B8_OFULL), k & 1, abortf);
       if (!ok) break;
       tc_fence_after();
@@ -405,8 +408,8 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     for (int phs = 0; ok && phs <= n_my; ++phs) {
       WorkItem wa = {}, wb = {};
       int TA = 0, TB = 0;
-      if (phs < n_my) { wa = decode_item<CAUSAL>(item_of(phs), p, qtiles); TA = wa.T2; }
-      if (phs >= 1) { wb = decode_item<CAUSAL>(item_of(phs - 1), p, qtiles); TB = wb.T2; }
+      if (phs < n_my) { wa = decode_item<CAUSAL>(item_at<CAUSAL>(phs), p, qtiles, seq); TA = wa.T2; }
+      if (phs >= 1) { wb = decode_item<CAUSAL>(item_at<CAUSAL>(phs - 1), p, qtiles, seq); TB = wb.T2; }
       const int va = CAUSAL ? tile_keys(wa) : 64, vb = CAUSAL ? tile_keys(wb) : 64;
       float smax = -INFINITY;                                   // this team's share of the maxima of item phs
       const int TM = TA > TB ? TA : TB;

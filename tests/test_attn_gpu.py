@@ -526,6 +526,33 @@ def test_padded_sequences_full_length_is_bit_identical_and_padding_content_is_ir
     assert int(status.item()) == 0
 
 
+@pytest.mark.parametrize("B", [2, 64, 65])           # the work items are ordered by length for up to 64 entries
+@pytest.mark.parametrize("causal,d,H,kv_heads,fp8", [(False, 64, 3, 3, False), (True, 128, 4, 2, False), (True, 64, 2, 2, True),
+                                                     (False, 128, 2, 1, True)])
+def test_padded_batches_equal_their_entries_alone(B, causal, d, H, kv_heads, fp8):
+    """Which CTA takes which item must not show: every entry of a batch of unlike lengths (zero and too large counts among
+    them, clamped into 1..N) has the bits of a call on that entry alone, and nothing beyond a length is left unwritten."""
+    from paper_2609_04105_b200 import binding as Bd
+    w = I.shrink(I.WORKLOADS["cfg1"], B=B, H=H, N=640, d=d)
+    q, k, v = (_dev(t) for t in I.make_qkv(w))
+    k, v = k[:, :kv_heads].contiguous(), v[:, :kv_heads].contiguous()
+    lens = [0, 700] if B == 2 else [int(n) for n in np.random.default_rng(B).integers(1, 641, B)]
+
+    def run(q, k, v, lens):
+        out = torch.full_like(q, float("nan"))
+        lse = torch.full(q.shape[:3], float("nan"), device="cuda")
+        vq = Bd.fp4attn_quantize_v_e4m3(v) if fp8 else Bd.fp4attn_quantize(v, Bd.FMT_MXFP4, Bd.ROLE_V)
+        return Bd.fp4attn_fwd(Bd.fp4attn_quantize(q, 0, Bd.ROLE_Q), Bd.fp4attn_quantize(k, 0, Bd.ROLE_K), vq, out=out, lse=lse, causal=causal,
+                              seq_len=torch.tensor(lens, dtype=torch.int32, device="cuda"))
+
+    O, L = run(q, k, v, lens)
+    assert torch.isfinite(O.float()).all() and torch.isfinite(L).all()
+    for b, n in enumerate(lens):
+        n = min(max(n, 1), w.N)
+        O1, L1 = run(q[b:b + 1].contiguous(), k[b:b + 1].contiguous(), v[b:b + 1].contiguous(), [n])
+        assert torch.equal(O[b, :, :n], O1[0, :, :n]) and torch.equal(L[b, :, :n], L1[0, :, :n]), (b, n)
+
+
 def test_padded_sequences_reject_what_they_do_not_cover():
     from paper_2609_04105_b200 import binding as Bd
     w = I.shrink(I.WORKLOADS["cfg3"], B=2, H=2, N=512)
