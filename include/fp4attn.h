@@ -335,13 +335,12 @@ size_t fp4attn_attention_host_workspace_bytes(int qk_fmt, int B, int H, int N, i
  * pointer of at least fp4attn_attention_host_workspace_bytes() bytes, 256-byte aligned.  The caller
  * synchronises `stream` before reading O_host: everything the call enqueues has completed by then.
  *
- * With MXFP4 Q, K and at least 8 (batch, head) units the call is pipelined over groups of units (they
- * are independent and MXFP4 needs no tensor-wide pass): the copy in of one group, the kernels of the
- * previous one and the copy out of the one before overlap, so the path costs about its largest leg
- * instead of the sum.  The copies then run on two internal streams (created on the first such call per
- * device and kept until the process exits; no device memory is allocated) that fork from `stream` and
- * join back into it through events.  NVFP4 (tensor-wide amax first) and small problems run on `stream`
- * alone.  Results are bit-identical either way.
+ * From some megabytes of input on, the call is pipelined over groups of (batch, head) units, which are independent: the
+ * copy in of one group, the kernels of the one before and the copy out of an earlier one overlap, so the path costs about
+ * its largest leg instead of the sum.  With MXFP4 a group is its units' Q, K and V; with NVFP4 Q and K (tensor-wide amax) come
+ * in whole first and the groups are of V.  The copies then run on two internal streams (created on the first such call per
+ * device and kept until the process exits; no device memory is allocated) that fork from `stream` and join back into it
+ * through events.  Small problems run on `stream` alone.  Results are bit-identical either way.
  *
  * status_host (HOST pointer, preferably pinned; may be NULL): the call keeps a status word in its workspace,
  * clears it before its first kernel, hands it to every attention launch and copies it to *status_host at the

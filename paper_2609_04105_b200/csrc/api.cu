@@ -63,17 +63,19 @@ bool plan(int fmt, int B, int H, int N, int d, HostPlan* p) {
   return true;
 }
 
-// ---- MXFP4 host path, pipelined over groups of (batch, head) units.
-// (batch, head) units are independent and MXFP4 needs no tensor-wide pass, so the copy in of group c + 1, the
-// kernels of group c and the copy out of group c - 1 overlap: the path then costs about as much as its
-// largest leg (the host-to-device copy) instead of the sum of the three.  The copies run on two internal
-// streams (created on first use per device, kept until the process exits) that fork from and join back into
-// the caller's stream through events, so the caller still synchronises only its own stream.
+// ---- Host path, pipelined over groups of (batch, head) units.
+// Bound by the host link.  Units are independent, so the copy in of group c + 1, the kernels of group c and the copy out of
+// group c - 1 overlap: the path then costs about as much as its largest leg (the host-to-device copy) instead of the sum of
+// the three.  MXFP4 needs no tensor-wide pass, so a group is its heads' Q, K and V.  NVFP4 needs all of Q and of K before it can
+// code any of either: K and Q come in whole, each coded under the next copy, and the groups are of V (B=2, H=16, N=4096,
+// d=128: 2.65 -> 2.11 ms, the copies in alone 1.81).  The copies run on two internal streams (created on first use per
+// device, kept until the process exits) that fork from and join back into the caller's stream through events, so the caller
+// still synchronises only its own stream.
 constexpr int kNoPipeline = -1;
 constexpr int kMaxGroups = 16;
 struct HostPipe {
   cudaStream_t h2d = nullptr, d2h = nullptr;
-  cudaEvent_t start = nullptr, end = nullptr, in[kMaxGroups] = {}, done[kMaxGroups] = {};
+  cudaEvent_t start = nullptr, end = nullptr, whole[2] = {}, in[kMaxGroups] = {}, done[kMaxGroups] = {};   // whole: all of Q, of K
   bool ready = false;
 };
 void destroy(HostPipe& hp) {
@@ -81,6 +83,8 @@ void destroy(HostPipe& hp) {
   if (hp.d2h) cudaStreamDestroy(hp.d2h);
   if (hp.start) cudaEventDestroy(hp.start);
   if (hp.end) cudaEventDestroy(hp.end);
+  for (int i = 0; i < 2; ++i)
+    if (hp.whole[i]) cudaEventDestroy(hp.whole[i]);
   for (int c = 0; c < kMaxGroups; ++c) {
     if (hp.in[c]) cudaEventDestroy(hp.in[c]);
     if (hp.done[c]) cudaEventDestroy(hp.done[c]);
@@ -99,6 +103,7 @@ HostPipe* host_pipe() {
               cudaStreamCreateWithFlags(&hp.d2h, cudaStreamNonBlocking) == cudaSuccess &&
               cudaEventCreateWithFlags(&hp.start, cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&hp.end, cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 0; ok && i < 2; ++i) ok = cudaEventCreateWithFlags(&hp.whole[i], cudaEventDisableTiming) == cudaSuccess;
     for (int c = 0; ok && c < kMaxGroups; ++c)
       ok = cudaEventCreateWithFlags(&hp.in[c], cudaEventDisableTiming) == cudaSuccess &&
            cudaEventCreateWithFlags(&hp.done[c], cudaEventDisableTiming) == cudaSuccess;
@@ -110,65 +115,91 @@ HostPipe* host_pipe() {
 // First unit of group c when BH units are cut into `groups` groups whose sizes differ by at most one: the larger groups
 // come first, so that what runs after the last copy in (the last group's kernels and copy out) is as short as possible.
 inline int group_begin(int BH, int groups, int c) { return BH - (int)((long long)BH * (groups - c) / groups); }
-int enqueue_groups(HostPipe* hp, int groups, const void* q_host, const void* k_host, const void* v_host, float softmax_scale,
+int enqueue_groups(HostPipe* hp, int fmt, int groups, const void* q_host, const void* k_host, const void* v_host, float softmax_scale,
                    int BH, int N, int d, void* O_host, float* LSE_host, char* ws, const HostPlan& p, size_t workspace_bytes,
                    int* dev_status, cudaStream_t st) {
   const size_t head_elems = (size_t)N * d;
-  const size_t sfq_head = fp4attn_scale_bytes(FP4ATTN_FMT_MXFP4, FP4ATTN_ROLE_Q, 1, 1, N, d);
-  const size_t sfv_head = fp4attn_scale_bytes(FP4ATTN_FMT_MXFP4, FP4ATTN_ROLE_V, 1, 1, N, d);
+  const bool nv = fmt == FP4ATTN_FMT_NVFP4;
+  const size_t sf_head[3] = {fp4attn_scale_bytes(fmt, FP4ATTN_ROLE_Q, 1, 1, N, d), fp4attn_scale_bytes(fmt, FP4ATTN_ROLE_K, 1, 1, N, d),
+                             fp4attn_scale_bytes(FP4ATTN_FMT_MXFP4, FP4ATTN_ROLE_V, 1, 1, N, d)};
   const char* src[3] = {(const char*)q_host, (const char*)k_host, (const char*)v_host};
+  float* G = (float*)(ws + p.G);
 #define FP4ATTN_CUDA_OK(call) do { if ((call) != cudaSuccess) return FP4ATTN_ERR_CUDA; } while (0)
+  auto copy_in = [&](int i, int h0, int nh) {
+    return cudaMemcpyAsync(ws + p.x[i] + h0 * head_elems * 2, src[i] + h0 * head_elems * 2, nh * head_elems * 2, cudaMemcpyHostToDevice, hp->h2d);
+  };
+  auto quantize = [&](int i, int h0, int nh) {
+    return fp4attn_quantize(ws + p.x[i] + h0 * head_elems * 2, i < 2 ? fmt : FP4ATTN_FMT_MXFP4, i, 1, nh, N, d,
+                            ws + p.packed[i] + h0 * head_elems / 2, ws + p.sf[i] + h0 * sf_head[i], nv && i < 2 ? G + i : nullptr,
+                            ws + p.qws, workspace_bytes - p.qws, (fp4attn_stream_t)st);
+  };
+  if (nv) {
+    for (int i = 1; i >= 0; --i) {                                // K, then Q
+      FP4ATTN_CUDA_OK(copy_in(i, 0, BH));
+      FP4ATTN_CUDA_OK(cudaEventRecord(hp->whole[i], hp->h2d));
+    }
+  }
   for (int c = 0; c < groups; ++c) {
     const int h0 = group_begin(BH, groups, c), nh = group_begin(BH, groups, c + 1) - h0;
-    for (int i = 0; i < 3; ++i)
-      FP4ATTN_CUDA_OK(cudaMemcpyAsync(ws + p.x[i] + h0 * head_elems * 2, src[i] + h0 * head_elems * 2, nh * head_elems * 2,
-                                      cudaMemcpyHostToDevice, hp->h2d));
+    for (int i = nv ? 2 : 0; i < 3; ++i) FP4ATTN_CUDA_OK(copy_in(i, h0, nh));
     FP4ATTN_CUDA_OK(cudaEventRecord(hp->in[c], hp->h2d));
+  }
+  if (nv) {
+    for (int i = 1; i >= 0; --i) {
+      FP4ATTN_CUDA_OK(cudaStreamWaitEvent(st, hp->whole[i], 0));
+      const int rc = quantize(i, 0, BH);
+      if (rc != FP4ATTN_OK) return rc;
+    }
   }
   for (int c = 0; c < groups; ++c) {
     const int h0 = group_begin(BH, groups, c), nh = group_begin(BH, groups, c + 1) - h0;
     FP4ATTN_CUDA_OK(cudaStreamWaitEvent(st, hp->in[c], 0));
-    const size_t sf_head[3] = {sfq_head, sfq_head, sfv_head};
-    for (int i = 0; i < 3; ++i) {
-      const int rc = fp4attn_quantize(ws + p.x[i] + h0 * head_elems * 2, FP4ATTN_FMT_MXFP4, i, 1, nh, N, d,
-                                      ws + p.packed[i] + h0 * head_elems / 2, ws + p.sf[i] + h0 * sf_head[i], nullptr,
-                                      ws + p.qws, workspace_bytes - p.qws, (fp4attn_stream_t)st);
+    for (int i = nv ? 2 : 0; i < 3; ++i) {
+      const int rc = quantize(i, h0, nh);
       if (rc != FP4ATTN_OK) return rc;
     }
     fp4attn_operands ops = {};
     ops.q = ws + p.packed[0] + h0 * head_elems / 2; ops.k = ws + p.packed[1] + h0 * head_elems / 2;
     ops.v = ws + p.packed[2] + h0 * head_elems / 2;
-    ops.q_sf = ws + p.sf[0] + h0 * sfq_head; ops.k_sf = ws + p.sf[1] + h0 * sfq_head; ops.v_sf = ws + p.sf[2] + h0 * sfv_head;
-    ops.qk_fmt = FP4ATTN_FMT_MXFP4;
+    ops.q_sf = ws + p.sf[0] + h0 * sf_head[0]; ops.k_sf = ws + p.sf[1] + h0 * sf_head[1]; ops.v_sf = ws + p.sf[2] + h0 * sf_head[2];
+    ops.q_G = nv ? G : nullptr; ops.k_G = nv ? G + 1 : nullptr;
+    ops.qk_fmt = fmt;
     ops.softmax_scale = softmax_scale;
     const int rc = fp4attn_fwd(&ops, 1, nh, N, d, ws + p.O + h0 * head_elems * 2, (float*)(ws + p.LSE) + (size_t)h0 * N, dev_status,
                                (fp4attn_stream_t)st);
     if (rc != FP4ATTN_OK) return rc;
     FP4ATTN_CUDA_OK(cudaEventRecord(hp->done[c], st));
     FP4ATTN_CUDA_OK(cudaStreamWaitEvent(hp->d2h, hp->done[c], 0));
+    // A copy in that is followed by another one in its stream completes, for that one, only when copies out that overlap its
+    // end have completed too.  So a group's copy out starts together with a copy in, one group later than it could
+    // (B=2, H=16, N=4096, NVFP4, 8 groups: 2.27 -> 2.11 ms; MXFP4 2.40 -> 2.18).
+    if (c + 1 < groups) FP4ATTN_CUDA_OK(cudaStreamWaitEvent(hp->d2h, hp->in[c + 1], 0));
     FP4ATTN_CUDA_OK(cudaMemcpyAsync((char*)O_host + h0 * head_elems * 2, ws + p.O + h0 * head_elems * 2, nh * head_elems * 2,
                                     cudaMemcpyDeviceToHost, hp->d2h));
-    if (LSE_host)
-      FP4ATTN_CUDA_OK(cudaMemcpyAsync(LSE_host + (size_t)h0 * N, (float*)(ws + p.LSE) + (size_t)h0 * N, (size_t)nh * N * 4,
-                                      cudaMemcpyDeviceToHost, hp->d2h));
   }
+  // LSE in one copy (a small one per group took 26 us each among the others)
+  if (LSE_host)
+    FP4ATTN_CUDA_OK(cudaMemcpyAsync(LSE_host, ws + p.LSE, (size_t)BH * N * 4, cudaMemcpyDeviceToHost, hp->d2h));
 #undef FP4ATTN_CUDA_OK
   return FP4ATTN_OK;
 }
-int attention_host_pipelined(const void* q_host, const void* k_host, const void* v_host, float softmax_scale, int B, int H,
+// Groups of about 2 MB of an operand, up to 8, and of 8 MB beyond: the first copies in and the last kernels and copy out,
+// which nothing overlaps, against some 15 us per group.  Measured over 1 .. 16 groups (us): 32 MB an operand, NVFP4 1 / 4 / 8 /
+// 16 groups 2620 / 2202 / 2112 / 2179, MXFP4 2605 / 2239 / 2179 / 2293; 8 MB 723 / 633 / 633 / 635; 2 MB, NVFP4 1 / 2 / 4 groups
+// 209 / 192 / 199, MXFP4 204 / 206 / 235.
+int host_groups(int fmt, int BH, int N, int d) {
+  const long long bytes = 2ll * BH * N * d;                       // of one operand
+  if (bytes < (fmt == FP4ATTN_FMT_NVFP4 ? 1 << 20 : 4 << 20)) return 1;
+  long long groups = bytes >> 21;
+  if (groups > 8) groups = (bytes >> 23) > 8 ? bytes >> 23 : 8;
+  if (groups > kMaxGroups) groups = kMaxGroups;
+  if (groups < 2) groups = 2;
+  return groups < BH ? (int)groups : BH;
+}
+int attention_host_pipelined(int fmt, const void* q_host, const void* k_host, const void* v_host, float softmax_scale, int B, int H,
                              int N, int d, void* O_host, float* LSE_host, char* ws, const HostPlan& p,
                              size_t workspace_bytes, int* dev_status, cudaStream_t st) {
-  const int BH = B * H;
-  // Groups of heads: at least 4 (8 from 32 heads on), and about one per 32 MB of input, so that the first copy in and
-  // the last kernels and copy out - the parts nothing overlaps - stay small against the whole (measured at
-  // B=1, H=16, N=32768: 4 / 8 / 12 / 16 groups 9.31 / 8.74 / 8.28 / 8.62 ms, the copies alone 7.56 ms; at B=4, H=16,
-  // N=4096: 4.34 / 4.39 / 4.64 ms for 4 / 8 / 16)
-  int groups = BH < 8 ? 1 : (BH < 2 * kMaxGroups ? 4 : 8);
-  if (groups > 1) {
-    const long long by_bytes = (long long)(3ull * BH * N * d * 2 / (32ull << 20));
-    if (by_bytes > groups) groups = (int)(by_bytes < kMaxGroups ? by_bytes : kMaxGroups);
-    if (groups > BH) groups = BH;
-  }
+  const int BH = B * H, groups = host_groups(fmt, BH, N, d);
   if (groups == 1) return kNoPipeline;
   std::lock_guard<std::mutex> lock(g_pipe_mutex);
   HostPipe* hp = host_pipe();
@@ -176,7 +207,7 @@ int attention_host_pipelined(const void* q_host, const void* k_host, const void*
   if (cudaEventRecord(hp->start, st) != cudaSuccess ||         // fork: the copies start after the stream's earlier work
       cudaStreamWaitEvent(hp->h2d, hp->start, 0) != cudaSuccess || cudaStreamWaitEvent(hp->d2h, hp->start, 0) != cudaSuccess)
     return FP4ATTN_ERR_CUDA;
-  const int rc = enqueue_groups(hp, groups, q_host, k_host, v_host, softmax_scale, BH, N, d, O_host, LSE_host, ws, p,
+  const int rc = enqueue_groups(hp, fmt, groups, q_host, k_host, v_host, softmax_scale, BH, N, d, O_host, LSE_host, ws, p,
                                 workspace_bytes, dev_status, st);
   // join on every exit, also a failed one: whatever reached the internal streams stays ordered before the
   // caller's later work on its stream (which may reuse the workspace and the host buffers)
@@ -219,11 +250,9 @@ extern "C" int fp4attn_attention_host(const void* q_host, const void* k_host, co
   const size_t elems = (size_t)B * H * N * d;
   int* dev_status = host_status_word(ws, p);
   if (cudaMemsetAsync(dev_status, 0, sizeof(int), st) != cudaSuccess) return FP4ATTN_ERR_CUDA;
-  if (qk_fmt == FP4ATTN_FMT_MXFP4) {
-    const int rc = attention_host_pipelined(q_host, k_host, v_host, softmax_scale, B, H, N, d, O_host, LSE_host, ws, p,
-                                            workspace_bytes, dev_status, st);
-    if (rc != kNoPipeline) return finish_host_call(rc, dev_status, status_host, st);
-  }
+  const int rc_pipe = attention_host_pipelined(qk_fmt, q_host, k_host, v_host, softmax_scale, B, H, N, d, O_host, LSE_host, ws, p,
+                                               workspace_bytes, dev_status, st);
+  if (rc_pipe != kNoPipeline) return finish_host_call(rc_pipe, dev_status, status_host, st);
   const void* src[3] = {q_host, k_host, v_host};
   for (int i = 0; i < 3; ++i)
     if (cudaMemcpyAsync(ws + p.x[i], src[i], elems * 2, cudaMemcpyHostToDevice, st) != cudaSuccess)

@@ -174,6 +174,30 @@ def test_host_buffer_entry_point_matches_device_path(kw):
             Bd.fp4attn_release()                                # internal streams, events, tensor maps: made again on the next call
 
 
+@pytest.mark.parametrize("name,kw", [("cfg1", dict(H=17, N=1024)),                # 4.3 MB an operand: two groups, 9 and 8 units
+                                     ("cfg1", dict(B=2, H=3, N=8192)),            # six units in as many groups
+                                     ("cfg1", dict(H=1, N=16384)),                # one unit: nothing to overlap
+                                     ("cfg3", dict(B=1, H=8, N=1024)),            # NVFP4, 1 MB: the smallest that is pipelined
+                                     ("cfg3", dict(B=1, H=5, N=8192, d=128))])    # NVFP4, five units
+@pytest.mark.parametrize("pinned", [True, False])
+def test_host_buffer_groups_match_the_device_path(name, kw, pinned):
+    from paper_2609_04105_b200 import binding as Bd
+    w = I.shrink(I.WORKLOADS[name], **{"B": 1, **kw})
+    g = torch.Generator(device="cuda")
+    g.manual_seed(w.N)
+    x = [torch.randn((w.B, w.H, w.N, w.d), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3)]
+    ops = [Bd.fp4attn_quantize(x[0], w.qk_fmt, Bd.ROLE_Q), Bd.fp4attn_quantize(x[1], w.qk_fmt, Bd.ROLE_K), Bd.fp4attn_quantize(x[2], 0, Bd.ROLE_V)]
+    O, L = Bd.fp4attn_fwd(*ops)
+    host = [t.cpu().pin_memory() if pinned else t.cpu() for t in x]
+    ws = torch.empty(Bd.fp4attn_attention_host_workspace_bytes(w.qk_fmt, w.B, w.H, w.N, w.d), dtype=torch.uint8, device="cuda")
+    out, lse = torch.zeros(O.shape, dtype=O.dtype, pin_memory=pinned), torch.zeros(L.shape, pin_memory=pinned)
+    for rep in range(2):
+        out.zero_()
+        Bd.fp4attn_attention_host(*host, w.qk_fmt, out, lse if rep == 0 else None, ws)
+        torch.cuda.synchronize()
+        assert torch.equal(out, O.cpu()) and torch.equal(lse, L.cpu())
+
+
 def test_host_buffer_entry_point_from_two_threads():
     """Two host threads, each with its own stream, workspace and host buffers, enqueue the pipelined host
     path at the same time (the library's internal copy streams and events are shared and guarded by a
