@@ -9,6 +9,8 @@
 
 #include <ATen/ATen.h>
 #include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDACachingAllocator.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 
 #include "../../include/fp4attn.h"
@@ -46,6 +48,48 @@ fp4attn_stream_t stream() { return reinterpret_cast<fp4attn_stream_t>(c10::cuda:
 at::Tensor device_empty(at::IntArrayRef size, at::ScalarType type, c10::Device device) {
   return at::Tensor(at::detail::empty_cuda(size, type, device, std::nullopt));
 }
+// The results of one call.  An allocation costs about as much host time as the rest of a call's marshalling, so up to
+// kShareBytes they are pieces of one (a step of B=1, H=2, N=256: 19.9 -> 17.0 us); beyond that (where the kernels take longer anyway) each has memory of its own, so that
+// keeping one alone does not keep them all.
+struct Results {
+  static constexpr size_t kShareBytes = 1 << 20, kMost = 4;
+  struct Piece {
+    int64_t sizes[4];
+    int dims;
+    at::ScalarType type;
+    at::Tensor tensor;
+  } piece[kMost];
+  int n = 0;
+  at::Tensor& add(std::initializer_list<int64_t> sizes, at::ScalarType type) {
+    Piece& p = piece[n++];
+    p.dims = (int)sizes.size();
+    p.type = type;
+    std::copy(sizes.begin(), sizes.end(), p.sizes);
+    return p.tensor;
+  }
+  void allocate(c10::Device device) {
+    int64_t at[kMost + 1] = {0}, count[kMost];
+    for (int i = 0; i < n; ++i) {
+      count[i] = 1;
+      for (int k = 0; k < piece[i].dims; ++k) count[i] *= piece[i].sizes[k];
+      at[i + 1] = at[i] + ((count[i] * (int64_t)c10::elementSize(piece[i].type) + 511) & ~511ll);   // as the allocator aligns
+    }
+    if (at[n] > (int64_t)kShareBytes) {
+      for (int i = 0; i < n; ++i) piece[i].tensor = device_empty(at::IntArrayRef(piece[i].sizes, piece[i].dims), piece[i].type, device);
+      return;
+    }
+    // straight from the caching allocator: a tensor of its own for the block would only be taken apart again
+    const c10::cuda::OptionalCUDAGuard guard(device);
+    c10::Allocator* const pool = c10::cuda::CUDACachingAllocator::get();
+    const c10::Storage block(c10::Storage::use_byte_size_t(), (size_t)at[n], pool->allocate((size_t)at[n]), pool, /*resizable=*/true);
+    for (int i = 0; i < n; ++i) {
+      piece[i].tensor = at::detail::make_tensor<c10::TensorImpl>(c10::Storage(block), c10::DispatchKeySet(c10::DispatchKey::CUDA), c10::scalarTypeToTypeMeta(piece[i].type));
+      c10::TensorImpl* impl = piece[i].tensor.unsafeGetTensorImpl();
+      impl->set_sizes_contiguous(at::IntArrayRef(piece[i].sizes, piece[i].dims));
+      impl->set_storage_offset(at[i] / (int64_t)c10::elementSize(piece[i].type));
+    }
+  }
+};
 void* data_of(PyObject* o) {                            // None: a null pointer
   return THPVariable_Check(o) ? THPVariable_Unpack(o).data_ptr() : nullptr;
 }
@@ -138,17 +182,14 @@ PyObject* py_quantize(PyObject*, PyObject* const* args, Py_ssize_t n) {
     PyErr_SetString(g_error, "fp4attn_quantize: unsupported arguments");
     return nullptr;
   }
-  const c10::Device dev = in.t->device();
-  at::Tensor packed = device_empty({(int64_t)nb}, at::kByte, dev), scales = device_empty({(int64_t)ns}, at::kByte, dev), G, ws;
-  if (fmt == FP4ATTN_FMT_NVFP4) G = device_empty({1}, at::kFloat, dev);
-  void* wptr = data_of(args[3]);
-  size_t wbytes = wptr ? (size_t)THPVariable_Unpack(args[3]).numel() : 0;
-  const size_t nw = g_api.quantize_workspace_bytes(fmt, role, in.B, in.H, in.N, in.d);
-  if (nw && args[3] == Py_None) {
-    ws = device_empty({(int64_t)nw}, at::kByte, dev);
-    wptr = ws.data_ptr();
-    wbytes = nw;
-  }
+  const size_t nw = args[3] == Py_None ? g_api.quantize_workspace_bytes(fmt, role, in.B, in.H, in.N, in.d) : 0;
+  Results r;
+  at::Tensor none, &packed = r.add({(int64_t)nb}, at::kByte), &scales = r.add({(int64_t)ns}, at::kByte);
+  at::Tensor& G = fmt == FP4ATTN_FMT_NVFP4 ? r.add({1}, at::kFloat) : none;
+  at::Tensor& ws = nw ? r.add({(int64_t)nw}, at::kByte) : none;
+  r.allocate(in.t->device());
+  void* const wptr = nw ? ws.data_ptr() : data_of(args[3]);
+  const size_t wbytes = nw ? nw : wptr ? (size_t)THPVariable_Unpack(args[3]).numel() : 0;
   const int rc = unlocked([&] { return g_api.quantize(in.t->data_ptr(), fmt, role, in.B, in.H, in.N, in.d, packed.data_ptr(), scales.data_ptr(),
                                 G.defined() ? G.data_ptr<float>() : nullptr, wptr, wbytes, stream()); });
   if (rc) return fail(rc, "fp4attn_quantize");
@@ -171,8 +212,9 @@ PyObject* py_rule(PyObject*, PyObject* const* args, Py_ssize_t n) {
     PyErr_SetString(g_error, "fp4attn_quantize_mxfp4_rule: unsupported arguments");
     return nullptr;
   }
-  const c10::Device dev = in.t->device();
-  at::Tensor packed = device_empty({(int64_t)nb}, at::kByte, dev), scales = device_empty({(int64_t)ns}, at::kByte, dev);
+  Results r;
+  at::Tensor &packed = r.add({(int64_t)nb}, at::kByte), &scales = r.add({(int64_t)ns}, at::kByte);
+  r.allocate(in.t->device());
   const int rc = unlocked([&] { return g_api.quantize_mxfp4_rule(in.t->data_ptr(), a[0], a[1], in.B, in.H, in.N, in.d, packed.data_ptr(), scales.data_ptr(), stream()); });
   if (rc) return fail(rc, "fp4attn_quantize_mxfp4_rule");
   return result(packed, &scales, nullptr, in);
@@ -195,9 +237,10 @@ PyObject* py_per_head(PyObject*, PyObject* const* args, Py_ssize_t n) {
     PyErr_SetString(g_error, "fp4attn_quantize_nvfp4_per_head: unsupported arguments");
     return nullptr;
   }
-  const c10::Device dev = in.t->device();
-  at::Tensor packed = device_empty({(int64_t)nb}, at::kByte, dev), scales = device_empty({(int64_t)ns}, at::kByte, dev);
-  at::Tensor G = device_empty({(int64_t)in.B * in.H}, at::kFloat, dev), ws = device_empty({(int64_t)nw}, at::kByte, dev);
+  Results r;
+  at::Tensor &packed = r.add({(int64_t)nb}, at::kByte), &scales = r.add({(int64_t)ns}, at::kByte);
+  at::Tensor &G = r.add({(int64_t)in.B * in.H}, at::kFloat), &ws = r.add({(int64_t)nw}, at::kByte);
+  r.allocate(in.t->device());
   const int rc = unlocked([&] { return g_api.per_head(in.t->data_ptr(), role, in.B, in.H, in.N, in.d, packed.data_ptr(), scales.data_ptr(), G.data_ptr<float>(),
                                 ws.data_ptr(), nw, stream()); });
   if (rc) return fail(rc, "fp4attn_quantize_nvfp4_per_head");
@@ -218,9 +261,10 @@ PyObject* py_e4m3(PyObject*, PyObject* const* args, Py_ssize_t n) {
     PyErr_SetString(g_error, "fp4attn_quantize_v_e4m3: unsupported arguments");
     return nullptr;
   }
-  const c10::Device dev = in.t->device();
-  at::Tensor out = device_empty({in.t->numel()}, at::kByte, dev), scales = device_empty({0}, at::kByte, dev);
-  at::Tensor G = device_empty({(int64_t)in.B * in.H}, at::kFloat, dev), ws = device_empty({(int64_t)nw}, at::kByte, dev);
+  Results r;
+  at::Tensor &out = r.add({in.t->numel()}, at::kByte), &scales = r.add({0}, at::kByte);
+  at::Tensor &G = r.add({(int64_t)in.B * in.H}, at::kFloat), &ws = r.add({(int64_t)nw}, at::kByte);
+  r.allocate(in.t->device());
   const int rc = unlocked([&] { return g_api.e4m3(in.t->data_ptr(), in.B, in.H, in.N, in.d, out.data_ptr(), G.data_ptr<float>(), ws.data_ptr(), nw, stream()); });
   if (rc) return fail(rc, "fp4attn_quantize_v_e4m3");
   return result(out, &scales, &G, in);
@@ -304,8 +348,13 @@ PyObject* py_fwd(PyObject*, PyObject* const* args, Py_ssize_t n) {
     if (!ints(args + 15, 1, &ops.fixed_reference)) return nullptr;
   }
   PyObject *out = Py_NewRef(args[4]), *lse = Py_NewRef(args[5]);
-  if (out == Py_None) Py_SETREF(out, THPVariable_Wrap(device_empty({B, H, N, d}, at::kBFloat16, q.device)));
-  if (lse == Py_None) Py_SETREF(lse, THPVariable_Wrap(device_empty({B, H, N}, at::kFloat, q.device)));
+  if (out == Py_None || lse == Py_None) {
+    Results r;
+    at::Tensor none, &o = out == Py_None ? r.add({B, H, N, d}, at::kBFloat16) : none, &l = lse == Py_None ? r.add({B, H, N}, at::kFloat) : none;
+    r.allocate(q.device);
+    if (out == Py_None) Py_SETREF(out, THPVariable_Wrap(o));
+    if (lse == Py_None) Py_SETREF(lse, THPVariable_Wrap(l));
+  }
   int rc = -1;
   if (out && lse) {
     void *o = data_of(out), *l = data_of(lse), *st = data_of(args[6]);
