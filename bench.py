@@ -333,7 +333,7 @@ def run_cuda(args, w):
     status = torch.zeros(1, dtype=torch.int32, device=dev)
     qws = torch.empty(max(16, Bd.lib().fp4attn_quantize_workspace_bytes(w.qk_fmt, 0, B, H, N, d)), dtype=torch.uint8, device=dev)
     flush = torch.empty(256 * 1024 * 1024, dtype=torch.uint8, device=dev)      # > 126 MB L2
-    launches_per_step = 4 if w.qk_fmt == I.FMT_MXFP4 else 8          # NVFP4: amax pass + encode factor + codes, for Q and for K
+    launches_per_step = 4 if w.qk_fmt == I.FMT_MXFP4 else 6          # NVFP4: amax pass + codes, for Q and for K
     pmap = Bd.PMAP_AFFINE if args.p_map == "affine" else Bd.PMAP_HYBRID if args.p_map in HYBRID_PATTERNS else Bd.PMAP_IDEAL
     pairs = HYBRID_PATTERNS.get(args.p_map, 0)
     pscale = {"thr16": Bd.PSCALE_THR16, "mse": Bd.PSCALE_MSE}.get(args.p_scale, Bd.PSCALE_CEIL)

@@ -42,7 +42,7 @@ struct Cfg {
   static constexpr int OFF_KSF = K_BYTES + V_BYTES + ONES_BYTES;   // within a stage
   static constexpr int OFF_VSF = OFF_KSF + KSF_BYTES;
   static constexpr int STAGE_BYTES = OFF_VSF + VSF_BYTES;
-  static constexpr int NST = (D == 128) ? 7 : 8;                // ring depth (stages of 128 keys)
+  static constexpr int NST = 8;                                 // ring depth (stages of 128 keys); at d = 128 the affine map takes 1-2 % longer with 7, the same with 9
   static constexpr int PSF_BYTES = 512;                         // one atom per stage: bytes {0,1} tile 0, {2,3} tile 1
   static constexpr int META_BYTES = BM * 16;                    // per stage parity and row: {E_0, E_1} of tile 0, of tile 1
   // shared-memory map (offsets from a 1024-byte aligned base)

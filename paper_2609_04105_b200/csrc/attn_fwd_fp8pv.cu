@@ -40,7 +40,7 @@ struct Cfg8 {
   static constexpr int ONES_BYTES = kOnesRows * BS;                   // rows of E4M3 1.0
   static constexpr int OFF_KSF = C1::K_BYTES + V_BYTES + ONES_BYTES;  // within a stage
   static constexpr int STAGE_BYTES = (OFF_KSF + C1::KSF_BYTES + 1023) / 1024 * 1024;
-  static constexpr int NST = (D == 128) ? 5 : 8;
+  static constexpr int NST = (D == 128) ? 5 : 8;                      // d = 128, N = 8192: 3 / 4 / 5 / 6 slots 1177 / 923 / 752 / 742 us, causal (6) 4 % longer
   static constexpr int OFF_Q = 0;                                     // two buffers
   static constexpr int OFF_QSF = OFF_Q + 2 * C1::Q_BYTES;             // two buffers of 1 KB
   static constexpr int OFF_RMAX = OFF_QSF + 2048;                     // [item parity][first-sweep team][row] float
@@ -83,22 +83,18 @@ __device__ __forceinline__ uint32_t cvt_e4m3x4_pos(float a, float b, float c, fl
   return w;
 }
 
-// 32 scores of one row -> 32 E4M3 bytes (8 words) against the row's final reference: x = fma(s, c, 8 - mu)
-template <bool MASKED>
-__device__ __forceinline__ void fp8_p_block(const uint32_t* sraw, float c32, float b, int visible, uint32_t* words) {
+// 32 scores of one row -> 32 E4M3 bytes (8 words) against the row's final reference: x = fma(s, c, 8 - mu), c2 = {c, c}
+__device__ __forceinline__ void fp8_p_block(const uint32_t* sraw, uint64_t c2, float b, uint32_t* words) {
+  const uint64_t bb = pack2(b, b);
 #pragma unroll
   for (int w = 0; w < 8; ++w) {
     float pv[4];
 #pragma unroll
     for (int i = 0; i < 4; i += 2) {
       float x0, x1;
-      fma2(__uint_as_float(sraw[4 * w + i]), __uint_as_float(sraw[4 * w + i + 1]), c32, b, x0, x1);
+      unpack2(fma2(pack2(__uint_as_float(sraw[4 * w + i]), __uint_as_float(sraw[4 * w + i + 1])), c2, bb), x0, x1);
       pv[i] = ex2_approx(x0);
       pv[i + 1] = ex2_approx(x1);
-      if (MASKED) {
-        if (4 * w + i >= visible) pv[i] = 0.f;
-        if (4 * w + i + 1 >= visible) pv[i + 1] = 0.f;
-      }
     }
     words[w] = cvt_e4m3x4_pos(pv[0], pv[1], pv[2], pv[3]);
   }
@@ -392,9 +388,12 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const uint32_t sfull = bar(B8_SFULL0 + pr), sempty = bar(B8_SEMPTY0 + pr);
     const uint32_t smdone = bar(B8_SMDONE0 + pr), pfree = bar(B8_PFREE0 + pr);
     const uint32_t tP = tmem + ((uint32_t)(quarter * 32) << 16) + k8ColP + 32 * pr + 16 * h;
-    float c32;
-    if (NV) c32 = __fdiv_rn(p.c_base, __fmul_rn(__ldcg(p.q_G), __ldcg(p.k_G)));
-    else    c32 = __fdiv_rn(p.c_base, 36.0f);
+    uint64_t c2 = p.c_mx2;                                      // MXFP4: a kernel parameter, read from uniform registers
+    if (NV) {
+      const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldcg(p.q_G), __ldcg(p.k_G)));
+      c2 = pack2(c, c);
+    }
+    const float c32 = __uint_as_float((uint32_t)c2);
     bool ok = true;
     uint32_t g = 0;                                             // steps so far (both kinds, all pairs)
     uint32_t nbt = 0;                                           // B-visits of this team so far
@@ -428,20 +427,14 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             const bool diag = CAUSAL && s2 == TA - 1;
             tmem_ld_32x32b_x32(tS, sraw);
             tmem_wait_ld();
-            if (diag) {
-#pragma unroll
-              for (int e = 0; e < 32; ++e) sraw[e] = (e < va) ? sraw[e] : 0xFF800000u;
-            }
+            if (diag) mask_scores(sraw, va);
             smax = fmaxf(smax, max32(sraw));
             tmem_ld_32x32b_x32(tS + 32, sraw);
             tmem_wait_ld();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(sempty);
-            if (diag) {
-#pragma unroll
-              for (int e = 0; e < 32; ++e) sraw[e] = (e < va - 32) ? sraw[e] : 0xFF800000u;
-            }
+            if (diag) mask_scores(sraw, va - 32);
             smax = fmaxf(smax, max32(sraw));
           } else {
             // ---- second sweep of item phs - 1: bytes against its final reference
@@ -449,15 +442,15 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             const bool diag = CAUSAL && s2 == TB - 1;
             tmem_ld_32x32b_x32(tS, sraw);
             tmem_wait_ld();
-            if (diag) fp8_p_block<true>(sraw, c32, b, vb, w);
-            else      fp8_p_block<false>(sraw, c32, b, 32, w);
+            if (diag) mask_scores(sraw, vb);
+            fp8_p_block(sraw, c2, b, w);
             tmem_ld_32x32b_x32(tS + 32, sraw);
             tmem_wait_ld();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(sempty);
-            if (diag) fp8_p_block<true>(sraw, c32, b, vb - 32, w + 8);
-            else      fp8_p_block<false>(sraw, c32, b, 32, w + 8);
+            if (diag) mask_scores(sraw, vb - 32);
+            fp8_p_block(sraw, c2, b, w + 8);
             // the pair's probability slot was last read by the PV product of this team's previous B-visit
             if (nbt > 0) ok = mbar_wait(pfree, (nbt - 1) & 1, abortf);
             if (!ok) break;
