@@ -257,6 +257,38 @@ quant_mx_v_kernel(const uint4* __restrict__ x, uint4* __restrict__ packed, uint8
   }
 }
 
+// ---- a unit's maximum within one thread-block cluster: every CTA reduces its share, the shares meet through distributed
+// shared memory.  The second barrier (cluster_leave) keeps a CTA's share readable until every other CTA has read it.
+__device__ __forceinline__ uint32_t cluster_size() { uint32_t n; asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n)); return n; }
+__device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm("mov.u32 %0, %%cluster_ctaid.x;" : "=r"(r)); return r; }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// `m`: each thread's maximum; all threads of all CTAs of the cluster; THREADS threads per CTA
+template <int THREADS>
+__device__ __forceinline__ uint32_t cluster_max(uint32_t m) {
+  __shared__ uint32_t wmax[THREADS / 32], share;
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    m = __reduce_max_sync(0xffffffffu, threadIdx.x < THREADS / 32 ? wmax[threadIdx.x] : 0u);
+    if (threadIdx.x == 0) share = m;
+  }
+  cluster_arrive();
+  cluster_wait();
+  const uint32_t lane = threadIdx.x & 31;
+  m = 0;
+  if (lane < cluster_size()) {
+    uint32_t remote;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"((uint32_t)__cvta_generic_to_shared(&share)), "r"(lane));
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(m) : "r"(remote) : "memory");
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  cluster_arrive();
+  return m;
+}
+__device__ __forceinline__ void cluster_leave() { cluster_wait(); }
+
 // Encode factor of a tensor or unit from its partial maxima: fl32(top / max), 1 for an all-zero one.  Each kernel that needs
 // the factor takes it so (at most 1024 partials, in L2) instead of waiting for a kernel of its own to form it.
 // encode_factor_warp: every warp by itself, at most 32 partials; encode_factor_block: the whole block, with a barrier.
@@ -398,6 +430,36 @@ __device__ __forceinline__ float e4m3_byte_to_f32(uint32_t b) {
   return __half2float(__ushort_as_half((unsigned short)(h2 & 0xFFFFu)));
 }
 
+// one chunk's codes and scale bytes from its bf16 words
+template <int D>
+__device__ __forceinline__ void nv_code_chunk(const uint32_t (&raw)[kLoads][8], float G, uint32_t chunk, uint2* packed, uint8_t* sf) {
+  constexpr uint32_t LPR = D / 16;                 // lanes per row
+  constexpr uint32_t CT = (D / 16 + 3) / 4;
+  const uint32_t seg = threadIdx.x % LPR;
+#pragma unroll
+  for (int k = 0; k < kLoads; ++k) {
+    const float a = __uint_as_float(absmax_bf16x16(raw[k]) << 16);
+    const float t = __fdiv_rn(__fmul_rn(a, G), 6.0f);
+    uint32_t sb = cvt_e4m3_byte(t);
+    const float S = e4m3_byte_to_f32(sb);
+    const float r = (S > 0.f) ? __fdiv_rn(G, S) : 0.f;
+    uint32_t w[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float v[8];
+      bf16x8_to_f32(make_uint4(raw[k][4 * h], raw[k][4 * h + 1], raw[k][4 * h + 2], raw[k][4 * h + 3]), v);
+      scale_values<8>(v, r);                                     // sign rides along; 0*r = 0 for zero blocks
+      w[h] = cvt_e2m1x8(v);
+    }
+    packed[(size_t)chunk * (kGroupsPerCta / 2) + threadIdx.x + k * kThreads] = make_uint2(w[0], w[1]);
+    sb |= __shfl_xor_sync(0xffffffffu, sb, 1) << 8;              // four columns' bytes as one word
+    sb |= __shfl_xor_sync(0xffffffffu, sb, 2) << 16;
+    const uint32_t row = chunk * (kGroupsPerCta / 2 / LPR) + (threadIdx.x + k * kThreads) / LPR;
+    if ((seg & 3) == 0)
+      *reinterpret_cast<uint32_t*>(sf + ((size_t)(row >> 7) * CT + (seg >> 2)) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4) = sb;
+  }
+}
+
 // ---------------------------------------------------------------- NVFP4 pass 2, blocks of 16 along d (Q, K)
 // Bound by HBM (twice over the tensor, less what is left of it in L2) and by the two IEEE divisions per block.  67 M elements,
 // both passes: 50.6 us; with a kernel of its own for the factor, a block's scale formed in two lanes and plain launches 61.6.
@@ -408,11 +470,8 @@ __global__ void __launch_bounds__(kThreads, kRowsCtas)
 quant_nv_rows_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, uint8_t* __restrict__ sf,
                      const float* __restrict__ partials, int n_partials, float* __restrict__ G_out, uint32_t n_chunks,
                      uint32_t chunks_per_unit) {
-  constexpr uint32_t LPR = D / 16;
-  constexpr uint32_t CT = (D / 16 + 3) / 4;
   launch_dependents();
   wait_prior_grids();
-  const uint32_t seg = threadIdx.x % LPR;
   uint32_t i = blockIdx.x, raw[kLoads][8];
 #pragma unroll
   for (int k = 0; k < kLoads; ++k) load_16<W32>(raw[k], x + (size_t)(n_chunks - 1 - i) * kGroupsPerCta + 2 * (threadIdx.x + k * kThreads));
@@ -434,34 +493,59 @@ quant_nv_rows_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, ui
       G = encode_factor_warp(partials + (size_t)unit * n_partials, n_partials, 2688.0f);
       if (threadIdx.x == 0 && unit * chunks_per_unit == chunk) G_out[unit] = G;
     }
-#pragma unroll
-    for (int k = 0; k < kLoads; ++k) {
-      const float a = __uint_as_float(absmax_bf16x16(raw[k]) << 16);
-      const float t = __fdiv_rn(__fmul_rn(a, G), 6.0f);
-      uint32_t sb = cvt_e4m3_byte(t);
-      const float S = e4m3_byte_to_f32(sb);
-      const float r = (S > 0.f) ? __fdiv_rn(G, S) : 0.f;
-      uint32_t w[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        float v[8];
-        bf16x8_to_f32(make_uint4(raw[k][4 * h], raw[k][4 * h + 1], raw[k][4 * h + 2], raw[k][4 * h + 3]), v);
-        scale_values<8>(v, r);                                     // sign rides along; 0*r = 0 for zero blocks
-        w[h] = cvt_e2m1x8(v);
-      }
-      packed[(size_t)chunk * (kGroupsPerCta / 2) + threadIdx.x + k * kThreads] = make_uint2(w[0], w[1]);
-      sb |= __shfl_xor_sync(0xffffffffu, sb, 1) << 8;              // four columns' bytes as one word
-      sb |= __shfl_xor_sync(0xffffffffu, sb, 2) << 16;
-      const uint32_t row = chunk * (kGroupsPerCta / 2 / LPR) + (threadIdx.x + k * kThreads) / LPR;
-      if ((seg & 3) == 0)
-        *reinterpret_cast<uint32_t*>(sf + ((size_t)(row >> 7) * CT + (seg >> 2)) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4) = sb;
-    }
+    nv_code_chunk<D>(raw, G, chunk, packed, sf);
     if (i >= n_chunks) return;
 #pragma unroll
     for (int k = 0; k < kLoads; ++k)
 #pragma unroll
       for (int j = 0; j < 8; ++j) raw[k][j] = ahead[k][j];
   }
+}
+
+// Both passes over a unit with a factor of its own in one launch: a cluster takes the unit, its CTAs every cluster_size()-th
+// chunk.  The second pass, from the last chunk back, finds the unit in L2 (a device's worth of clusters holds some tens of
+// megabytes), so the tensor is read from memory once.
+template <int D, bool W32>
+__global__ void __launch_bounds__(kThreads, kRowsCtas)
+quant_nv_unit_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, uint8_t* __restrict__ sf, float* __restrict__ G_out,
+                     int chunks_per_unit) {
+  launch_dependents();
+  wait_prior_grids();
+  const int step = (int)cluster_size(), unit = blockIdx.x / step, first = unit * chunks_per_unit, rank = (int)cluster_rank();
+  uint32_t raw[kLoads][8], m = 0;
+  const int mine = (chunks_per_unit - rank + step - 1) / step;    // chunks first + rank, first + rank + step, ...
+  auto load = [&](int k_chunk, uint32_t (&r)[kLoads][8]) {
+    const uint4* src = x + (size_t)(first + rank + k_chunk * step) * kGroupsPerCta;
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k) load_16<W32>(r[k], src + 2 * (threadIdx.x + k * kThreads));
+  };
+  if (mine > 0) load(0, raw);
+  for (int c = 0; c < mine; ++c) {
+    uint32_t ahead[kLoads][8];
+    if (c + 1 < mine) load(c + 1, ahead);
+#pragma unroll
+    for (int k = 0; k < kLoads; ++k) m = max(m, absmax_bf16x16(raw[k]));
+    if (c + 1 < mine) {
+#pragma unroll
+      for (int k = 0; k < kLoads; ++k)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) raw[k][j] = ahead[k][j];
+    }
+  }
+  const float G = encode_factor_of(__uint_as_float(cluster_max<kThreads>(m) << 16), 2688.0f);
+  if (rank == 0 && threadIdx.x == 0) G_out[unit] = G;
+  for (int c = mine - 1; c >= 0; --c) {                           // the last chunk is still in registers
+    uint32_t ahead[kLoads][8];
+    if (c > 0) load(c - 1, ahead);
+    nv_code_chunk<D>(raw, G, (uint32_t)(first + rank + c * step), packed, sf);
+    if (c > 0) {
+#pragma unroll
+      for (int k = 0; k < kLoads; ++k)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) raw[k][j] = ahead[k][j];
+    }
+  }
+  cluster_leave();
 }
 
 }  // namespace fp4attn
@@ -516,18 +600,24 @@ static void launch_mx_v(const uint4* xs, int n_tiles, int N, void* packed, void*
                     (uint8_t*)scales, N, n_tiles);
 }
 
+static int device_sms() {                          // 0 if the runtime does not tell
+  static std::atomic<int> sm_count[kMaxDevices];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+  int sms = sm_count[dev].load(std::memory_order_acquire);
+  if (!sms) {
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return 0;
+    sm_count[dev].store(sms, std::memory_order_release);
+  }
+  return sms;
+}
+
 // Persistent CTAs of the rows kernels: at most what the device holds at once, each with the same number of chunks (within
 // one).  One CTA per chunk would pay a CTA's start - its launch, the wait for the kernels before, the encode factor - every
 // 16 KB.
 static unsigned rows_grid(size_t n_chunks) {
-  static std::atomic<int> sm_count[kMaxDevices];
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return (unsigned)n_chunks;
-  sms = sm_count[dev].load(std::memory_order_acquire);
-  if (!sms) {
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return (unsigned)n_chunks;
-    sm_count[dev].store(sms, std::memory_order_release);
-  }
+  const int sms = device_sms();
+  if (!sms) return (unsigned)n_chunks;
   const size_t resident = (size_t)kRowsCtas * sms, rounds = (n_chunks + resident - 1) / resident;
   return (unsigned)((n_chunks + rounds - 1) / rounds);
 }
@@ -548,6 +638,17 @@ static void launch_mx(const uint4* xs, int role, int B, int H, int N, int d, voi
   }
 }
 
+// CTAs of the cluster that takes a unit of so many chunks: up to eight (the portable limit)
+static unsigned cluster_for(size_t chunks) { return chunks >= 8 ? 8 : chunks >= 4 ? 4 : chunks >= 2 ? 2 : 1; }
+// One launch for both passes where the clusters fill the device about twice, so that some read while others write, or where
+// every CTA has at most two chunks and the second launch costs more than it brings.  Microseconds back to back, two launches
+// against one: 64 units of 64 chunks 28.8 / 24.6, 128 of 64 53.2 / 44.8, 328 of 4 13.0 / 11.5, 2 of 16 4.1 / 3.7, 2 of 4 4.0 /
+// 3.0; beyond the line 16 units of 64 chunks 10.6 / 15.2, 1 of 32 4.2 / 5.1.
+static bool nv_in_one_launch(size_t units, size_t chunks) {
+  const unsigned cluster = cluster_for(chunks);
+  return chunks <= 2 * cluster || units * cluster >= (size_t)2 * device_sms();
+}
+
 int launch_quantize(const void* x, int fmt, int role, int B, int H, int N, int d, void* packed, void* scales,
                     float* G_out, float* partials, cudaStream_t st, int mx_rule, bool per_head = false) {
   const size_t n_groups = (size_t)B * H * N * d / 8;
@@ -559,6 +660,15 @@ int launch_quantize(const void* x, int fmt, int role, int B, int H, int N, int d
     else if (mx_rule == FP4ATTN_QSCALE_MSE)   launch_mx<FP4ATTN_QSCALE_MSE>(xs, role, B, H, N, d, packed, scales, st);
     else                                      launch_mx<FP4ATTN_QSCALE_CEIL>(xs, role, B, H, N, d, packed, scales, st);
   } else {
+    const size_t units = per_head ? (size_t)B * H : 1, per_unit = per_head ? unit_chunks : n_chunks;
+    if (nv_in_one_launch(units, per_unit)) {
+      const bool w32u = ((uintptr_t)xs & 31) == 0;
+      const unsigned cluster = cluster_for(per_unit);
+      launch_overlapped_clusters(d == 128 ? (w32u ? quant_nv_unit_kernel<128, true> : quant_nv_unit_kernel<128, false>)
+                                 : (w32u ? quant_nv_unit_kernel<64, true> : quant_nv_unit_kernel<64, false>),
+                        dim3((unsigned)units * cluster), kThreads, 0, st, cluster, xs, (uint2*)packed, (uint8_t*)scales, G_out, (int)per_unit);
+      return cudaGetLastError() == cudaSuccess ? FP4ATTN_OK : FP4ATTN_ERR_CUDA;
+    }
     const unsigned most = per_head ? (unsigned)kPartialsPerHead : (unsigned)kMaxPartials;
     const size_t want = per_head ? unit_chunks : n_chunks;
     const int n_partials = (int)(want < most ? want : most);

@@ -220,6 +220,30 @@ def test_quantizers_at_chunk_edges_and_alignments(B, H, N, d, offset):
     assert np.array_equal(e.G.cpu().numpy().reshape(B, H), want["G"])
 
 
+@pytest.mark.parametrize("B,H,N,d", [(1, 1, 256, 64),        # a cluster of two, one chunk each
+                                     (3, 1, 896, 64),        # seven chunks a unit: a cluster of four, two or one chunk each
+                                     (1, 2, 1152, 128),      # eighteen: just too many for one launch
+                                     (2, 20, 640, 128),      # forty units fill the device: ten chunks over eight CTAs
+                                     (5, 9, 1536, 64)])      # twelve
+@pytest.mark.parametrize("offset", [0, 8])
+def test_nvfp4_one_launch_and_two_launch_sizes(B, H, N, d, offset):
+    """Units (and small tensors) that one cluster quantizes by itself, and sizes just beyond: bytes and factors of the oracle;
+    one unit is zero, magnitudes differ between units."""
+    from paper_2609_04105_b200 import binding as Bd
+    w = I.shrink(I.WORKLOADS["cfg3"], B=B, H=H, N=N, d=d)
+    x = Qz.bf16_bits_to_f64(I.make_qkv(w)[0]) * 2.0 ** np.random.default_rng(N).integers(-20, 10, size=(B, H, 1, 1))
+    x[B - 1, H - 1] *= 0.0 if B * H > 1 else 1.0
+    bits = I.f32_to_bf16_bits(x.astype(np.float32))
+    buf = torch.empty(bits.size + offset, dtype=torch.bfloat16, device="cuda")
+    t = buf[offset:].view(B, H, N, d)
+    t.copy_(_dev(bits))
+    got, want = Bd.fp4attn_quantize_nvfp4_per_head(t, Bd.ROLE_Q), Qz.quantize_qk(bits, "nv", per_head=True)
+    G = want.pop("G")
+    _check_operand(got, {**want, "G": None}, Bd.ROLE_Q)
+    assert np.array_equal(got.G.cpu().numpy(), G.reshape(-1))
+    _check_operand(Bd.fp4attn_quantize(t, Bd.FMT_NVFP4, Bd.ROLE_K), Qz.quantize_qk(bits, "nv"), Bd.ROLE_K)
+
+
 def test_nvfp4_per_head_rejects_v_and_missing_workspace():
     from paper_2609_04105_b200 import binding as Bd
     x = torch.zeros((1, 2, 128, 64), dtype=torch.bfloat16, device="cuda")
