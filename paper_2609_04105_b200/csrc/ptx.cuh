@@ -48,8 +48,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // read, a look at the abort flag and a warp vote around it all 967 | 750 us; bare polls with the hint 923 | 687 us; without
 // it 903 | 619 us; four polls per trip of the counter 916 | 620 us.  All lanes of a warp poll the same barrier in the same
 // instruction, so they leave together without a vote.
-// Limit: 2^22 polls of about 80 clocks, a good tenth of a second (a poll may be suspended for longer, never for less).
-constexpr uint32_t kWaitPolls = 1u << 22;
+// Limit: 2^25 polls, at some 80 clocks each more than a second of SM clocks (a poll may be suspended for longer, never for
+// less).  The longest wait of a healthy kernel lasts as long as one work item (the producer's, for a Q buffer).
+constexpr uint32_t kWaitPolls = 1u << 25;
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   uint32_t ok;
   asm volatile(
