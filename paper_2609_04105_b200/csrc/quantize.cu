@@ -158,6 +158,8 @@ quant_mx_rows_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, ui
 // four scale bytes meet by lane exchange; 16-byte chunk c of a tile row sits at c ^ 2 (key block), which keeps the reads of
 // the four blocks in different banks.  (One warp per key block, with half-sector stores and the scale bytes meeting in shared
 // memory: 29.5 us for 67 M elements at d = 128; this way 29.0.)
+// Registers are not capped: at 102 a thread two CTAs fit an SM and take 27.6 us (d = 64: 27.7); capped to 80, three with 29.1
+// (30.5); three tile buffers 29.3, four 27.0 (31.0).
 // Persistent CTAs walk the tiles with two tile buffers: the asynchronous copies (cp.async, 16 bytes per thread
 // and copy, no registers in between) of the next tile are in flight while the current one is converted, so the
 // memory system always has work although each tile passes through a load -> barrier -> convert sequence.
@@ -172,7 +174,7 @@ template <int PENDING>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
 
 template <int D, int RULE>
-__global__ void __launch_bounds__(2 * D, RULE == FP4ATTN_QSCALE_MSE ? 1 : (D == 128 ? 3 : 6))
+__global__ void __launch_bounds__(2 * D, 1)
 quant_mx_v_kernel(const uint4* __restrict__ x, uint4* __restrict__ packed, uint8_t* __restrict__ sf, int N, int n_tiles) {
   constexpr int T = 2 * D;                         // threads: D/2 column pairs x 4 key blocks
   constexpr int LOADS = 128 * D / 8 / T;           // 16-byte copies per thread and tile: 8
