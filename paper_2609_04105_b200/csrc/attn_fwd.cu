@@ -50,6 +50,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* sgen = smem_raw + (sbase - smem_u32(smem_raw));
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sgen + C::OFF_BAR + 768);
+  const uint32_t abort_at = sbase + C::OFF_BAR + 776;
   volatile int* abortf = reinterpret_cast<volatile int*>(sgen + C::OFF_BAR + 776);
   auto bar = [&](int i) { return sbase + C::OFF_BAR + 8u * i; };
   auto bar_full = [&](int s) { return bar(BAR_RING + s); };
@@ -118,7 +119,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       const WorkItem wi = work(i, item);
       const int T2 = wi.T2;
       const int qb = i & 1;
-      if (i >= 2) ok = mbar_wait(bar(BAR_QFREE0 + qb), ((i >> 1) - 1) & 1, abortf);
+      if (i >= 2) ok = mbar_wait(bar(BAR_QFREE0 + qb), ((i >> 1) - 1) & 1, abort_at);
       if (!ok) break;
       if (elect_one()) {
         mbar_arrive_expect_tx(bar(BAR_QFULL0 + qb), C::Q_BYTES + C::QSF_BYTES);
@@ -129,7 +130,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       const uint8_t* vsf = p.v_sf + (size_t)wi.kvh * qtiles * C::VSF_BYTES;
       const int krow0 = wi.kvh * p.N, vrow0 = wi.kvh * D;
       for (int s2 = 0; s2 < T2; ++s2) {
-        if (!mbar_wait(bar_empty(s), ph ^ 1, abortf)) { ok = false; break; }   // (a fresh barrier passes)
+        if (!mbar_wait(bar_empty(s), ph ^ 1, abort_at)) { ok = false; break; }   // (a fresh barrier passes)
         const uint32_t fb = bar_full(s);
         if (elect_one()) {
           mbar_arrive_expect_tx(fb, C::K_BYTES + C::V_BYTES + C::KSF_BYTES + C::VSF_BYTES);
@@ -161,7 +162,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     for (int item = blockIdx.x; ok && mine(i, item); ++i, item += gridDim.x) {
       const int T2 = work(i, item).T2;
       const int qb = i & 1;
-      ok = mbar_wait(bar(BAR_QFULL0 + qb), (i >> 1) & 1, abortf);
+      ok = mbar_wait(bar(BAR_QFULL0 + qb), (i >> 1) & 1, abort_at);
       if (!ok) break;
       tc_fence_after();
       const uint32_t tSFQ = tmem + kColSFQ + 8 * qb;
@@ -173,8 +174,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       for (int s2 = 0; s2 < T2; ++s2, ++g) {
         const int pr = g & 1;
         const uint32_t m = g >> 1;
-        ok = mbar_wait(bar_full(sq), phq, abortf);
-        if (ok) ok = mbar_wait(bar(BAR_SEMPTY0 + pr), (m & 1) ^ 1, abortf);   // both teams have read the pair (a fresh barrier passes)
+        ok = mbar_wait(bar_full(sq), phq, abort_at);
+        if (ok) ok = mbar_wait(bar(BAR_SEMPTY0 + pr), (m & 1) ^ 1, abort_at);   // both teams have read the pair (a fresh barrier passes)
         if (!ok) break;
         tc_fence_after();
         const uint32_t tSFK = tmem + kColSFK + 8 * pr;
@@ -219,13 +220,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     int i = 0;
     for (int item = blockIdx.x; ok && mine(i, item); ++i, item += gridDim.x) {
       const int T2 = work(i, item).T2;
-      if (i >= 1) ok = mbar_wait(bar(BAR_OFREE), (i - 1) & 1, abortf);   // epilogue has read O
+      if (i >= 1) ok = mbar_wait(bar(BAR_OFREE), (i - 1) & 1, abort_at);   // epilogue has read O
       for (int s2 = 0; ok && s2 < T2; ++s2, ++g) {
         const int pr = g & 1;
         const uint32_t m = g >> 1;
         // codes of both tiles are in tensor memory, their scale bytes in shared memory (written by the correction
         // warps, or with a fixed reference by the teams themselves)
-        ok = mbar_wait(bar((FIXREF ? BAR_SMDONE0 : BAR_PFULL0) + pr), m & 1, abortf);
+        ok = mbar_wait(bar((FIXREF ? BAR_SMDONE0 : BAR_PFULL0) + pr), m & 1, abort_at);
         if (!ok) break;
         tc_fence_after();
         const uint32_t tSFP = tmem + kColSFP + 4 * pr, tSFV = tmem + kColSFV + 8 * pr;
@@ -280,7 +281,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       for (uint32_t g = FIXREF ? g0 + (uint32_t)T2 : g0 + (first_served ? 1u : 0u); g < g0 + (uint32_t)T2; ++g) {
         const bool first_of_item = g == g0;
         const int pr = g & 1;
-        ok = mbar_wait(bar(BAR_SMDONE0 + pr), (g >> 1) & 1, abortf);
+        ok = mbar_wait(bar(BAR_SMDONE0 + pr), (g >> 1) & 1, abort_at);
         if (!ok) break;
         const int4 me = *reinterpret_cast<const int4*>(sgen + C::OFF_META + C::META_BYTES * pr + row * 16);
         const int Emax = max(max(me.x, me.y), max(me.z, me.w));
@@ -302,7 +303,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             // O holds the item's earlier stages once their PV has landed (an item's first stage never
             // touches O: it may still belong to the previous item)
             const uint32_t gprev = g - 1;
-            ok = mbar_wait(bar(BAR_PFREE0 + (gprev & 1)), (gprev >> 1) & 1, abortf);
+            ok = mbar_wait(bar(BAR_PFREE0 + (gprev & 1)), (gprev >> 1) & 1, abort_at);
             if (!ok) break;
             tc_fence_after();
 #pragma unroll 1
@@ -330,7 +331,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       if (!ok) break;
       first_served = false;
       // ---- epilogue: with L_hw = column d of the accumulator, O = O_hw / (6 L_hw), LSE = ln2 (mu + log2(L_hw / 6))
-      ok = mbar_wait(bar(BAR_OFULL), i & 1, abortf);
+      ok = mbar_wait(bar(BAR_OFULL), i & 1, abort_at);
       if (!ok) break;
       tc_fence_after();
       float Lhw;
@@ -386,7 +387,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // sequences either way and serves the stage in its own loop, after the epilogue.)
         const uint32_t g = g0 + (uint32_t)T2;
         const int pr = g & 1;
-        ok = mbar_wait(bar(BAR_SMDONE0 + pr), (g >> 1) & 1, abortf);
+        ok = mbar_wait(bar(BAR_SMDONE0 + pr), (g >> 1) & 1, abort_at);
         if (!ok) break;
         const int4 me = *reinterpret_cast<const int4*>(sgen + C::OFF_META + C::META_BYTES * pr + row * 16);
         mu_next = max(max(me.x, me.y), max(me.z, me.w)) + kRefHeadroom;
@@ -447,7 +448,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       }
       for (uint32_t g = g0 + ((g0 & 1) != (uint32_t)pr); g < g0 + T2; g += 2) {   // this team's stages of the item
         const uint32_t par = (g >> 1) & 1;
-        if (!mbar_wait(sfull, par, abortf)) { ok = false; break; }
+        if (!mbar_wait(sfull, par, abort_at)) { ok = false; break; }
         tc_fence_after();
         uint32_t sraw[32], pw[8];
         int E0, E1;
@@ -463,7 +464,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if (lane == 0) mbar_arrive(sempty);                     // pair may take the stage after next
         if (CAUSAL && g == gdiag) mask_scores(sraw, vis - 64 * (team & 1) - 32);
         direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E1, pw + 4);
-        if (!mbar_wait(pfree, par ^ 1, abortf)) { ok = false; break; }   // PV of the pair's previous stage is done (a fresh barrier passes)
+        if (!mbar_wait(pfree, par ^ 1, abort_at)) { ok = false; break; }   // PV of the pair's previous stage is done (a fresh barrier passes)
         // fixed reference: E8M0 bytes of the two blocks against the constant; below the range a zero block (no codes,
         // so that a row without any live block shows as a zero row sum), above it an error
         const int b0 = FIXREF ? E0 - p.ref_fixed + 127 : 0, b1 = FIXREF ? E1 - p.ref_fixed + 127 : 0;
@@ -511,6 +512,7 @@ __global__ void __launch_bounds__(128, 1) mma_peak_kernel(int iters, unsigned lo
   // A: 128 rows x 32 B, B: 128 rows x 32 B (one K64 slice each), scale atoms 2 x 512 B, all zero
   for (int i = threadIdx.x; i < (4096 + 4096 + 1024) / 4; i += 128) reinterpret_cast<uint32_t*>(sgen)[i] = 0;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sgen + 9216 + 64);
+  const uint32_t abort_at = sbase + 9216 + 72;
   volatile int* abortf = reinterpret_cast<volatile int*>(sgen + 9216 + 72);
   if (threadIdx.x == 0) { mbar_init(sbase + 9216, 1); *abortf = 0; fence_barrier_init(); }
   fence_proxy_async_smem();
@@ -527,7 +529,7 @@ __global__ void __launch_bounds__(128, 1) mma_peak_kernel(int iters, unsigned lo
     const long long t0 = clock64();
     for (int i = 0; i < iters; ++i) tc_mma_fp4_2x(tmem + 128 * (i & 1), ad, bd, idesc, tmem + 480, tmem + 484, 1);
     tc_commit(sbase + 9216);
-    const bool ok = mbar_wait(sbase + 9216, 0, abortf);
+    const bool ok = mbar_wait(sbase + 9216, 0, abort_at);
     const long long t1 = clock64();
     if (ok) atomicMax(cycles_out, (unsigned long long)(t1 - t0));
   }
@@ -537,15 +539,17 @@ __global__ void __launch_bounds__(128, 1) mma_peak_kernel(int iters, unsigned lo
 }
 
 // ------------------------------------------------------------------ bounded-wait self-test
-// One warp waits on an mbarrier that nothing will ever complete, with a short limit, and must come
-// back through the same time-out path the attention kernel uses (abort flag -> status word).
-__global__ void __launch_bounds__(32, 1) bounded_wait_selftest_kernel(long long limit_cycles, int* status) {
+// One warp waits twice on an mbarrier that nothing will ever complete, in the attention kernels' own mbar_wait with a short
+// limit, and must come back through their time-out path (abort word -> status word), from the second wait at its first look.
+__global__ void __launch_bounds__(32, 1) bounded_wait_selftest_kernel(uint32_t limit_cycles, int* status) {
   __shared__ __align__(8) uint64_t never;
-  __shared__ int abort_flag;
-  if (threadIdx.x == 0) { mbar_init(smem_u32(&never), 1); abort_flag = 0; fence_barrier_init(); }
+  __shared__ int abort_word;
+  if (threadIdx.x == 0) { mbar_init(smem_u32(&never), 1); abort_word = 0; fence_barrier_init(); }
   __syncwarp();
-  const bool ok = __all_sync(0xffffffffu, mbar_wait_limit(smem_u32(&never), 0, &abort_flag, limit_cycles));
-  if (threadIdx.x == 0) *status = (!ok && abort_flag) ? FP4ATTN_ERR_TIMEOUT : FP4ATTN_OK;
+  bool ok = false;
+  for (int i = 0; i < 2; ++i) ok |= mbar_wait(smem_u32(&never), 0, smem_u32(&abort_word), limit_cycles);
+  ok = __any_sync(0xffffffffu, ok);
+  if (threadIdx.x == 0) *status = (!ok && *(volatile int*)&abort_word) ? FP4ATTN_ERR_TIMEOUT : FP4ATTN_OK;
 }
 
 // ------------------------------------------------------------------ host side
@@ -826,6 +830,6 @@ extern "C" int fp4attn_selftest_bounded_wait(long long limit_cycles, int* device
   if (!device_status || limit_cycles <= 0 || limit_cycles > (1ll << 31)) return FP4ATTN_ERR_INVALID_ARG;
   int rc = check_device_sm100();
   if (rc != FP4ATTN_OK) return rc;
-  bounded_wait_selftest_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(limit_cycles, device_status);
+  bounded_wait_selftest_kernel<<<1, 32, 0, (cudaStream_t)stream>>>((uint32_t)limit_cycles, device_status);
   return cudaGetLastError() == cudaSuccess ? FP4ATTN_OK : FP4ATTN_ERR_CUDA;
 }

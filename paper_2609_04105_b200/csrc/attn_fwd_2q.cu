@@ -76,6 +76,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* sgen = smem_raw + (sbase - smem_u32(smem_raw));
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sgen + C2::OFF_BAR + 768);
+  const uint32_t abort_at = sbase + C2::OFF_BAR + 776;
   volatile int* abortf = reinterpret_cast<volatile int*>(sgen + C2::OFF_BAR + 776);
   auto bar = [&](int i) { return sbase + C2::OFF_BAR + 8u * i; };
   auto bar_full = [&](int s) { return bar(B2_RING + s); };
@@ -131,7 +132,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     for (int item = blockIdx.x; ok && item < p.n_items; item += gridDim.x, ++i) {
       const WorkItem2 wi = decode_item2(item, p, pairs);
       const int ib = i & 1;
-      if (i >= 2) ok = mbar_wait(bar(B2_QFREE0 + ib), ((i >> 1) - 1) & 1, abortf);
+      if (i >= 2) ok = mbar_wait(bar(B2_QFREE0 + ib), ((i >> 1) - 1) & 1, abort_at);
       if (!ok) break;
       if (elect_one()) {
         mbar_arrive_expect_tx(bar(B2_QFULL0 + ib), 2 * (C::Q_BYTES + C::QSF_BYTES));
@@ -146,7 +147,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       const uint8_t* vsf = p.v_sf + (size_t)wi.kvh * T2 * C::VSF_BYTES;
       const int krow0 = wi.kvh * p.N, vrow0 = wi.kvh * D;
       for (int s2 = 0; s2 < T2; ++s2, ++gs) {
-        if (gs >= (uint32_t)C::NST) ok = mbar_wait(bar_empty(s), ph ^ 1, abortf);
+        if (gs >= (uint32_t)C::NST) ok = mbar_wait(bar_empty(s), ph ^ 1, abort_at);
         if (!ok) break;
         const uint32_t fb = bar_full(s);
         if (elect_one()) {
@@ -175,7 +176,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     int i = 0;
     for (int item = blockIdx.x; ok && item < p.n_items; item += gridDim.x, ++i) {
       const int ib = i & 1;
-      ok = mbar_wait(bar(B2_QFULL0 + ib), (i >> 1) & 1, abortf);
+      ok = mbar_wait(bar(B2_QFULL0 + ib), (i >> 1) & 1, abort_at);
       if (!ok) break;
       tc_fence_after();
       if (elect_one()) {
@@ -184,7 +185,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           tc_cp_32x128b_warpx4(tmem + k2ColSFQ + 4 * (2 * ib + q), at(kDescSF, sbase + C2::OFF_QSF + (2 * ib + q) * 1024));
       }
       for (int s2 = 0; s2 < T2; ++s2, ++ms) {
-        ok = mbar_wait(bar_full(sq), phq, abortf);
+        ok = mbar_wait(bar_full(sq), phq, abort_at);
         if (!ok) break;
         tc_fence_after();
         const uint32_t tSFK = tmem + k2ColSFK + 4 * (ms & 1);
@@ -192,7 +193,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         if (elect_one()) tc_cp_32x128b_warpx4(tSFK, at(kDescSF, stq + C::OFF_KSF));
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-          if (ms > 0) ok = mbar_wait(bar(B2_SEMPTY0 + q), (ms - 1) & 1, abortf);   // both teams of the query have read S_q
+          if (ms > 0) ok = mbar_wait(bar(B2_SEMPTY0 + q), (ms - 1) & 1, abort_at);   // both teams of the query have read S_q
           if (!ok) break;
           tc_fence_after();
           if (elect_one()) {
@@ -226,8 +227,8 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         const uint64_t dV = at(kDescV, stp + C::K_BYTES);
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-          if (s2 == 0 && i >= 1) ok = mbar_wait(bar(B2_OFREE0 + q), (i - 1) & 1, abortf);   // epilogue has read O_q
-          if (ok) ok = mbar_wait(bar(B2_PFULL0 + q), ms & 1, abortf);
+          if (s2 == 0 && i >= 1) ok = mbar_wait(bar(B2_OFREE0 + q), (i - 1) & 1, abort_at);   // epilogue has read O_q
+          if (ok) ok = mbar_wait(bar(B2_PFULL0 + q), ms & 1, abort_at);
           if (!ok) break;
           tc_fence_after();
           if (q == 0) {
@@ -268,7 +269,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       for (uint32_t ms = ms0; ok && ms < ms0 + (uint32_t)T2; ++ms) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-          ok = mbar_wait(bar(B2_SMDONE0 + q), ms & 1, abortf);
+          ok = mbar_wait(bar(B2_SMDONE0 + q), ms & 1, abort_at);
           if (!ok) break;
           const int4 me = *reinterpret_cast<const int4*>(sgen + C2::OFF_META + C::META_BYTES * q + row * 16);
           const int Emax = max(max(me.x, me.y), max(me.z, me.w));
@@ -281,7 +282,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             const float f = (delta > 126) ? 0.f : __uint_as_float((uint32_t)(127 - delta) << 23);
             mu[q] = (delta > 126) ? runmax[q] + kRefHeadroom : mu[q] + delta;
             if (ms != ms0) {
-              ok = mbar_wait(bar(B2_PFREE0 + q), (ms - 1) & 1, abortf);   // PV of the previous stage has landed
+              ok = mbar_wait(bar(B2_PFREE0 + q), (ms - 1) & 1, abort_at);   // PV of the previous stage has landed
               if (!ok) break;
               tc_fence_after();
 #pragma unroll 1
@@ -309,7 +310,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
       // ---- epilogue, query 0 then query 1: O = O_hw / (6 L_hw), LSE = ln2 (mu + log2(L_hw / 6))
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        ok = mbar_wait(bar(B2_OFULL0 + q), i & 1, abortf);
+        ok = mbar_wait(bar(B2_OFULL0 + q), i & 1, abort_at);
         if (!ok) break;
         tc_fence_after();
         const uint32_t tO = tObase + k2OCols * q;
@@ -376,7 +377,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     uint32_t ms = 0;
     for (int item = blockIdx.x; ok && item < p.n_items; item += gridDim.x) {
       for (int s2 = 0; s2 < T2; ++s2, ++ms) {
-        ok = mbar_wait(sfull, ms & 1, abortf);
+        ok = mbar_wait(sfull, ms & 1, abort_at);
         if (!ok) break;
         tc_fence_after();
         uint32_t sraw[32], w0[4], w1[4];
@@ -390,7 +391,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         __syncwarp();
         if (lane == 0) mbar_arrive(sempty);                     // S_q may take the next stage
         direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E1, w1);
-        if (ms > 0) ok = mbar_wait(pfree, (ms - 1) & 1, abortf);   // PV of the query's previous stage is done
+        if (ms > 0) ok = mbar_wait(pfree, (ms - 1) & 1, abort_at);   // PV of the query's previous stage is done
         if (!ok) break;
         {
           const uint32_t pw[8] = {w0[0], w0[1], w0[2], w0[3], w1[0], w1[1], w1[2], w1[3]};

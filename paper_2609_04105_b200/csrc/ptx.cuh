@@ -39,43 +39,42 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
-// Bounded waits.  `abort_flag` (shared memory) tells the end of the kernel that some wait ran out; every role that waits
-// for one that has left runs out in turn, so the CTA falls out together.
+// Bounded waits.  The word at `abort_at` (shared memory) tells the end of the kernel that some wait ran out, and every other
+// wait of the CTA, so that its roles fall out together.
 //
-// mbar_wait is a bare poll loop: the instruction's own (short, hardware-chosen) suspension, a counter, nothing else.  The
+// A wait is a bare poll loop: the instruction's own (short, hardware-chosen) suspension, a counter, nothing else.  The
 // waiting warps share their schedulers with the softmax warps, whose time is instruction dispatch, so what a wait executes
 // is taken from them.  Attention at B=4, H=16, N=8192, d=128 (exact | affine map): a poll with a suspend-time hint, a clock
 // read, a look at the abort flag and a warp vote around it all 967 | 750 us; bare polls with the hint 923 | 687 us; without
 // it 903 | 619 us; four polls per trip of the counter 916 | 620 us.  All lanes of a warp poll the same barrier in the same
 // instruction, so they leave together without a vote.
-// Limit: 2^25 polls, at some 80 clocks each more than a second of SM clocks (a poll may be suspended for longer, never for
-// less).  The longest wait of a healthy kernel lasts as long as one work item (the producer's, for a Q buffer).
-constexpr uint32_t kWaitPolls = 1u << 25;
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+// How long the hardware suspends a poll is its own choice (measured on a barrier that nothing completes: 4 us), so a count of
+// polls bounds no time: every kPolls polls the wait looks at the abort word and the clock.  Both loops are one piece of assembly and the word goes by its shared-memory
+// address: the same as C++ statements after the poll loop, with a generic pointer, spilled up to 32 bytes a thread and
+// took 3-6 % longer.
+constexpr uint32_t kPolls = 1u << 6;           // a look every 0.25 ms
+constexpr uint32_t kWaitClocks = 1u << 31;     // SM clocks, about a second; the longest wait of a healthy kernel lasts as long as one work item
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, uint32_t abort_at, uint32_t limit) {
   uint32_t ok;
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\t.reg .u32 n;\n\t"
-      "mov.u32 n, %3;\n"
+      "{\n\t.reg .pred p, q;\n\t.reg .u32 n, v, t;\n\t"
+      "mov.u32 n, 0;\n"
       "MBAR_POLL:\n\t"
       "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
       "@p bra MBAR_DONE;\n\t"
-      "sub.u32 n, n, 1;\n\tsetp.ne.u32 q, n, 0;\n\t@q bra MBAR_POLL;\n"
+      "add.u32 n, n, 1;\n\tand.b32 v, n, %5;\n\tsetp.ne.u32 q, v, 0;\n\t@q bra MBAR_POLL;\n\t"
+      "ld.volatile.shared.u32 v, [%3];\n\tsetp.ne.u32 q, v, 0;\n\t@q bra MBAR_DONE;\n\t"
+      "mov.u32 v, %%clock;\n\tsetp.eq.u32 q, n, %6;\n\t@q mov.u32 t, v;\n\t"                  // t: the first look
+      "sub.u32 v, v, t;\n\tsetp.lt.u32 q, v, %4;\n\t@q bra MBAR_POLL;\n"
       "MBAR_DONE:\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity), "n"(kWaitPolls) : "memory");
-  if (!ok) *abort_flag = 1;
+      : "=r"(ok) : "r"(bar), "r"(parity), "r"(abort_at), "r"(limit), "n"(kPolls - 1), "n"(kPolls) : "memory");
   return ok != 0;
 }
-// The same with a limit in SM clocks, for the self-test of the time-out path.
-__device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long limit) {
-  const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
-    if (clock64() - t0 > limit) {
-      *abort_flag = 1;
-      return false;
-    }
-  }
-  return true;
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t abort_at, uint32_t limit = kWaitClocks) {
+  if (mbar_poll(bar, parity, abort_at, limit)) return true;
+  asm volatile("st.volatile.shared.u32 [%0], 1;" ::"r"(abort_at) : "memory");
+  return false;
 }
 
 __device__ __forceinline__ void fence_barrier_init() {

@@ -288,6 +288,22 @@ def test_bounded_wait_times_out_and_reports_status():
         Bd.fp4attn_selftest_bounded_wait(0, status)
 
 
+@pytest.mark.parametrize("limit", [1, 1 << 28])
+def test_bounded_wait_limit_is_a_time_and_ends_the_other_waits(limit):
+    """Two waits in the kernels' own wait code: the first lasts its limit in SM clocks (2 GHz at most), the second ends with
+    it.  A look at the clock comes every 64 polls, each suspended for some 4 us: under a millisecond."""
+    from paper_2609_04105_b200 import binding as Bd
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    Bd.fp4attn_selftest_bounded_wait(1, status)
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    a.record()
+    Bd.fp4attn_selftest_bounded_wait(limit, status)
+    b.record()
+    torch.cuda.synchronize()
+    assert int(status.item()) == Bd.ERR_TIMEOUT
+    assert limit / 2.1e6 < a.elapsed_time(b) < 1.5 * limit / 1.2e6 + 20      # milliseconds; 1.2 GHz: far below any clock under this load
+
+
 def test_softmax_arithmetic_probe_respects_the_special_function_unit():
     """The probe runs the kernel's score -> code arithmetic alone.  With exact codes 24 of a block's 32 elements per
     row take ex2.approx, at 16 per clock and SM = 8 clocks per warp instruction and scheduler: no less than 192
