@@ -391,9 +391,10 @@ int fp4attn_softmax_arith_probe(int p_map, int exact_pairs, int iters, unsigned 
 
 /*
  * Self-test of the bounded in-kernel waits (the failure-detection path; the paper has no
- * counterpart).  Launches one warp that waits on a barrier nothing completes, in the very code the
- * attention kernels wait with, with a limit of `limit_cycles` SM clocks (1 .. 2^31; theirs is 2^31,
- * and is looked at every 0.25 ms or so), and then once more, which the first wait's time-out
+ * counterpart).  Launches one warp whose even lanes wait on a barrier nothing completes, its odd
+ * lanes on a complete one (no lane may leave alone), in the very code the attention kernels wait
+ * with, with a limit of `limit_cycles` SM clocks (1 .. 2^31; theirs is 2^31, and is looked at every
+ * 0.25 ms or so), and then once more, which the first wait's time-out
  * must end at once.  *device_status receives what an attention kernel would write:
  * FP4ATTN_ERR_TIMEOUT once the limit has run out (expected), FP4ATTN_OK otherwise.  The warp
  * returns normally; the context stays usable.

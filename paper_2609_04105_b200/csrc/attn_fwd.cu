@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(128, 1) mma_peak_kernel(int iters, unsigned lo
     const long long t0 = clock64();
     for (int i = 0; i < iters; ++i) tc_mma_fp4_2x(tmem + 128 * (i & 1), ad, bd, idesc, tmem + 480, tmem + 484, 1);
     tc_commit(sbase + 9216);
-    const bool ok = mbar_wait(sbase + 9216, 0, abort_at);
+    const bool ok = mbar_wait_thread(sbase + 9216, 0, abort_at);
     const long long t1 = clock64();
     if (ok) atomicMax(cycles_out, (unsigned long long)(t1 - t0));
   }
@@ -539,15 +539,23 @@ __global__ void __launch_bounds__(128, 1) mma_peak_kernel(int iters, unsigned lo
 }
 
 // ------------------------------------------------------------------ bounded-wait self-test
-// One warp waits twice on an mbarrier that nothing will ever complete, in the attention kernels' own mbar_wait with a short
-// limit, and must come back through their time-out path (abort word -> status word), from the second wait at its first look.
+// One warp waits twice in the attention kernels' own mbar_wait with a short limit and must come back through their time-out
+// path (abort word -> status word), from the second wait at its first look.  Even lanes wait on an mbarrier that nothing will
+// ever complete, odd lanes on one that is complete: none may leave without the others.
 __global__ void __launch_bounds__(32, 1) bounded_wait_selftest_kernel(uint32_t limit_cycles, int* status) {
-  __shared__ __align__(8) uint64_t never;
+  __shared__ __align__(8) uint64_t barrier[2];
   __shared__ int abort_word;
-  if (threadIdx.x == 0) { mbar_init(smem_u32(&never), 1); abort_word = 0; fence_barrier_init(); }
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 2; ++i) mbar_init(smem_u32(&barrier[i]), 1);
+    abort_word = 0;
+    fence_barrier_init();
+    mbar_arrive(smem_u32(&barrier[1]));
+  }
   __syncwarp();
   bool ok = false;
-  for (int i = 0; i < 2; ++i) ok |= mbar_wait(smem_u32(&never), 0, smem_u32(&abort_word), limit_cycles);
+  const uint32_t bar = smem_u32(&barrier[threadIdx.x & 1]), word = smem_u32(&abort_word);
+  ok |= mbar_wait<true>(bar, 0, word, limit_cycles);
+  ok |= mbar_wait<false>(bar, 0, word, limit_cycles);
   ok = __any_sync(0xffffffffu, ok);
   if (threadIdx.x == 0) *status = (!ok && *(volatile int*)&abort_word) ? FP4ATTN_ERR_TIMEOUT : FP4ATTN_OK;
 }

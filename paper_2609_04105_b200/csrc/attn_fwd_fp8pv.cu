@@ -181,7 +181,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       if (phs >= 1) { wb = decode_item<CAUSAL>(item_at<CAUSAL>(phs - 1), p, qtiles, seq); TB = wb.T2; }
       if (phs < n_my) {
         const int qb = phs & 1;
-        if (phs >= 2) ok = mbar_wait(bar(B8_QFREE0 + qb), ((phs >> 1) - 1) & 1, abort_at);
+        if (phs >= 2) ok = mbar_wait<false>(bar(B8_QFREE0 + qb), ((phs >> 1) - 1) & 1, abort_at);
         if (!ok) break;
         if (elect_one()) {
           mbar_arrive_expect_tx(bar(B8_QFULL0 + qb), C::Q_BYTES + C::QSF_BYTES);
@@ -196,7 +196,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           const int kind = j ^ (s2 & 1);                            // 0: A-step of item phs, 1: B-step of item phs - 1
           if (s2 >= (kind ? TB : TA)) continue;
           const WorkItem& wi = kind ? wb : wa;
-          if (gs >= (uint32_t)C8::NST) ok = mbar_wait(bar_empty(s), ph ^ 1, abort_at);
+          if (gs >= (uint32_t)C8::NST) ok = mbar_wait<false>(bar_empty(s), ph ^ 1, abort_at);
           if (!ok) break;
           const uint32_t fb = bar_full(s);
           if (elect_one()) {
@@ -230,7 +230,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       if (phs >= 1) TB = decode_item<CAUSAL>(item_at<CAUSAL>(phs - 1), p, qtiles, seq).T2;
       if (phs < n_my) {
         const int qb = phs & 1;
-        ok = mbar_wait(bar(B8_QFULL0 + qb), (phs >> 1) & 1, abort_at);
+        ok = mbar_wait<false>(bar(B8_QFULL0 + qb), (phs >> 1) & 1, abort_at);
         if (!ok) break;
         tc_fence_after();
         if (elect_one()) {
@@ -249,8 +249,8 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           const int qb = (kind ? phs - 1 : phs) & 1;              // the Q buffer of the step's item
           const int pr = g & 1;
           const uint32_t m = g >> 1;
-          ok = mbar_wait(bar_full(sq), phq, abort_at);
-          if (ok && m > 0) ok = mbar_wait(bar(B8_SEMPTY0 + pr), (m - 1) & 1, abort_at);   // both teams have read the slot
+          ok = mbar_wait<false>(bar_full(sq), phq, abort_at);
+          if (ok && m > 0) ok = mbar_wait<false>(bar(B8_SEMPTY0 + pr), (m - 1) & 1, abort_at);   // both teams have read the slot
           if (!ok) break;
           tc_fence_after();
           const uint32_t tSFQ = tmem + kColSFQ + 8 * qb;
@@ -292,7 +292,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       int TA = 0, TB = 0;
       if (phs < n_my) TA = decode_item<CAUSAL>(item_at<CAUSAL>(phs), p, qtiles, seq).T2;
       if (phs >= 1) TB = decode_item<CAUSAL>(item_at<CAUSAL>(phs - 1), p, qtiles, seq).T2;
-      if (phs >= 2) ok = mbar_wait(bar(B8_OFREE), (phs - 2) & 1, abort_at);   // epilogue of item phs - 2 has read O
+      if (phs >= 2) ok = mbar_wait<false>(bar(B8_OFREE), (phs - 2) & 1, abort_at);   // epilogue of item phs - 2 has read O
       const int TM = TA > TB ? TA : TB;
       for (int s2 = 0; ok && s2 < TM; ++s2) {
 #pragma unroll
@@ -301,7 +301,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           if (s2 >= (kind ? TB : TA)) continue;
           if (kind == 0) { ++g; continue; }                       // an A-step: only its slot is counted
           const int pr = g & 1;
-          ok = mbar_wait(bar(B8_SMDONE0 + pr), (pr ? nb[1] : nb[0]) & 1, abort_at);   // bytes of both tiles are in tensor memory
+          ok = mbar_wait<false>(bar(B8_SMDONE0 + pr), (pr ? nb[1] : nb[0]) & 1, abort_at);   // bytes of both tiles are in tensor memory
           if (!ok) break;
           if (pr) ++nb[1]; else ++nb[0];
           tc_fence_after();
@@ -331,7 +331,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     bool ok = true;
     for (int k = 0; ok && k < n_my; ++k) {
       const WorkItem wi = decode_item<CAUSAL>(item_at<CAUSAL>(k), p, qtiles, seq);
-      ok = mbar_wait(bar(B8_OFULL), k & 1, abort_at);
+      ok = mbar_wait<false>(bar(B8_OFULL), k & 1, abort_at);
       if (!ok) break;
       tc_fence_after();
       const int mu = reinterpret_cast<const int*>(sgen + C8::OFF_MU)[(k & 1) * BM + row];   // written before any PV of the item
@@ -419,7 +419,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           const int kind = j ^ (s2 & 1);
           if (s2 >= (kind ? TB : TA)) continue;
           if ((int)(g & 1) != pr) { ++g; continue; }              // the other pair's step
-          ok = mbar_wait(sfull, (g >> 1) & 1, abort_at);
+          ok = mbar_wait<false>(sfull, (g >> 1) & 1, abort_at);
           if (!ok) break;
           tc_fence_after();
           uint32_t sraw[32];
@@ -453,7 +453,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             if (diag) mask_scores(sraw, vb - 32);
             fp8_p_block(sraw, c2, b, w + 8);
             // the pair's probability slot was last read by the PV product of this team's previous B-visit
-            if (nbt > 0) ok = mbar_wait(pfree, (nbt - 1) & 1, abort_at);
+            if (nbt > 0) ok = mbar_wait<false>(pfree, (nbt - 1) & 1, abort_at);
             if (!ok) break;
             tmem_st_32x32b_x16(tP, w);
             tmem_wait_st();
@@ -472,7 +472,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         rmax[team * BM + row] = smax;                           // (-inf from a team that served none of the item's A-steps)
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(B8_MURDY0 + (phs & 1)));
-        ok = mbar_wait(bar(B8_MURDY0 + (phs & 1)), (phs >> 1) & 1, abort_at);
+        ok = mbar_wait<false>(bar(B8_MURDY0 + (phs & 1)), (phs >> 1) & 1, abort_at);
         if (!ok) break;
         const float mall = fmaxf(fmaxf(rmax[row], rmax[BM + row]), fmaxf(rmax[2 * BM + row], rmax[3 * BM + row]));
         const float ymax = fminf(fmaxf(__fmul_rn(mall, c32), -2097152.0f), 2097152.0f);

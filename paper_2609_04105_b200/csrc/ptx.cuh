@@ -46,8 +46,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // waiting warps share their schedulers with the softmax warps, whose time is instruction dispatch, so what a wait executes
 // is taken from them.  Attention at B=4, H=16, N=8192, d=128 (exact | affine map): a poll with a suspend-time hint, a clock
 // read, a look at the abort flag and a warp vote around it all 967 | 750 us; bare polls with the hint 923 | 687 us; without
-// it 903 | 619 us; four polls per trip of the counter 916 | 620 us.  All lanes of a warp poll the same barrier in the same
-// instruction, so they leave together without a vote.
+// it 903 | 619 us; four polls per trip of the counter 916 | 620 us.
 // How long the hardware suspends a poll is its own choice (measured on a barrier that nothing completes: 4 us), so a count of
 // polls bounds no time: every kPolls polls the wait looks at the abort word and the clock.  Both loops are one piece of assembly and the word goes by its shared-memory
 // address: the same as C++ statements after the poll loop, with a generic pointer, spilled up to 32 bytes a thread and
@@ -71,10 +70,20 @@ __device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, uint32_
       : "=r"(ok) : "r"(bar), "r"(parity), "r"(abort_at), "r"(limit), "n"(kPolls - 1), "n"(kPolls) : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t abort_at, uint32_t limit = kWaitClocks) {
+// One thread waits by itself.
+__device__ __forceinline__ bool mbar_wait_thread(uint32_t bar, uint32_t parity, uint32_t abort_at, uint32_t limit = kWaitClocks) {
   if (mbar_poll(bar, parity, abort_at, limit)) return true;
   asm volatile("st.volatile.shared.u32 [%0], 1;" ::"r"(abort_at) : "memory");
   return false;
+}
+// The whole warp waits and leaves as one, with one answer: a poll's answer is each thread's own, the warp may come here split
+// (from an arrival of lane 0), and what follows are warp-wide instructions, which a part of a warp must not enter.
+// VOTE_FIRST: a first poll with a vote of its own, which most waits end with: d = 64,
+// N = 8192, NVFP4 1852 us without, 1815 with it; not in the FP8 P/V kernels (masked, N = 9600: 214 us without, 220 with it).
+template <bool VOTE_FIRST = true>
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t abort_at, uint32_t limit = kWaitClocks) {
+  if (VOTE_FIRST && __all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait_thread(bar, parity, abort_at, limit));
 }
 
 __device__ __forceinline__ void fence_barrier_init() {

@@ -290,7 +290,8 @@ def test_bounded_wait_times_out_and_reports_status():
 
 @pytest.mark.parametrize("limit", [1, 1 << 28])
 def test_bounded_wait_limit_is_a_time_and_ends_the_other_waits(limit):
-    """Two waits in the kernels' own wait code: the first lasts its limit in SM clocks (2 GHz at most), the second ends with
+    """Two waits in the kernels' own wait code, on a barrier that nothing completes for half of the warp's lanes and a complete
+    one for the others (which must not leave alone: the status would be 0): the first lasts its limit in SM clocks (2 GHz at most), the second ends with
     it.  A look at the clock comes every 64 polls, each suspended for some 4 us: under a millisecond."""
     from paper_2609_04105_b200 import binding as Bd
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
