@@ -319,10 +319,21 @@ __host__ __device__ constexpr uint32_t counted_words_of(int pmap) { return pmap 
 // RULE: block exponent from the block maximum - 0 ceiling, 1 threshold rule, 2 the better of ceiling and ceiling - 1 by
 // squared error of the 32 represented values (ideal map only; see direct_p_block_mse)
 __device__ __forceinline__ void direct_p_block_mse(const uint32_t* sraw, float c32, int& E, uint32_t* words);
-// keys from `visible` on (causal mask, padding) get -inf: they never raise a block maximum and always code to 0
+// keys from `visible` on (causal mask, padding) get -inf: they never raise a block maximum
 __device__ __forceinline__ void mask_scores(uint32_t* sraw, int visible) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) sraw[i] = (i < visible) ? sraw[i] : 0xFF800000u;
+}
+
+// ... and their probabilities are cleared, KEYS to a word of codes or bytes: -inf alone makes them 0 only where the score
+// constant is not 0 (NVFP4 Q and K so small that the product of their encode factors overflows)
+template <int KEYS, int WORDS>
+__device__ __forceinline__ void mask_probabilities(uint32_t* words, int visible) {
+#pragma unroll
+  for (int i = 0; i < WORDS; ++i) {
+    const int n = visible - KEYS * i;
+    words[i] = n >= KEYS ? words[i] : n <= 0 ? 0u : words[i] & ((1u << (32 / KEYS * n)) - 1u);
+  }
 }
 
 // c2 = {c, c}, ca2 = {fl32(A c), fl32(A c)}: 64-bit so that they can stay in uniform registers (kernel parameters)

@@ -457,6 +457,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // masked stage: this row sees the first `vis` keys of the stage; the team's tile starts at key 64*(team&1)
         if (CAUSAL && g == gdiag) mask_scores(sraw, vis - 64 * (team & 1));
         direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E0, pw);
+        if (CAUSAL && g == gdiag) mask_probabilities<8, 4>(pw, vis - 64 * (team & 1));
         tmem_ld_32x32b_x32(tS + 32, sraw);
         tmem_wait_ld();
         tc_fence_before();
@@ -464,6 +465,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if (lane == 0) mbar_arrive(sempty);                     // pair may take the stage after next
         if (CAUSAL && g == gdiag) mask_scores(sraw, vis - 64 * (team & 1) - 32);
         direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E1, pw + 4);
+        if (CAUSAL && g == gdiag) mask_probabilities<8, 4>(pw + 4, vis - 64 * (team & 1) - 32);
         if (!mbar_wait(pfree, par ^ 1, abort_at)) { ok = false; break; }   // PV of the pair's previous stage is done (a fresh barrier passes)
         // fixed reference: E8M0 bytes of the two blocks against the constant; below the range a zero block (no codes,
         // so that a row without any live block shows as a zero row sum), above it an error
