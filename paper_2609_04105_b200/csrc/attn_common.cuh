@@ -172,6 +172,13 @@ __device__ __forceinline__ void fill_skipped(const SeqTable* st, const AttnParam
   }
 }
 
+// two bf16 of O, round to nearest even, the largest finite value instead of an infinity
+__device__ __forceinline__ uint32_t bf16x2_finite(float lo, float hi) {
+  uint32_t w;
+  asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(hi), "f"(lo));
+  return w;
+}
+
 // floor(n / d) for n < 2^31 through the precomputed reciprocal ceil(2^64 / d) (0 stands for d = 1): the
 // roles decode a work item on their critical path, and a 32-bit division costs some fifty instructions
 __device__ __forceinline__ int fast_div(int n, unsigned long long recip) {
@@ -283,7 +290,8 @@ __device__ __forceinline__ void fma2(float s0, float s1, float c, float b, float
 //   u1 = a1 x + k1    crosses 1/4, 3/4      at log2 1/4, log2 7/4
 //   u2 = a2 x + k2    crosses 1/4, 3/4      at log2 3/4, log2 7/2
 // The next crossing of each lies above 3.32, and x never exceeds log2 7.5 = 2.91 (log2 6 under the ceiling rule) by
-// construction of the block exponent, which leaves room for its rounding up to |y| = 2^21; negative arguments are clamped to code 0 by the conversion.  The three counts never sum to more than 7, so the packed
+// construction of the block exponent, which leaves room for its rounding up to |y| = 2^21 (beyond, where the exponent is
+// clamped, counts of 8 and more are possible: other codes, signs and carries; the epilogue keeps what follows finite); negative arguments are clamped to code 0 by the conversion.  The three counts never sum to more than 7, so the packed
 // words of eight codes simply add.  The arguments are float32, so the codes are those of the exact exponential up to the
 // rounding of x at a boundary, as with ex2.approx (2-million-score sweeps at |y| up to 2000: no mismatch further than
 // 0.3 spacings of y from a boundary for either).

@@ -341,8 +341,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         tmem_wait_ld();
         Lhw = __uint_as_float(r16[0]);
       }
-      const float inv = __frcp_rn(6.0f * Lhw);
       if (FIXREF && !(Lhw > 0.f && Lhw < INFINITY) && p.status) *p.status = FP4ATTN_ERR_RANGE;   // nothing of the row is inside the byte range
+      if (!(Lhw > 0.f)) Lhw = 1.f;                              // logits beyond 2^21: codes of any sign
+      const float inv = __frcp_rn(6.0f * Lhw);
       const size_t grow = (size_t)wi.qrow0 + row;
       // stage the bf16 tile in shared memory (128-byte rows, 128B-swizzled like the tensor map) and
       // let TMA write it out, so O is released after four TMEM reads instead of after 16 global stores
@@ -363,8 +364,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
           uint32_t pk[4];
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(o[c + 2 * q]) * inv, __uint_as_float(o[c + 2 * q + 1]) * inv);
-            pk[q] = *reinterpret_cast<const uint32_t*>(&hh);
+            pk[q] = bf16x2_finite(__uint_as_float(o[c + 2 * q]) * inv, __uint_as_float(o[c + 2 * q + 1]) * inv);
           }
           const int chunk = ((c0 & 63) + c) >> 3;               // 16-byte chunk of the 128-byte row
           *reinterpret_cast<uint4*>(half + ((chunk ^ (row & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);

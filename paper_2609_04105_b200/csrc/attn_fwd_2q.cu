@@ -321,6 +321,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
           tmem_wait_ld();
           Lhw = __uint_as_float(r16[0]);
         }
+        if (!(Lhw > 0.f)) Lhw = 1.f;                            // logits beyond 2^21: codes of any sign
         const float inv = __frcp_rn(6.0f * Lhw);
         if (lane == 0) bulk_wait_read_all();                    // this warp's previous store has read the buffer
         __syncwarp();
@@ -340,8 +341,7 @@ attn_fwd_2q_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             uint32_t pk[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              const __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(o[k + 2 * j]) * inv, __uint_as_float(o[k + 2 * j + 1]) * inv);
-              pk[j] = *reinterpret_cast<const uint32_t*>(&hh);
+              pk[j] = bf16x2_finite(__uint_as_float(o[k + 2 * j]) * inv, __uint_as_float(o[k + 2 * j + 1]) * inv);
             }
             const int chunk = (16 * c + k) >> 3;
             *reinterpret_cast<uint4*>(orow + ((chunk ^ (row & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);

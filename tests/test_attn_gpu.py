@@ -261,6 +261,19 @@ def test_cached_tensor_maps_follow_the_buffers():
         Bd.fp4attn_release()
 
 
+@pytest.mark.parametrize("schedule,d", [(0, 64), (0, 128), (1, 64)])
+@pytest.mark.parametrize("softmax_scale", [3e5, 1e6, 1e8])
+def test_logits_beyond_the_stated_range_give_finite_results(schedule, d, softmax_scale):
+    """|y| < 2^21 is the range of the logits; beyond it the results are unspecified, but finite."""
+    from paper_2609_04105_b200 import binding as Bd
+    g = torch.Generator(device="cuda").manual_seed(d)
+    x = [torch.randn((2, 4, 512, d), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3)]
+    for fmt in (Bd.FMT_MXFP4, Bd.FMT_NVFP4):
+        O, L = Bd.fp4attn_fwd(Bd.fp4attn_quantize(x[0], fmt, Bd.ROLE_Q), Bd.fp4attn_quantize(x[1], fmt, Bd.ROLE_K),
+                              Bd.fp4attn_quantize(x[2], Bd.FMT_MXFP4, Bd.ROLE_V), softmax_scale=softmax_scale, schedule=schedule)
+        assert torch.isfinite(O.float()).all() and torch.isfinite(L).all()
+
+
 def test_invalid_arguments_are_rejected_before_launch():
     from paper_2609_04105_b200 import binding as Bd
     x = torch.zeros((1, 1, 100, 128), dtype=torch.bfloat16, device="cuda")
