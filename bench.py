@@ -640,11 +640,8 @@ def run_cuda(args, w):
     roof_softmax = {"kernel": roof["kernel"], "bound": "alu", "achieved": attn_tflops, "peak": arith_peak, "unit": UNIT,
                     "frac": attn_tflops / arith_peak if arith_peak else None, "traffic": None,
                     "clk_per_32x32_block_per_scheduler": arith_clk_per_block,
-                    "peak_source": "measured on this device: the score -> code arithmetic for map '%s' (exact codes: with 12 of 16 "
-                                   "pairs on ex2.approx, where the kernel has 8) run alone, four "
-                                   "warps per scheduler (fp4attn_softmax_arith_probe), at the median SM clock of the timed steps; "
-                                   "for exact codes the SFU's 16 ex2/clk/SM (12 of 16 pairs -> 192 clk per block) is the unit "
-                                   "that binds" % args.p_map}
+                    "peak_source": "measured on this device: the kernel's score -> code arithmetic for map '%s' run alone, four "
+                                   "warps per scheduler (fp4attn_softmax_arith_probe), at the median SM clock of the timed steps" % args.p_map}
     for rec in other_maps.values():                                  # the same arithmetic ceiling for the other code maps
         if "softmax_arith_clk_per_block" in rec and sm_hz:
             pk = sms * 4 * (4.0 * 32 * 32 * w.d) / rec["softmax_arith_clk_per_block"] * sm_hz * 1e6 / 1e12

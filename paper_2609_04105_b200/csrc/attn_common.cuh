@@ -345,12 +345,12 @@ __device__ __forceinline__ void mask_probabilities(uint32_t* words, int visible)
 }
 
 // c2 = {c, c}, ca2 = {fl32(A c), fl32(A c)}: 64-bit so that they can stay in uniform registers (kernel parameters)
-template <int PMAP, int RULE, uint32_t COUNTED = counted_words_of(PMAP)>
+template <int PMAP, int RULE>
 __device__ __forceinline__ void direct_p_block(const uint32_t* sraw, uint64_t c2, uint64_t ca2, float A, float B, int& E, uint32_t* words) {
   const float c32 = __uint_as_float((uint32_t)c2);
   if (RULE == 2) { direct_p_block_mse(sraw, c32, E, words); return; }
   constexpr bool THR16 = RULE == 1;
-  constexpr uint32_t kExact = exact_pairs_of(PMAP);
+  constexpr uint32_t kExact = exact_pairs_of(PMAP), kCounted = counted_words_of(PMAP);
   const float LOG2_6 = 2.5849625007211560f;
   // y is clamped to +-2^21 (scores beyond that are outside any softmax's range; a fully masked block,
   // max = -inf, lands on the lower clamp and becomes a zero block)
@@ -364,10 +364,10 @@ __device__ __forceinline__ void direct_p_block(const uint32_t* sraw, uint64_t c2
   E = (int)(__float_as_uint(t) - 0x4B400000u);
   const float bB = __fsub_rn(LOG2_6, __fsub_rn(t, M));          // t - M = (float)E, exact
   const float bA = __fmaf_rn(A, bB, B);                          // affine pairs only
-  static_assert(COUNTED == 0u || kExact == 0xFFFFu || kExact == 0x7777u, "a counted word has its first three pairs exact, or all four");
+  static_assert(kCounted == 0u || kExact == 0xFFFFu || kExact == 0x7777u, "a counted word has its first three pairs exact, or all four");
 #pragma unroll
   for (int w = 0; w < 4; ++w) {
-    const bool counted = (COUNTED >> w) & 1u;
+    const bool counted = (kCounted >> w) & 1u;
     float pv[8], q1[8], q2[8];
 #pragma unroll
     for (int i = 0; i < 8; i += 2) {

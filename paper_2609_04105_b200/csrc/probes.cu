@@ -15,8 +15,6 @@ __device__ __forceinline__ void probe_sts4(uint32_t addr, const uint32_t* r) {
   asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" :: "r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]));
 }
 
-// The ideal map runs with one counted word, i.e. 24 of a block's 32 elements per row on ex2.approx: the probe states what the
-// special-function unit allows with that share (192 clocks per block), the attention kernel leaves it 16.
 // Every warp converts `iters` blocks of 32 rows x 32 scores.  The scores of a block come from shared memory through
 // eight loads that all lanes address alike (one wavefront each, so the loads cost issue slots like the kernel's
 // tensor-memory load but no shared-memory bandwidth); the four code words go back to shared memory.
@@ -42,7 +40,7 @@ __global__ void __launch_bounds__(32 * kProbeWarps, 1) softmax_arith_probe_kerne
     int E;
 #pragma unroll
     for (int j = 0; j < 8; ++j) probe_lds4(in + 16 * j, &sraw[4 * j]);
-    direct_p_block<PMAP, 0, (PMAP == 0 ? 1u : 0u)>(sraw, pack2(c32, c32), pack2(A * c32, A * c32), A, B, E, w);
+    direct_p_block<PMAP, 0>(sraw, pack2(c32, c32), pack2(A * c32, A * c32), A, B, E, w);
     probe_sts4(out, w);
     acc += E;
   }
