@@ -90,8 +90,29 @@ struct Results {
     }
   }
 };
-void* data_of(PyObject* o) {                            // None: a null pointer
-  return THPVariable_Check(o) ? THPVariable_Unpack(o).data_ptr() : nullptr;
+// What a Python caller's `None if o is None else o.data_ptr()` gives: a null pointer for None, and an error for what has no
+// memory (an argument that is not a tensor must not pass for one that was left out).
+bool data_of(PyObject* o, void** ptr) {
+  *ptr = nullptr;
+  if (o == Py_None) return true;
+  if (THPVariable_Check(o)) {
+    *ptr = THPVariable_Unpack(o).data_ptr();
+    return true;
+  }
+  PyObject* p = PyObject_CallMethod(o, "data_ptr", nullptr);
+  if (p) *ptr = PyLong_AsVoidPtr(p);
+  Py_XDECREF(p);
+  return !PyErr_Occurred();
+}
+bool numel_of(PyObject* o, size_t* n) {
+  if (THPVariable_Check(o)) {
+    *n = (size_t)THPVariable_Unpack(o).numel();
+    return true;
+  }
+  PyObject* p = PyObject_CallMethod(o, "numel", nullptr);
+  if (p) *n = PyLong_AsSize_t(p);
+  Py_XDECREF(p);
+  return !PyErr_Occurred();
 }
 
 struct Input {
@@ -118,21 +139,26 @@ PyObject* result(const at::Tensor& packed, const at::Tensor* scales, const at::T
   return Py_BuildValue("(NNNN)", THPVariable_Wrap(packed), s, g, in.shape());
 }
 
-bool ints(PyObject* const* args, Py_ssize_t n, int* out) {
+// whole numbers; `convert`: whatever int() takes
+bool ints(PyObject* const* args, Py_ssize_t n, int* out, bool convert = false) {
   for (Py_ssize_t i = 0; i < n; ++i) {
-    long v;
-    if (PyLong_Check(args[i])) {
-      v = PyLong_AsLong(args[i]);
-    } else {                                            // whatever int() takes
-      PyObject* o = PyNumber_Long(args[i]);
-      if (!o) return false;
-      v = PyLong_AsLong(o);
-      Py_DECREF(o);
+    if (!convert && !PyLong_Check(args[i])) {
+      PyErr_Format(PyExc_TypeError, "int expected instead of %s instance", Py_TYPE(args[i])->tp_name);
+      return false;
     }
+    PyObject* o = PyLong_Check(args[i]) ? Py_NewRef(args[i]) : PyNumber_Long(args[i]);
+    const long v = o ? PyLong_AsLong(o) : -1;
+    Py_XDECREF(o);
     if (v == -1 && PyErr_Occurred()) return false;
     out[i] = (int)v;
   }
   return true;
+}
+bool number(PyObject* o, float* out) {                  // whatever float() takes
+  PyObject* f = PyNumber_Float(o);
+  if (f) *out = (float)PyFloat_AsDouble(f);
+  Py_XDECREF(f);
+  return f != nullptr;
 }
 // A call into the library, which may block on a full launch queue, without the interpreter lock (nothing in it may touch a
 // Python object).
@@ -187,9 +213,11 @@ PyObject* py_quantize(PyObject*, PyObject* const* args, Py_ssize_t n) {
   at::Tensor none, &packed = r.add({(int64_t)nb}, at::kByte), &scales = r.add({(int64_t)ns}, at::kByte);
   at::Tensor& G = fmt == FP4ATTN_FMT_NVFP4 ? r.add({1}, at::kFloat) : none;
   at::Tensor& ws = nw ? r.add({(int64_t)nw}, at::kByte) : none;
+  void* wptr = nullptr;
+  size_t wbytes = nw;
+  if (args[3] != Py_None && (!data_of(args[3], &wptr) || !numel_of(args[3], &wbytes))) return nullptr;
   r.allocate(in.t->device());
-  void* const wptr = nw ? ws.data_ptr() : data_of(args[3]);
-  const size_t wbytes = nw ? nw : wptr ? (size_t)THPVariable_Unpack(args[3]).numel() : 0;
+  if (nw) wptr = ws.data_ptr();
   const int rc = unlocked([&] { return g_api.quantize(in.t->data_ptr(), fmt, role, in.B, in.H, in.N, in.d, packed.data_ptr(), scales.data_ptr(),
                                 G.defined() ? G.data_ptr<float>() : nullptr, wptr, wbytes, stream()); });
   if (rc) return fail(rc, "fp4attn_quantize");
@@ -285,7 +313,12 @@ struct Operand {
       v[i] = PyObject_GetAttr(o, g_names[i]);
       ok = v[i] != nullptr;
     }
-    if (ok && (!THPVariable_Check(v[A_PACKED]) || !PyTuple_Check(v[A_SHAPE]) || PyTuple_GET_SIZE(v[A_SHAPE]) != 4)) {
+    if (ok && !PyTuple_Check(v[A_SHAPE])) {
+      PyObject* const t = PySequence_Tuple(v[A_SHAPE]);
+      Py_SETREF(v[A_SHAPE], t);
+      ok = t != nullptr;
+    }
+    if (ok && (!THPVariable_Check(v[A_PACKED]) || PyTuple_GET_SIZE(v[A_SHAPE]) != 4)) {
       PyErr_SetString(PyExc_TypeError, "fp4attn_fwd takes QuantizedOperand arguments");
       ok = false;
     }
@@ -293,12 +326,11 @@ struct Operand {
       const at::Tensor& t = THPVariable_Unpack(v[A_PACKED]);
       packed = t.data_ptr();
       device = t.device();
-      scales = data_of(v[A_SCALES]);
-      G = data_of(v[A_G]);
-      fmt = (int)PyLong_AsLong(v[A_FMT]);
-      per_head = PyObject_IsTrue(v[A_PER_HEAD]) == 1;
-      for (int i = 0; i < 4; ++i) shape[i] = (int)PyLong_AsLong(PyTuple_GET_ITEM(v[A_SHAPE], i));
-      ok = !PyErr_Occurred();
+      if (!data_of(v[A_SCALES], &scales) || !data_of(v[A_G], &G)) ok = false;
+      fmt = ok ? (int)PyLong_AsLong(v[A_FMT]) : 0;
+      per_head = ok && PyObject_IsTrue(v[A_PER_HEAD]) == 1;
+      for (int i = 0; ok && i < 4; ++i) shape[i] = (int)PyLong_AsLong(PyTuple_GET_ITEM(v[A_SHAPE], i));
+      ok = ok && !PyErr_Occurred();
     }
     for (int i = 0; i < A_COUNT; ++i) Py_XDECREF(v[i]);
     return ok;
@@ -335,30 +367,29 @@ PyObject* py_fwd(PyObject*, PyObject* const* args, Py_ssize_t n) {
   ops.g_per_head = q.per_head ? 1 : 0;
   ops.pv_fmt = fp8 ? FP4ATTN_PV_E4M3 : FP4ATTN_PV_MXFP4;
   ops.v_G = fp8 ? (const float*)v.G : nullptr;
-  ops.softmax_scale = (float)PyFloat_AsDouble(args[3]);
-  ops.affine_a = (float)PyFloat_AsDouble(args[8]);
-  ops.affine_b = (float)PyFloat_AsDouble(args[9]);
-  if (PyErr_Occurred() || !ints(args + 7, 1, &ops.p_map) || !ints(args + 10, 1, &ops.p_scale_rule) ||
-      !ints(args + 12, 1, &ops.exact_pairs) || !ints(args + 13, 1, &ops.schedule))
+  void *seq_len, *out_ptr, *lse_ptr, *status;
+  if (!number(args[3], &ops.softmax_scale) || !number(args[8], &ops.affine_a) || !number(args[9], &ops.affine_b) ||
+      !ints(args + 7, 1, &ops.p_map, true) || !ints(args + 10, 1, &ops.p_scale_rule, true) ||
+      !ints(args + 12, 1, &ops.exact_pairs, true) || !ints(args + 13, 1, &ops.schedule, true) || !data_of(seq, &seq_len) ||
+      !data_of(args[4], &out_ptr) || !data_of(args[5], &lse_ptr) || !data_of(args[6], &status))
     return nullptr;
-  ops.causal = PyObject_IsTrue(args[11]);
-  ops.seq_len = (const int*)data_of(seq);
+  if ((ops.causal = PyObject_IsTrue(args[11])) < 0) return nullptr;
+  ops.seq_len = (const int*)seq_len;
   if (args[15] != Py_None) {
     ops.row_reference = FP4ATTN_REFERENCE_FIXED;
-    if (!ints(args + 15, 1, &ops.fixed_reference)) return nullptr;
+    if (!ints(args + 15, 1, &ops.fixed_reference, true)) return nullptr;
   }
   PyObject *out = Py_NewRef(args[4]), *lse = Py_NewRef(args[5]);
   if (out == Py_None || lse == Py_None) {
     Results r;
     at::Tensor none, &o = out == Py_None ? r.add({B, H, N, d}, at::kBFloat16) : none, &l = lse == Py_None ? r.add({B, H, N}, at::kFloat) : none;
     r.allocate(q.device);
-    if (out == Py_None) Py_SETREF(out, THPVariable_Wrap(o));
-    if (lse == Py_None) Py_SETREF(lse, THPVariable_Wrap(l));
+    if (out == Py_None) { out_ptr = o.data_ptr(); Py_SETREF(out, THPVariable_Wrap(o)); }
+    if (lse == Py_None) { lse_ptr = l.data_ptr(); Py_SETREF(lse, THPVariable_Wrap(l)); }
   }
   int rc = -1;
   if (out && lse) {
-    void *o = data_of(out), *l = data_of(lse), *st = data_of(args[6]);
-    rc = unlocked([&] { return g_api.fwd(&ops, B, H, N, d, o, (float*)l, (int*)st, stream()); });
+    rc = unlocked([&] { return g_api.fwd(&ops, B, H, N, d, out_ptr, (float*)lse_ptr, (int*)status, stream()); });
   }
   if (rc) {
     Py_XDECREF(out);

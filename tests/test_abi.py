@@ -105,3 +105,20 @@ def test_header_is_plain_c_and_the_struct_layout_matches_the_binding(lib, tmp_pa
     assert int(out["packed"]) == 4 * 16 * 4096 * 128 // 2
     assert int(out["null_ops"]) == binding.ERR_INVALID_ARG
     assert out["status"] == "invalid argument"
+
+
+def _cpu_operands(N=128, d=64):
+    import torch
+    from paper_2609_04105_b200 import binding as Bd
+    z = torch.zeros(N * d // 2, dtype=torch.uint8)
+    return [Bd.QuantizedOperand(z, z, None, Bd.FMT_MXFP4, role, (1, 1, N, d)) for role in (0, 1, 2)]
+
+
+@pytest.mark.parametrize("name,value", [("status", "x"), ("status", 0), ("lse", [1.0]), ("out", object())])
+def test_forward_refuses_an_argument_without_memory(lib, name, value):
+    """An argument that is not a tensor (and has no data_ptr) must not pass for one that was left out."""
+    import torch
+    from paper_2609_04105_b200 import binding as Bd
+    kw = {"out": torch.zeros((1, 1, 128, 64), dtype=torch.bfloat16), "lse": torch.zeros((1, 1, 128)), name: value}
+    with pytest.raises(AttributeError):
+        Bd.fp4attn_fwd(*_cpu_operands(), **kw)

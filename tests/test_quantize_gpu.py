@@ -244,6 +244,18 @@ def test_nvfp4_one_launch_and_two_launch_sizes(B, H, N, d, offset):
     _check_operand(Bd.fp4attn_quantize(t, Bd.FMT_NVFP4, Bd.ROLE_K), Qz.quantize_qk(bits, "nv"), Bd.ROLE_K)
 
 
+def test_quantizers_take_whole_numbers_and_tensors_only():
+    from paper_2609_04105_b200 import binding as Bd
+    x = torch.zeros((1, 1, 128, 64), dtype=torch.bfloat16, device="cuda")
+    for fmt, role in ((0.0, 0), ("0", 0), (0, 1.5)):
+        with pytest.raises(TypeError):
+            Bd.fp4attn_quantize(x, fmt, role)
+    with pytest.raises(TypeError):
+        Bd.fp4attn_quantize_mxfp4_rule(x, 0, "0")
+    with pytest.raises(AttributeError):
+        Bd.fp4attn_quantize(x, Bd.FMT_NVFP4, Bd.ROLE_Q, workspace=1)
+
+
 def test_nvfp4_per_head_rejects_v_and_missing_workspace():
     from paper_2609_04105_b200 import binding as Bd
     x = torch.zeros((1, 2, 128, 64), dtype=torch.bfloat16, device="cuda")
