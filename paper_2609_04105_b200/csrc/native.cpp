@@ -6,6 +6,7 @@
 // queries, torch.empty, stream look-up) took about 15 us per call: B=1, H=2, N=256 ran at 66 us per step, all of it host
 // time.
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/utils/object_ptr.h>
 
 #include <ATen/ATen.h>
 #include <ATen/cuda/EmptyTensor.h>
@@ -175,14 +176,14 @@ int unlocked(F call) {
 #define FP4_CATCH                                                                              \
   }                                                                                            \
   catch (const c10::OutOfMemoryError& e) {                                                     \
-    PyErr_SetString(THPException_OutOfMemory(), e.what_without_backtrace());                   \
+    PyErr_SetString(out_of_memory_class(), e.what_without_backtrace());                   \
     return nullptr;                                                                            \
   }                                                                                            \
   catch (const std::exception& e) {                                                            \
     PyErr_SetString(PyExc_RuntimeError, e.what());                                             \
     return nullptr;                                                                            \
   }
-PyObject* THPException_OutOfMemory() {                  // torch.OutOfMemoryError
+PyObject* out_of_memory_class() {                       // torch.OutOfMemoryError
   static PyObject* cls = [] {
     PyObject* torch = PyImport_ImportModule("torch");
     PyObject* c = torch ? PyObject_GetAttrString(torch, "OutOfMemoryError") : nullptr;
@@ -379,24 +380,18 @@ PyObject* py_fwd(PyObject*, PyObject* const* args, Py_ssize_t n) {
     ops.row_reference = FP4ATTN_REFERENCE_FIXED;
     if (!ints(args + 15, 1, &ops.fixed_reference, true)) return nullptr;
   }
-  PyObject *out = Py_NewRef(args[4]), *lse = Py_NewRef(args[5]);
-  if (out == Py_None || lse == Py_None) {
+  THPObjectPtr out(Py_NewRef(args[4])), lse(Py_NewRef(args[5]));        // given back on every way out, an exception's too
+  if (out.get() == Py_None || lse.get() == Py_None) {
     Results r;
-    at::Tensor none, &o = out == Py_None ? r.add({B, H, N, d}, at::kBFloat16) : none, &l = lse == Py_None ? r.add({B, H, N}, at::kFloat) : none;
+    at::Tensor none, &o = out.get() == Py_None ? r.add({B, H, N, d}, at::kBFloat16) : none, &l = lse.get() == Py_None ? r.add({B, H, N}, at::kFloat) : none;
     r.allocate(q.device);
-    if (out == Py_None) { out_ptr = o.data_ptr(); Py_SETREF(out, THPVariable_Wrap(o)); }
-    if (lse == Py_None) { lse_ptr = l.data_ptr(); Py_SETREF(lse, THPVariable_Wrap(l)); }
+    if (o.defined()) { out_ptr = o.data_ptr(); out = THPVariable_Wrap(o); }
+    if (l.defined()) { lse_ptr = l.data_ptr(); lse = THPVariable_Wrap(l); }
+    if (!out || !lse) return nullptr;
   }
-  int rc = -1;
-  if (out && lse) {
-    rc = unlocked([&] { return g_api.fwd(&ops, B, H, N, d, out_ptr, (float*)lse_ptr, (int*)status, stream()); });
-  }
-  if (rc) {
-    Py_XDECREF(out);
-    Py_XDECREF(lse);
-    return rc < 0 ? nullptr : fail(rc, "fp4attn_fwd");
-  }
-  return Py_BuildValue("(NN)", out, lse);
+  const int rc = unlocked([&] { return g_api.fwd(&ops, B, H, N, d, out_ptr, (float*)lse_ptr, (int*)status, stream()); });
+  if (rc) return fail(rc, "fp4attn_fwd");
+  return Py_BuildValue("(NN)", out.release(), lse.release());
   FP4_CATCH
 }
 

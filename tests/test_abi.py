@@ -122,3 +122,18 @@ def test_forward_refuses_an_argument_without_memory(lib, name, value):
     kw = {"out": torch.zeros((1, 1, 128, 64), dtype=torch.bfloat16), "lse": torch.zeros((1, 1, 128)), name: value}
     with pytest.raises(AttributeError):
         Bd.fp4attn_fwd(*_cpu_operands(), **kw)
+
+
+def test_forward_gives_back_what_it_was_given_when_an_allocation_fails(lib):
+    """The other output's allocation fails (no device memory for operands in host memory): no reference to `out` is kept."""
+    import sys
+    import torch
+    from paper_2609_04105_b200 import binding as Bd
+    if torch.cuda.is_available():
+        pytest.skip("needs a machine on which device memory cannot be allocated")
+    out = torch.zeros((1, 1, 128, 64), dtype=torch.bfloat16)
+    before = sys.getrefcount(out)
+    for _ in range(3):
+        with pytest.raises(Exception):
+            Bd.fp4attn_fwd(*_cpu_operands(), out=out)
+    assert sys.getrefcount(out) == before
