@@ -340,7 +340,8 @@ size_t fp4attn_attention_host_workspace_bytes(int qk_fmt, int B, int H, int N, i
  * its largest leg instead of the sum.  With MXFP4 a group is its units' Q, K and V; with NVFP4 Q and K (tensor-wide amax) come
  * in whole first and the groups are of V.  The copies then run on two internal streams (created on the first such call per
  * device and kept until the process exits; no device memory is allocated) that fork from `stream` and join back into it
- * through events.  Small problems run on `stream` alone.  Results are bit-identical either way.
+ * through events.  Small problems run on `stream` alone, and so does any other call between a pipelined call that was
+ * captured into a graph and the end of that capture.  Results are bit-identical either way.
  *
  * status_host (HOST pointer, preferably pinned; may be NULL): the call keeps a status word in its workspace,
  * clears it before its first kernel, hands it to every attention launch and copies it to *status_host at the

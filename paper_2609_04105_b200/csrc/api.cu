@@ -196,6 +196,15 @@ int host_groups(int fmt, int BH, int N, int d) {
   if (groups < 2) groups = 2;
   return groups < BH ? (int)groups : BH;
 }
+// A pipelined call that is captured into a graph draws the internal streams into that capture until it ends.  Any other call
+// - one that runs now, or one in another capture - must leave them alone and run on its own stream.
+bool in_another_capture(cudaStream_t internal, cudaStream_t st) {
+  cudaStreamCaptureStatus theirs, mine;
+  unsigned long long their_id = 0, my_id = 0;
+  if (cudaStreamGetCaptureInfo(internal, &theirs, &their_id) != cudaSuccess) return true;
+  if (theirs == cudaStreamCaptureStatusNone) return false;
+  return cudaStreamGetCaptureInfo(st, &mine, &my_id) != cudaSuccess || mine != cudaStreamCaptureStatusActive || my_id != their_id;
+}
 int attention_host_pipelined(int fmt, const void* q_host, const void* k_host, const void* v_host, float softmax_scale, int B, int H,
                              int N, int d, void* O_host, float* LSE_host, char* ws, const HostPlan& p,
                              size_t workspace_bytes, int* dev_status, cudaStream_t st) {
@@ -204,6 +213,7 @@ int attention_host_pipelined(int fmt, const void* q_host, const void* k_host, co
   std::lock_guard<std::mutex> lock(g_pipe_mutex);
   HostPipe* hp = host_pipe();
   if (!hp) return kNoPipeline;
+  if (in_another_capture(hp->h2d, st)) return kNoPipeline;
   if (cudaEventRecord(hp->start, st) != cudaSuccess ||         // fork: the copies start after the stream's earlier work
       cudaStreamWaitEvent(hp->h2d, hp->start, 0) != cudaSuccess || cudaStreamWaitEvent(hp->d2h, hp->start, 0) != cudaSuccess)
     return FP4ATTN_ERR_CUDA;

@@ -198,6 +198,44 @@ def test_host_buffer_groups_match_the_device_path(name, kw, pinned):
         assert torch.equal(out, O.cpu()) and torch.equal(lse, L.cpu())
 
 
+@pytest.mark.parametrize("captured,other", [(0, 1), (1, 0)])           # MXFP4, NVFP4
+def test_host_path_in_a_capture_and_beside_it(captured, other):
+    """A pipelined call that is captured holds the library's internal streams until the capture ends: a call on another stream
+    in between runs all the same, and the graph replays."""
+    from paper_2609_04105_b200 import binding as Bd
+    w = I.shrink(I.WORKLOADS["cfg1"], B=1, H=16, N=1024, d=128)
+
+    def problem(fmt, seed):
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        x = [torch.randn((w.B, w.H, w.N, w.d), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3)]
+        want = Bd.fp4attn_fwd(Bd.fp4attn_quantize(x[0], fmt, Bd.ROLE_Q), Bd.fp4attn_quantize(x[1], fmt, Bd.ROLE_K), Bd.fp4attn_quantize(x[2], 0, Bd.ROLE_V))
+        out, lse = torch.zeros(x[0].shape, dtype=torch.bfloat16, pin_memory=True), torch.zeros(x[0].shape[:3], pin_memory=True)
+        ws = torch.empty(Bd.fp4attn_attention_host_workspace_bytes(fmt, w.B, w.H, w.N, w.d), dtype=torch.uint8, device="cuda")
+        return [t.cpu().pin_memory() for t in x] + [fmt, out, lse, ws], [t.cpu() for t in want]
+
+    (a, want_a), (b, want_b) = problem(captured, 1), problem(other, 2)
+    for args in (a, b):                                                     # streams and kernels exist before the capture
+        Bd.fp4attn_attention_host(*args)
+    torch.cuda.synchronize()
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    for t in (*a[4:6], *b[4:6]):
+        t.zero_()
+    with torch.cuda.graph(graph, capture_error_mode="relaxed"):
+        Bd.fp4attn_attention_host(*a)
+        with torch.cuda.stream(side):
+            Bd.fp4attn_attention_host(*b)
+        Bd.fp4attn_attention_host(*a)                                       # and again in the same capture
+    torch.cuda.synchronize()
+    assert torch.equal(b[4], want_b[0]) and torch.equal(b[5], want_b[1])
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(a[4], want_a[0]) and torch.equal(a[5], want_a[1])
+    a[4].zero_()
+    Bd.fp4attn_attention_host(*a)                                           # pipelined again after the capture
+    torch.cuda.synchronize()
+    assert torch.equal(a[4], want_a[0])
+
+
 def test_host_buffer_entry_point_from_two_threads():
     """Two host threads, each with its own stream, workspace and host buffers, enqueue the pipelined host
     path at the same time (the library's internal copy streams and events are shared and guarded by a
