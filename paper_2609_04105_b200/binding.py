@@ -1,6 +1,6 @@
 """Thin binding over libfp4attn.so: argument marshalling only.
 
-The calls of a step (the quantizers and the forward) are marshalled by the native module _fp4attn_native.so, the others by
+The calls of a step (the quantizers and the forward) are marshalled by the native module _fp4attn_native, the others by
 ctypes.  PyTorch appears here for device memory and streams; every step of the path runs inside the library's CUDA kernels.
 The first call fails loudly when the library or the module is missing.
 """
@@ -15,6 +15,8 @@ from typing import Optional, Tuple
 
 import torch
 
+from .build import native_path
+
 FMT_MXFP4, FMT_NVFP4 = 0, 1
 ROLE_Q, ROLE_K, ROLE_V = 0, 1, 2
 PMAP_IDEAL, PMAP_AFFINE, PMAP_HYBRID = 0, 1, 2
@@ -27,7 +29,7 @@ QSCALE_CEIL, QSCALE_THR16, QSCALE_FLOOR, QSCALE_MSE = 0, 1, 2, 3
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libfp4attn.so")
-NATIVE_PATH = os.path.join(_HERE, "_fp4attn_native.so")
+NATIVE_PATH = native_path()
 
 EXPORTS = [
     "fp4attn_status_string", "fp4attn_version", "fp4attn_packed_bytes", "fp4attn_scale_bytes",
@@ -110,8 +112,8 @@ _NATIVE_CALLS = ["fp4attn_status_string", "fp4attn_packed_bytes", "fp4attn_scale
 
 def _load_native(lib_: ctypes.CDLL):
     if not os.path.exists(NATIVE_PATH):
-        raise Fp4AttnError(f"{NATIVE_PATH} is missing: build it with `python -m paper_2609_04105_b200.build` "
-                           "(there is no fallback path)")
+        raise Fp4AttnError(f"{NATIVE_PATH} is missing: build it for this Python and torch with "
+                           "`python -m paper_2609_04105_b200.build` (there is no fallback path)")
     loader = importlib.machinery.ExtensionFileLoader("_fp4attn_native", NATIVE_PATH)
     module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_fp4attn_native", loader))
     loader.exec_module(module)

@@ -137,3 +137,16 @@ def test_forward_gives_back_what_it_was_given_when_an_allocation_fails(lib):
         with pytest.raises(Exception):
             Bd.fp4attn_fwd(*_cpu_operands(), out=out)
     assert sys.getrefcount(out) == before
+
+
+def test_marshalling_module_is_tied_to_the_torch_it_was_built_for(lib, monkeypatch):
+    """Another torch or Python: another file, which is stale until it is built and which the binding asks for."""
+    import importlib.metadata
+    from paper_2609_04105_b200 import binding as Bd, build
+    here = build.native_path()
+    assert os.path.exists(here) and Bd.NATIVE_PATH == here
+    monkeypatch.setattr(importlib.metadata, "version", lambda name: "0.0")
+    assert build.native_path() != here and build._stale(build.native_path(), [])
+    monkeypatch.setattr(Bd, "NATIVE_PATH", build.native_path())
+    with pytest.raises(Bd.Fp4AttnError, match="build it for this Python and torch"):
+        Bd._load_native(Bd.lib())
