@@ -327,20 +327,21 @@ __host__ __device__ constexpr uint32_t counted_words_of(int pmap) { return pmap 
 // RULE: block exponent from the block maximum - 0 ceiling, 1 threshold rule, 2 the better of ceiling and ceiling - 1 by
 // squared error of the 32 represented values (ideal map only; see direct_p_block_mse)
 __device__ __forceinline__ void direct_p_block_mse(const uint32_t* sraw, float c32, int& E, uint32_t* words);
-// keys from `visible` on (causal mask, padding) get -inf: they never raise a block maximum
+// Keys from `visible` on (causal mask, padding) get -inf: they never raise a block maximum, and they code to 0 as long as the
+// score constant is not 0 (which NVFP4 Q and K make it that are so small that the product of their encode factors overflows).
 __device__ __forceinline__ void mask_scores(uint32_t* sraw, int visible) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) sraw[i] = (i < visible) ? sraw[i] : 0xFF800000u;
 }
-
-// ... and their probabilities are cleared, KEYS to a word of codes or bytes: -inf alone makes them 0 only where the score
-// constant is not 0 (NVFP4 Q and K so small that the product of their encode factors overflows)
-template <int KEYS, int WORDS>
-__device__ __forceinline__ void mask_probabilities(uint32_t* words, int visible) {
+// The score constant for masked keys: the smallest normal number instead of 0, which changes no score by 1e-25.
+__host__ __device__ __forceinline__ float nonzero(float c) { return c == 0.f ? 1.17549435e-38f : c; }
+// The FP8 P/V kernels clear the bytes of masked keys instead (half the instructions of a second masking of the scores; in the
+// FP4 kernels, which mask the scores for the block maximum anyway, clearing the codes too took 2.5 % of a causal step).
+__device__ __forceinline__ void mask_bytes(uint32_t* words, int visible) {
 #pragma unroll
-  for (int i = 0; i < WORDS; ++i) {
-    const int n = visible - KEYS * i;
-    words[i] = n >= KEYS ? words[i] : n <= 0 ? 0u : words[i] & ((1u << (32 / KEYS * n)) - 1u);
+  for (int i = 0; i < 8; ++i) {
+    const int n = visible - 4 * i;
+    words[i] = n >= 4 ? words[i] : n <= 0 ? 0u : words[i] & ((1u << (8 * n)) - 1u);
   }
 }
 

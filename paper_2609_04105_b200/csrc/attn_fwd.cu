@@ -421,10 +421,14 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     const uint32_t tP = tmem + ((uint32_t)(quarter * 32) << 16) + kColP + 8 * team;
     int2* meta = reinterpret_cast<int2*>(sgen + C::OFF_META + C::META_BYTES * pr + row * 16 + 8 * (team & 1));
     uint64_t c2 = p.c_mx2, ca2 = p.ca_mx2;
+    auto set_constant = [&](float c, float ca) {                // masked kernels: never 0, so that a masked key's -inf stays one
+      if (CAUSAL) { c = nonzero(c); ca = nonzero(ca); }
+      c2 = pack2(c, c);
+      ca2 = pack2(ca, ca);
+    };
     if (NV) {
       const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldcg(p.q_G), __ldcg(p.k_G)));
-      c2 = pack2(c, c);
-      ca2 = pack2(__fmul_rn(p.aff_a, c), __fmul_rn(p.aff_a, c));
+      set_constant(c, __fmul_rn(p.aff_a, c));
     }
     uint32_t g0 = 0;
     bool ok = true;
@@ -442,8 +446,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         vis = seen - (T2 - 1) * BS;
         if (NV == 2) {                                          // this unit's own pair of encode factors
           const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldcg(p.q_G + wi.bh), __ldcg(p.k_G + wi.kvh)));
-          c2 = pack2(c, c);
-          ca2 = pack2(__fmul_rn(p.aff_a, c), __fmul_rn(p.aff_a, c));
+          set_constant(c, __fmul_rn(p.aff_a, c));
         }
       }
       for (uint32_t g = g0 + ((g0 & 1) != (uint32_t)pr); g < g0 + T2; g += 2) {   // this team's stages of the item
@@ -457,7 +460,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         // masked stage: this row sees the first `vis` keys of the stage; the team's tile starts at key 64*(team&1)
         if (CAUSAL && g == gdiag) mask_scores(sraw, vis - 64 * (team & 1));
         direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E0, pw);
-        if (CAUSAL && g == gdiag) mask_probabilities<8, 4>(pw, vis - 64 * (team & 1));
         tmem_ld_32x32b_x32(tS + 32, sraw);
         tmem_wait_ld();
         tc_fence_before();
@@ -465,7 +467,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         if (lane == 0) mbar_arrive(sempty);                     // pair may take the stage after next
         if (CAUSAL && g == gdiag) mask_scores(sraw, vis - 64 * (team & 1) - 32);
         direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E1, pw + 4);
-        if (CAUSAL && g == gdiag) mask_probabilities<8, 4>(pw + 4, vis - 64 * (team & 1) - 32);
         if (!mbar_wait(pfree, par ^ 1, abort_at)) { ok = false; break; }   // PV of the pair's previous stage is done (a fresh barrier passes)
         // fixed reference: E8M0 bytes of the two blocks against the constant; below the range a zero block (no codes,
         // so that a row without any live block shows as a zero row sum), above it an error
@@ -734,8 +735,8 @@ extern "C" int fp4attn_fwd(const fp4attn_operands* ops, int B, int H, int N, int
   prm.aff_b = ops->affine_a != 0.f ? ops->affine_b : 1.2f;
   auto twice = [](float f) { uint32_t u; memcpy(&u, &f, 4); return (unsigned long long)u << 32 | u; };
   const float c_mx = prm.c_base / 36.0f;                           // IEEE division and products, as on the device
-  prm.c_mx2 = twice(c_mx);
-  prm.ca_mx2 = twice(prm.aff_a * c_mx);
+  prm.c_mx2 = twice(nonzero(c_mx));
+  prm.ca_mx2 = twice(nonzero(prm.aff_a * c_mx));
   prm.thr16 = ops->p_scale_rule == FP4ATTN_PSCALE_THR16;
   if (ops->schedule != FP4ATTN_SCHEDULE_ONE_QUERY && ops->schedule != FP4ATTN_SCHEDULE_TWO_QUERY) return FP4ATTN_ERR_INVALID_ARG;
   if (ops->pv_fmt != FP4ATTN_PV_MXFP4 && ops->pv_fmt != FP4ATTN_PV_E4M3) return FP4ATTN_ERR_INVALID_ARG;

@@ -444,14 +444,14 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             tmem_ld_32x32b_x32(tS, sraw);
             tmem_wait_ld();
             fp8_p_block(sraw, c2, b, w);
-            if (diag) mask_probabilities<4, 8>(w, vb);
+            if (diag) mask_bytes(w, vb);
             tmem_ld_32x32b_x32(tS + 32, sraw);
             tmem_wait_ld();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(sempty);
             fp8_p_block(sraw, c2, b, w + 8);
-            if (diag) mask_probabilities<4, 8>(w + 8, vb - 32);
+            if (diag) mask_bytes(w + 8, vb - 32);
             // the pair's probability slot was last read by the PV product of this team's previous B-visit
             if (nbt > 0) ok = mbar_wait<false>(pfree, (nbt - 1) & 1, abort_at);
             if (!ok) break;
