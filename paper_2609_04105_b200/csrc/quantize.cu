@@ -1,5 +1,6 @@
 // Operand quantizers: bf16 -> packed E2M1 + scale bytes in the 128x4 atom order.
-// HBM-bound: 128-bit loads, block amax by lane shuffles, 32-bit / 128-bit stores.  Loads are ld.global.cg: a kernel may have
+// HBM-bound: 256-bit loads (128-bit ones from tensors on a 16-byte boundary, and cp.async into shared memory for V), block
+// maxima by lane shuffles, 32- to 128-bit stores.  Loads are ld.global.cg: a kernel may have
 // started before its inputs were written (programmatic dependent launch), which rules out the non-coherent path.
 #include "common.cuh"
 
