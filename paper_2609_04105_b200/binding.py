@@ -3,6 +3,11 @@
 The calls of a step (the quantizers and the forward) are marshalled by the native module _fp4attn_native, the others by
 ctypes.  PyTorch appears here for device memory and streams; every step of the path runs inside the library's CUDA kernels.
 The first call fails loudly when the library or the module is missing.
+
+Memory of the results: what one call allocates (the tensors of an operand and its scratch; `out` and `lse`) is one block when
+it comes to no more than 1 MB, in separate ones otherwise.  Results that share a block share a storage: keeping one keeps the
+block, saving one saves it whole, and none may be resized in place (`resize_`, `out=` of another size).  A result that goes a
+way of its own is to be cloned, or `out` and `lse` given.
 """
 from __future__ import annotations
 

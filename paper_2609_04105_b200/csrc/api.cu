@@ -186,7 +186,9 @@ int enqueue_groups(HostPipe* hp, int fmt, int groups, const void* q_host, const 
 // Groups of about 2 MB of an operand, up to 8, and of 8 MB beyond: the first copies in and the last kernels and copy out,
 // which nothing overlaps, against some 15 us per group.  Measured over 1 .. 16 groups (us): 32 MB an operand, NVFP4 1 / 4 / 8 /
 // 16 groups 2620 / 2202 / 2112 / 2179, MXFP4 2605 / 2239 / 2179 / 2293; 8 MB 723 / 633 / 633 / 635; 2 MB, NVFP4 1 / 2 / 4 groups
-// 209 / 192 / 199, MXFP4 204 / 206 / 235.
+// 209 / 192 / 199, MXFP4 204 / 206 / 235.  8 / 12 / 16 groups, d = 128: 64 MB, MXFP4 4225 / 4307 / 4219, NVFP4 4119 / 4299 / 4047;
+// 96 MB 6219 / 6206 / 6225, 6144 / 6034 / 6304; 128 MB, N = 32768, 8460 / 8307 / 8312, 9480 / 9403 / 9271; N = 8192 8256 / 8229 /
+// 8190, 8184 / 8109 / 7951.
 int host_groups(int fmt, int BH, int N, int d) {
   const long long bytes = 2ll * BH * N * d;                       // of one operand
   if (bytes < (fmt == FP4ATTN_FMT_NVFP4 ? 1 << 20 : 4 << 20)) return 1;
