@@ -507,8 +507,9 @@ quant_nv_rows_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, ui
 }
 
 // Both passes over a unit with a factor of its own in one launch: a cluster takes the unit, its CTAs every cluster_size()-th
-// chunk.  The second pass, from the last chunk back, finds the unit in L2 (a device's worth of clusters holds some tens of
-// megabytes), so the tensor is read from memory once.
+// chunk, and the second pass runs from the last chunk back.  Units of up to 1 MB are still in L2 then (the resident clusters
+// hold 74 MB of them), so the tensor is read from memory once; of larger ones the part that is.  All resident clusters
+// read, meet and write at about the same time: 64 units of 1 MB take 25 us, 3.5 TB/s of input and output.
 template <int D, bool W32>
 __global__ void __launch_bounds__(kThreads, kRowsCtas)
 quant_nv_unit_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, uint8_t* __restrict__ sf, float* __restrict__ G_out,
@@ -642,14 +643,21 @@ static void launch_mx(const uint4* xs, int role, int B, int H, int N, int d, voi
   }
 }
 
-// CTAs of the cluster that takes a unit of so many chunks: up to eight (the portable limit)
-static unsigned cluster_for(size_t chunks) { return chunks >= 8 ? 8 : chunks >= 4 ? 4 : chunks >= 2 ? 2 : 1; }
-// One launch for both passes where the clusters fill the device about twice, so that some read while others write, or where
-// every CTA has at most two chunks and the second launch costs more than it brings.  Microseconds back to back, two launches
-// against one: 64 units of 64 chunks 28.8 / 24.6, 128 of 64 53.2 / 44.8, 328 of 4 13.0 / 11.5, 2 of 16 4.1 / 3.7, 2 of 4 4.0 /
-// 3.0; beyond the line 16 units of 64 chunks 10.6 / 15.2, 1 of 32 4.2 / 5.1.
+// CTAs of the cluster that takes a unit of so many chunks: up to eight (the portable limit), but four for 8 to 15 chunks once
+// clusters of eight would not all be resident: with one chunk a CTA (two at most) a wave brings too little for its start and
+// its two meetings.  128 / 192 KB a unit, us for clusters of eight / four: 64 units 5.8 / 6.1, 7.5 / 8.0; 128 units 9.9 / 8.2,
+// 12.3 / 10.7; 512 units 32.8 / 23.3, 39.7 / 34.2 (two launches 27.8, 42.1).
+static unsigned cluster_for(size_t units, size_t chunks) {
+  if (chunks >= 16 || (chunks >= 8 && units * 8 <= (size_t)kRowsCtas * device_sms())) return 8;
+  return chunks >= 4 ? 4 : chunks >= 2 ? 2 : 1;
+}
+// One launch for both passes where the clusters make two CTAs an SM, or where every CTA has at most two chunks and the second
+// launch costs more than it brings.  Below that two launches are faster, which give every CTA of the device a share.
+// Microseconds from a graph, two launches against one: 1 / 4 / 16 / 32 units of 512 KB 3.4 / 4.7, 3.9 / 4.9, 6.4 / 8.4, 10.0 /
+// 10.5; 4 / 8 of 1 MB 5.6 / 8.2, 7.1 / 11.1; 8 / 64 / 512 of 128 KB 3.6 / 2.8, 6.4 / 5.8, 27.8 / 23.3; 512 of 256 / 512 KB 54.6 / 45.6,
+// 101 / 81; 64 of 1 / 2 / 4 / 8 MB 28.6 / 25.0, 55.1 / 50.4, 98.3 / 89.5, 192 / 179.
 static bool nv_in_one_launch(size_t units, size_t chunks) {
-  const unsigned cluster = cluster_for(chunks);
+  const unsigned cluster = cluster_for(units, chunks);
   return chunks <= 2 * cluster || units * cluster >= (size_t)2 * device_sms();
 }
 
@@ -667,7 +675,7 @@ int launch_quantize(const void* x, int fmt, int role, int B, int H, int N, int d
     const size_t units = per_head ? (size_t)B * H : 1, per_unit = per_head ? unit_chunks : n_chunks;
     if (nv_in_one_launch(units, per_unit)) {
       const bool w32u = ((uintptr_t)xs & 31) == 0;
-      const unsigned cluster = cluster_for(per_unit);
+      const unsigned cluster = cluster_for(units, per_unit);
       launch_overlapped_clusters(d == 128 ? (w32u ? quant_nv_unit_kernel<128, true> : quant_nv_unit_kernel<128, false>)
                                  : (w32u ? quant_nv_unit_kernel<64, true> : quant_nv_unit_kernel<64, false>),
                         dim3((unsigned)units * cluster), kThreads, 0, st, cluster, xs, (uint2*)packed, (uint8_t*)scales, G_out, (int)per_unit);

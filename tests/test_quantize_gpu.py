@@ -224,7 +224,9 @@ def test_quantizers_at_chunk_edges_and_alignments(B, H, N, d, offset):
                                      (3, 1, 896, 64),        # seven chunks a unit: a cluster of four, two or one chunk each
                                      (1, 2, 1152, 128),      # eighteen: just too many for one launch
                                      (2, 20, 640, 128),      # forty units fill the device: ten chunks over eight CTAs
-                                     (5, 9, 1536, 64)])      # twelve
+                                     (5, 9, 1536, 64),       # twelve
+                                     (3, 25, 512, 128),      # eight chunks, more units than clusters of eight are resident: of four
+                                     (5, 15, 1152, 64)])     # nine
 @pytest.mark.parametrize("offset", [0, 8])
 def test_nvfp4_one_launch_and_two_launch_sizes(B, H, N, d, offset):
     """Units (and small tensors) that one cluster quantizes by itself, and sizes just beyond: bytes and factors of the oracle;
