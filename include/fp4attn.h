@@ -277,8 +277,8 @@ typedef struct {
  * With causal = 1 (the forward the paper's training section starts from, Section "Causal backward")
  * keys j > i are removed from row i before anything else: they never raise a block maximum, always
  * code to 0, and a block without a visible key contributes nothing.  (Should c come out as 0 - NVFP4
- * operands so small that G_q * G_k overflows - the kernels that remove keys take 2^-126 in its place.)  B, H, N, d describe Q and O;
- * K and V have kv_heads heads.
+ * operands so small that G_q * G_k overflows - the FP4 kernels that remove keys take 2^-126 in its place.)
+ * B, H, N, d describe Q and O; K and V have kv_heads heads.
  *
  * Padded sequences.  With seq_len != NULL, batch entry b holds a sequence of L = seq_len[b] tokens (1 <= L <= N) in
  * buffers laid out for N: keys L..N-1 are removed from every row of that entry exactly as a causal row's invisible
