@@ -24,6 +24,7 @@ constexpr int kRefHeadroom = 60; // ... and is then set this far ABOVE that expo
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColS = 0, kColO = 256, kColSFQ = 400, kColSFK = 416, kColSFV = 432, kColSFP = 448,
                    kColP = 456;      // P codes: [stage parity][tile] x 8 columns (64 keys x 4 bits per row)
+constexpr int kItemTable = 64;   // work items of a CTA that are decoded ahead (ItemRec)
 constexpr int kOnesRows = 16;    // rows of ones appended to V^T (the MMA's N must be a multiple of 16)
 
 template <int D, bool NV>
@@ -56,7 +57,8 @@ struct Cfg {
   static constexpr int OUT_BYTES = (D / 64) * BM * 128;
   static constexpr int OFF_BAR = OFF_OUT + OUT_BYTES;
   static constexpr int OFF_SEQ = OFF_BAR + 1024;                // SeqTable
-  static constexpr int SMEM_BYTES = OFF_SEQ + 1536 + 1024;      // + alignment slack
+  static constexpr int OFF_ITEMS = OFF_SEQ + 1536;              // item table
+  static constexpr int SMEM_BYTES = OFF_ITEMS + kItemTable * 32 + 1024;   // + alignment slack
   static constexpr uint64_t SWZ_QK = (ROW_BYTES == 64) ? kSwz64 : kSwz32;
   static_assert(STAGE_BYTES % 512 == 0 && OFF_STAGE % 1024 == 0 && OFF_OUT % 1024 == 0, "stage alignment");
   static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
@@ -242,6 +244,37 @@ __device__ __forceinline__ WorkItem decode_item(int item, const AttnParams& p, i
   return w;
 }
 
+// ---- the items of a CTA, decoded once
+// A masked item's decoding is some two hundred instructions (integer divisions, the ranks of a SeqTable), a unit's score
+// constant two loads from L2 and a division, and each of the 23 warps did both for every item, on schedulers whose issue slots
+// are what these kernels are bound by.  So the CTA's first kItemTable items are decoded when it starts, one warp an item; later
+// ones by every role for itself.  Attention alone, with the blocks of a masked stage told apart (masked_scores): B=2, H=32/8,
+// N=4096, d=128, causal, one NVFP4 factor per unit 140 -> 131 us; the same without a mask (B=4, H=16) 230 -> 226; padded batch
+// B=6, H=12, N=2176, d=64 59.8 -> 57.9.
+struct __align__(16) ItemRec {
+  WorkItem w;
+  float c;                 // the unit's score constant (NVFP4 factors per unit)
+};
+static_assert(sizeof(ItemRec) == 32, "the space behind the SeqTable");
+__device__ __forceinline__ float unit_score_constant(const AttnParams& p, const WorkItem& w) {
+  return __fdiv_rn(p.c_base, __fmul_rn(__ldcg(p.q_G + w.bh), __ldcg(p.k_G + w.kvh)));
+}
+// all threads; ends with a barrier
+template <bool MASKED, bool UNIT_CONSTANT>
+__device__ __forceinline__ void build_item_table(ItemRec* tab, int n_my, const AttnParams& p, int qtiles, const SeqTable* st) {
+  for (int i = threadIdx.x >> 5; i < min(n_my, kItemTable); i += kAttnThreads / 32) {
+    ItemRec r;
+    r.w = decode_item<MASKED>(item_at<MASKED>(i), p, qtiles, st);
+    r.c = UNIT_CONSTANT ? unit_score_constant(p, r.w) : 0.f;
+    if ((threadIdx.x & 31) == 0) tab[i] = r;
+  }
+  __syncthreads();
+}
+template <bool MASKED>
+__device__ __forceinline__ WorkItem item_of_cta(int i, const ItemRec* tab, const AttnParams& p, int qtiles, const SeqTable* st) {
+  return i < kItemTable ? tab[i].w : decode_item<MASKED>(item_at<MASKED>(i), p, qtiles, st);
+}
+
 // barrier slots (8 bytes each)
 enum { BAR_QFULL0 = 0, BAR_QFREE0 = 2, BAR_OFULL = 4, BAR_OFREE = 5, BAR_SFULL0 = 6, BAR_SEMPTY0 = 8,
        BAR_PFULL0 = 10, BAR_PFREE0 = 12, BAR_SMDONE0 = 14, BAR_DRAIN0 = 16, BAR_RING = 18 };
@@ -332,6 +365,20 @@ __device__ __forceinline__ void direct_p_block_mse(const uint32_t* sraw, float c
 __device__ __forceinline__ void mask_scores(uint32_t* sraw, int visible) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) sraw[i] = (i < visible) ? sraw[i] : 0xFF800000u;
+}
+// The scores of a block of a masked kernel, of whose 32 keys this row sees the first `visible`.  Whole warp.  False (and the
+// scores as they were): none of the warp's rows sees any.  Most blocks of a masked stage are seen by all rows of a warp or by
+// none (of a diagonal tile's sixteen, six and six), so only the others are masked.  (The FP8 P/V kernels lose 5 % with it.)
+__device__ __forceinline__ bool masked_scores(uint32_t* sraw, int visible) {
+  if (__all_sync(0xffffffffu, visible >= 32)) return true;
+  if (!__any_sync(0xffffffffu, visible > 0)) return false;
+  mask_scores(sraw, visible);
+  return true;
+}
+// what direct_p_block makes of 32 times -inf
+__device__ __forceinline__ void empty_block(int& E, uint32_t* words) {
+  E = -2097152;
+  words[0] = words[1] = words[2] = words[3] = 0u;
 }
 // The score constant for masked keys: the smallest normal number instead of 0, which changes no score by 1e-25.
 __host__ __device__ __forceinline__ float nonzero(float c) { return c == 0.f ? 1.17549435e-38f : c; }

@@ -105,8 +105,13 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   // this CTA's items.  Masked: item_at(0 .. n_my - 1).  Unmasked: blockIdx.x, blockIdx.x + gridDim.x, ... (every role counting
   // rounds instead of items costs these kernels registers: -1.6 % at d = 64)
   const int n_my = CAUSAL ? items_of_cta<CAUSAL>(p.sorted ? seq->first[p.B] : p.n_items) : 0;
+  constexpr bool kTable = CAUSAL || NV == 2;
+  ItemRec* const tab = reinterpret_cast<ItemRec*>(sgen + C::OFF_ITEMS);
+  if (kTable) build_item_table<CAUSAL, NV == 2>(tab, CAUSAL ? n_my : items_of_cta<false>(p.n_items), p, qtiles, seq);
   auto mine = [&](int i, int item) { return CAUSAL ? i < n_my : item < p.n_items; };
-  auto work = [&](int i, int item) { return decode_item<CAUSAL>(CAUSAL ? item_at<true>(i) : item, p, qtiles, seq); };
+  auto work = [&](int i, int item) {
+    return kTable ? item_of_cta<CAUSAL>(i, tab, p, qtiles, seq) : decode_item<false>(item, p, qtiles, seq);
+  };
 
   if (warp == 0) {
     // ===================================================================== TMA producer
@@ -426,7 +431,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
       c2 = pack2(c, c);
       ca2 = pack2(ca, ca);
     };
-    if (NV) {
+    if (NV == 1) {
       const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldcg(p.q_G), __ldcg(p.k_G)));
       set_constant(c, __fmul_rn(p.aff_a, c));
     }
@@ -445,7 +450,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         const int seen = (CAUSAL && p.causal) ? min(wi.len, wi.qt * BM + row + 1) : wi.len;
         vis = seen - (T2 - 1) * BS;
         if (NV == 2) {                                          // this unit's own pair of encode factors
-          const float c = __fdiv_rn(p.c_base, __fmul_rn(__ldcg(p.q_G + wi.bh), __ldcg(p.k_G + wi.kvh)));
+          const float c = i < kItemTable ? tab[i].c : unit_score_constant(p, wi);
           set_constant(c, __fmul_rn(p.aff_a, c));
         }
       }
@@ -455,18 +460,19 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         tc_fence_after();
         uint32_t sraw[32], pw[8];
         int E0, E1;
+        // masked stage: this row sees the first `vis` keys of the stage; the team's tile starts at key 64*(team&1)
+        const int v0 = CAUSAL && g == gdiag ? vis - 64 * (team & 1) : 64;
         tmem_ld_32x32b_x32(tS, sraw);
         tmem_wait_ld();
-        // masked stage: this row sees the first `vis` keys of the stage; the team's tile starts at key 64*(team&1)
-        if (CAUSAL && g == gdiag) mask_scores(sraw, vis - 64 * (team & 1));
-        direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E0, pw);
+        if (!CAUSAL || masked_scores(sraw, v0)) direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E0, pw);
+        else empty_block(E0, pw);
         tmem_ld_32x32b_x32(tS + 32, sraw);
         tmem_wait_ld();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(sempty);                     // pair may take the stage after next
-        if (CAUSAL && g == gdiag) mask_scores(sraw, vis - 64 * (team & 1) - 32);
-        direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E1, pw + 4);
+        if (!CAUSAL || masked_scores(sraw, v0 - 32)) direct_p_block<PMAP, THR16>(sraw, c2, ca2, p.aff_a, p.aff_b, E1, pw + 4);
+        else empty_block(E1, pw + 4);
         if (!mbar_wait(pfree, par ^ 1, abort_at)) { ok = false; break; }   // PV of the pair's previous stage is done (a fresh barrier passes)
         // fixed reference: E8M0 bytes of the two blocks against the constant; below the range a zero block (no codes,
         // so that a row without any live block shows as a zero row sum), above it an error
