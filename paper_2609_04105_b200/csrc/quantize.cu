@@ -434,19 +434,37 @@ __device__ __forceinline__ float e4m3_byte_to_f32(uint32_t b) {
   return __half2float(__ushort_as_half((unsigned short)(h2 & 0xFFFFu)));
 }
 
-// one chunk's codes and scale bytes from its bf16 words
+// fl32(x / 6), x >= 0: the rounded product with fl32(1/6) and one Newton step on its exact remainder (Markstein's theorem; every
+// significand checked against the division), three instructions where the general division takes about ten and a branch.
+// For x below 2^103; below 2^-100 the remainder may be subnormal and the result off by a unit, far under the smallest scale.
+__device__ __forceinline__ float sixth(float x) {
+  const float r = 0.16666667163372040f, q = __fmul_rn(x, r);
+  return __fmaf_rn(__fmaf_rn(-6.0f, q, x), r, q);
+}
+// G / S for scale byte b, 0 for S = 0 (a zero block) and for a NaN
+__device__ __forceinline__ float nv_ratio(uint32_t b, float G) {
+  const float S = e4m3_byte_to_f32(b);
+  return (S > 0.f) ? __fdiv_rn(G, S) : 0.f;
+}
+// The ratios of a tensor or unit by scale byte (bit 7 is never set but in a NaN): 128 divisions instead of one per block.
+// Whole block; ends with a barrier.
+__device__ __forceinline__ void nv_ratio_table(float* table, float G) {
+  if (threadIdx.x < 128) table[threadIdx.x] = nv_ratio(threadIdx.x, G);
+  __syncthreads();
+}
+
+// one chunk's codes and scale bytes from its bf16 words; `table`: nv_ratio_table, or null where the factor changes too often for one
 template <int D>
-__device__ __forceinline__ void nv_code_chunk(const uint32_t (&raw)[kLoads][8], float G, uint32_t chunk, uint2* packed, uint8_t* sf) {
+__device__ __forceinline__ void nv_code_chunk(const uint32_t (&raw)[kLoads][8], float G, const float* table, uint32_t chunk, uint2* packed, uint8_t* sf) {
   constexpr uint32_t LPR = D / 16;                 // lanes per row
   constexpr uint32_t CT = (D / 16 + 3) / 4;
   const uint32_t seg = threadIdx.x % LPR;
+  const bool plain = G < 1.2676506e30f;            // 2^100: a * G is then finite (a of a NaN tensor apart, which any quotient leaves one)
 #pragma unroll
   for (int k = 0; k < kLoads; ++k) {
-    const float a = __uint_as_float(absmax_bf16x16(raw[k]) << 16);
-    const float t = __fdiv_rn(__fmul_rn(a, G), 6.0f);
-    uint32_t sb = cvt_e4m3_byte(t);
-    const float S = e4m3_byte_to_f32(sb);
-    const float r = (S > 0.f) ? __fdiv_rn(G, S) : 0.f;
+    const float aG = __fmul_rn(__uint_as_float(absmax_bf16x16(raw[k]) << 16), G);
+    uint32_t sb = cvt_e4m3_byte(plain ? sixth(aG) : __fdiv_rn(aG, 6.0f));
+    const float r = table ? table[sb & 127u] : nv_ratio(sb, G);
     uint32_t w[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -465,11 +483,13 @@ __device__ __forceinline__ void nv_code_chunk(const uint32_t (&raw)[kLoads][8], 
 }
 
 // ---------------------------------------------------------------- NVFP4 pass 2, blocks of 16 along d (Q, K)
-// Bound by HBM (twice over the tensor, less what is left of it in L2) and by the two IEEE divisions per block.  67 M elements,
-// both passes: 50.6 us; with a kernel of its own for the factor, a block's scale formed in two lanes and plain launches 61.6.
+// Bound by HBM (twice over the tensor, less what is left of it in L2); where L2 holds the tensor, by its instructions.  67 M
+// elements, both passes: 48.9 us (two IEEE divisions per block: 49.5; with a kernel of its own for the factor, a block's scale
+// formed in two lanes and plain launches 61.6), 8.4 M 9.0 (9.3).
 // The chunks and the grid of quant_mx_rows_kernel, walked from the tensor's end (the amax pass has read that last).  A chunk
-// lies within one unit; `chunks_per_unit` is 0 when the tensor has one factor, else a CTA forms its unit's for every chunk.
-template <int D, bool W32>
+// lies within one unit; where units have factors of their own a CTA forms its unit's for every chunk.
+// UNITS: one factor per unit.
+template <int D, bool W32, bool UNITS>
 __global__ void __launch_bounds__(kThreads, kRowsCtas)
 quant_nv_rows_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, uint8_t* __restrict__ sf,
                      const float* __restrict__ partials, int n_partials, float* __restrict__ G_out, uint32_t n_chunks,
@@ -479,10 +499,12 @@ quant_nv_rows_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, ui
   uint32_t i = blockIdx.x, raw[kLoads][8];
 #pragma unroll
   for (int k = 0; k < kLoads; ++k) load_16<W32>(raw[k], x + (size_t)(n_chunks - 1 - i) * kGroupsPerCta + 2 * (threadIdx.x + k * kThreads));
+  __shared__ float ratio[128];
   float G = 0.f;
-  if (!chunks_per_unit) {
+  if (!UNITS) {
     G = encode_factor_block(partials, n_partials, 2688.0f);
     if (blockIdx.x == 0 && threadIdx.x == 0) G_out[0] = G;
+    nv_ratio_table(ratio, G);
   }
   while (true) {
     const uint32_t chunk = n_chunks - 1 - i;
@@ -492,12 +514,12 @@ quant_nv_rows_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, ui
 #pragma unroll
       for (int k = 0; k < kLoads; ++k) load_16<W32>(ahead[k], x + (size_t)(n_chunks - 1 - i) * kGroupsPerCta + 2 * (threadIdx.x + k * kThreads));
     }
-    if (chunks_per_unit) {
+    if (UNITS) {
       const uint32_t unit = chunk / chunks_per_unit;
       G = encode_factor_warp(partials + (size_t)unit * n_partials, n_partials, 2688.0f);
       if (threadIdx.x == 0 && unit * chunks_per_unit == chunk) G_out[unit] = G;
     }
-    nv_code_chunk<D>(raw, G, chunk, packed, sf);
+    nv_code_chunk<D>(raw, G, UNITS ? nullptr : ratio, chunk, packed, sf);
     if (i >= n_chunks) return;
 #pragma unroll
     for (int k = 0; k < kLoads; ++k)
@@ -509,7 +531,9 @@ quant_nv_rows_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, ui
 // Both passes over a unit with a factor of its own in one launch: a cluster takes the unit, its CTAs every cluster_size()-th
 // chunk, and the second pass runs from the last chunk back.  Units of up to 1 MB are still in L2 then (the resident clusters
 // hold 74 MB of them), so the tensor is read from memory once; of larger ones the part that is.  All resident clusters
-// read, meet and write at about the same time: 64 units of 1 MB take 25 us, 3.5 TB/s of input and output.
+// read, meet and write at about the same time, and the second half is bound by instructions: 64 units of 1 MB take 23.4 us (two
+// divisions per block instead of a table of ratios and sixth(): 24.6), 3.7 TB/s of input and output.  (Held in shared memory for
+// the second pass by one CTA of 512 threads per SM: 32.8 us, its sixteen warps are too few for the conversion's latency.)
 template <int D, bool W32>
 __global__ void __launch_bounds__(kThreads, kRowsCtas)
 quant_nv_unit_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, uint8_t* __restrict__ sf, float* __restrict__ G_out,
@@ -539,10 +563,12 @@ quant_nv_unit_kernel(const uint4* __restrict__ x, uint2* __restrict__ packed, ui
   }
   const float G = encode_factor_of(__uint_as_float(cluster_max<kThreads>(m) << 16), 2688.0f);
   if (rank == 0 && threadIdx.x == 0) G_out[unit] = G;
+  __shared__ float ratio[128];
+  nv_ratio_table(ratio, G);
   for (int c = mine - 1; c >= 0; --c) {                           // the last chunk is still in registers
     uint32_t ahead[kLoads][8];
     if (c > 0) load(c - 1, ahead);
-    nv_code_chunk<D>(raw, G, (uint32_t)(first + rank + c * step), packed, sf);
+    nv_code_chunk<D>(raw, G, ratio, (uint32_t)(first + rank + c * step), packed, sf);
     if (c > 0) {
 #pragma unroll
       for (int k = 0; k < kLoads; ++k)
@@ -687,8 +713,11 @@ int launch_quantize(const void* x, int fmt, int role, int B, int H, int N, int d
     const bool w32 = ((uintptr_t)xs & 31) == 0;
     launch_overlapped(w32 ? amax_partials_kernel<true> : amax_partials_kernel<false>, per_head ? dim3(n_partials, B * H) : dim3(n_partials), kThreads, 0, st, xs,
                       per_head ? n_groups / ((size_t)B * H) : n_groups, partials);
-    launch_overlapped(d == 128 ? (w32 ? quant_nv_rows_kernel<128, true> : quant_nv_rows_kernel<128, false>)
-                               : (w32 ? quant_nv_rows_kernel<64, true> : quant_nv_rows_kernel<64, false>), dim3(rows_grid(n_chunks)), kThreads, 0, st, xs,
+    auto rows = per_head ? (d == 128 ? (w32 ? quant_nv_rows_kernel<128, true, true> : quant_nv_rows_kernel<128, false, true>)
+                                     : (w32 ? quant_nv_rows_kernel<64, true, true> : quant_nv_rows_kernel<64, false, true>))
+                         : (d == 128 ? (w32 ? quant_nv_rows_kernel<128, true, false> : quant_nv_rows_kernel<128, false, false>)
+                                     : (w32 ? quant_nv_rows_kernel<64, true, false> : quant_nv_rows_kernel<64, false, false>));
+    launch_overlapped(rows, dim3(rows_grid(n_chunks)), kThreads, 0, st, xs,
                       (uint2*)packed, (uint8_t*)scales, (const float*)partials, n_partials, G_out, (uint32_t)n_chunks,
                       (uint32_t)(per_head ? unit_chunks : 0));
   }

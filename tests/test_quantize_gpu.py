@@ -246,6 +246,20 @@ def test_nvfp4_one_launch_and_two_launch_sizes(B, H, N, d, offset):
     _check_operand(Bd.fp4attn_quantize(t, Bd.FMT_NVFP4, Bd.ROLE_K), Qz.quantize_qk(bits, "nv"), Bd.ROLE_K)
 
 
+@pytest.mark.parametrize("exponent", [60, 0, -85, -95, -110])        # encode factors of 2^-51 ... 2^119; from 2^100 on a block's scale is divided for
+@pytest.mark.parametrize("kw", [dict(B=1, H=2, N=128, d=64), dict(B=1, H=20, N=2048)])     # one launch, two launches
+def test_nvfp4_of_very_small_and_large_tensors_matches_oracle(exponent, kw):
+    from paper_2609_04105_b200 import binding as Bd
+    w = I.shrink(I.WORKLOADS["cfg1"], **kw)
+    q, _, _ = I.make_qkv(w)
+    bits = I.f32_to_bf16_bits(np.ldexp(I.bf16_bits_to_f32(q), exponent))
+    _check_operand(Bd.fp4attn_quantize(_dev(bits), Bd.FMT_NVFP4, Bd.ROLE_Q), Qz.quantize_qk(bits, "nv"), Bd.ROLE_Q)
+    got, want = Bd.fp4attn_quantize_nvfp4_per_head(_dev(bits), Bd.ROLE_Q), Qz.quantize_qk(bits, "nv", per_head=True)
+    assert np.array_equal(got.G.cpu().numpy().reshape(w.B, w.H), want["G"])
+    assert np.array_equal(Qz.strip_negative_zero(got.packed.cpu().numpy()), Qz.strip_negative_zero(Qz.pack_nibbles(want["nib"]).reshape(-1)))
+    assert np.array_equal(got.scales.cpu().numpy(), Qz.swizzle_scales(want["sf"]).reshape(-1))
+
+
 def test_quantizers_take_whole_numbers_and_tensors_only():
     from paper_2609_04105_b200 import binding as Bd
     x = torch.zeros((1, 1, 128, 64), dtype=torch.bfloat16, device="cuda")
