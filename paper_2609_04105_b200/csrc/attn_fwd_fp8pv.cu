@@ -16,8 +16,8 @@
 // and the first sweep of the CTA's next item run interleaved stage by stage (see the schedule comment in the
 // kernel), so that SFU-heavy and SFU-free visits alternate on every team.
 //
-//   warp 0        TMA producer: Q tile per item; ring of {K, K scales} for A-steps and {K, V8^T, K scales} for B-steps
-//   warp 1        QK issuer (both kinds of step; after an A-step it also hands the ring slot back)
+//   warp 0        TMA producer: Q tile per item; a ring of {K, K scales} for all steps and one of V8^T for B-steps
+//   warp 1        QK issuer (both kinds of step)
 //   warp 2        PV issuer (B-steps): four K32 products per 128-key stage, A operand from tensor memory
 //   warps 3-6     epilogue: O = O_hw / (L_hw G_V), LSE
 //   warps 7-22    softmax teams as in attn_fwd.cu (team 2p + h: h-th 64 keys of the steps with parity p)
@@ -38,19 +38,25 @@ struct Cfg8 {
   using C1 = Cfg<D, NV>;
   static constexpr int V_BYTES = D * BS;                              // V8^T: d rows x 128 bytes
   static constexpr int ONES_BYTES = kOnesRows * BS;                   // rows of E4M3 1.0
-  static constexpr int OFF_KSF = C1::K_BYTES + V_BYTES + ONES_BYTES;  // within a stage
-  static constexpr int STAGE_BYTES = (OFF_KSF + C1::KSF_BYTES + 1023) / 1024 * 1024;
-  static constexpr int NST = (D == 128) ? 5 : 8;                      // d = 128, N = 8192: 3 / 4 / 5 / 6 slots 1177 / 923 / 752 / 742 us, causal (6) 4 % longer
+  // Two rings: a slot of K is handed back by the score product, one of V8^T by the PV product some two steps later, and only
+  // every other step needs V.  Attention alone (B=2, H=16, N=8192, d=128 | causal | d=64 | B=16, H=16, N=1024, d=128), us: one
+  // ring of 5 slots (d=64: 8) 749 | 402 | 719 | 110; K and V slots 8 and 4 736 | 396 | 717 | 102; 8 and 3 723 | 397 | 704 |
+  // 104; 4 and 3 723 | 398 | - | 104; 8 and 5 736; 8 and 2 902 | 480 | 853 | 120.
+  static constexpr int KST_BYTES = (C1::K_BYTES + C1::KSF_BYTES + 1023) / 1024 * 1024;   // K, K scales
+  static constexpr int VST_BYTES = V_BYTES + ONES_BYTES;
+  static constexpr int KST = 8, VST = 3;
   static constexpr int OFF_Q = 0;                                     // two buffers
   static constexpr int OFF_QSF = OFF_Q + 2 * C1::Q_BYTES;             // two buffers of 1 KB
   static constexpr int OFF_RMAX = OFF_QSF + 2048;                     // [item parity][first-sweep team][row] float
   static constexpr int OFF_MU = OFF_RMAX + 2 * 4 * BM * 4;            // [item parity][row] int
-  static constexpr int OFF_STAGE = (OFF_MU + 2 * BM * 4 + 1023) / 1024 * 1024;
-  static constexpr int OFF_OUT = OFF_STAGE + NST * STAGE_BYTES;
+  static constexpr int OFF_K = (OFF_MU + 2 * BM * 4 + 1023) / 1024 * 1024;
+  static constexpr int OFF_V = OFF_K + KST * KST_BYTES;
+  static constexpr int OFF_OUT = OFF_V + VST * VST_BYTES;
   static constexpr int OFF_BAR = OFF_OUT + C1::OUT_BYTES;
   static constexpr int OFF_SEQ = OFF_BAR + 1024;                      // SeqTable
-  static constexpr int SMEM_BYTES = OFF_SEQ + 1536 + 1024;
-  static_assert(OFF_STAGE % 1024 == 0 && OFF_OUT % 1024 == 0 && SMEM_BYTES <= 227 * 1024, "shared memory");
+  static constexpr int OFF_ITEMS = OFF_SEQ + 1536;                    // item table
+  static constexpr int SMEM_BYTES = OFF_ITEMS + kItemTable * 32 + 1024;
+  static_assert(OFF_K % 1024 == 0 && OFF_V % 1024 == 0 && OFF_OUT % 1024 == 0 && SMEM_BYTES <= 227 * 1024, "shared memory");
 };
 
 enum { B8_QFULL0 = 0, B8_QFREE0 = 2, B8_OFULL = 4, B8_OFREE = 5, B8_SFULL0 = 6, B8_SEMPTY0 = 8, B8_PFREE0 = 10,
@@ -115,8 +121,10 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   const uint32_t abort_at = sbase + C8::OFF_BAR + 776;
   volatile int* abortf = reinterpret_cast<volatile int*>(sgen + C8::OFF_BAR + 776);
   auto bar = [&](int i) { return sbase + C8::OFF_BAR + 8u * i; };
-  auto bar_full = [&](int s) { return bar(B8_RING + s); };
-  auto bar_empty = [&](int s) { return bar(B8_RING + C8::NST + s); };
+  auto k_full = [&](int s) { return bar(B8_RING + s); };
+  auto k_empty = [&](int s) { return bar(B8_RING + C8::KST + s); };
+  auto v_full = [&](int s) { return bar(B8_RING + 2 * C8::KST + s); };
+  auto v_empty = [&](int s) { return bar(B8_RING + 2 * C8::KST + C8::VST + s); };
   constexpr uint64_t kDescSF = (uint64_t)(16 >> 4) << 16 | (uint64_t)(128 >> 4) << 32 | 1ull << 46;
   constexpr uint64_t kDescQK = (uint64_t)(16 >> 4) << 16 | (uint64_t)((8 * C::ROW_BYTES) >> 4) << 32 | 1ull << 46 | C::SWZ_QK << 61;
   constexpr uint64_t kDescV = (uint64_t)(16 >> 4) << 16 | (uint64_t)(1024 >> 4) << 32 | 1ull << 46 | kSwz128 << 61;   // 128-byte rows
@@ -137,7 +145,8 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     }
     mbar_init(bar(B8_OFULL), 1);
     mbar_init(bar(B8_OFREE), 4);
-    for (int s = 0; s < C8::NST; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
+    for (int s = 0; s < C8::KST; ++s) { mbar_init(k_full(s), 1); mbar_init(k_empty(s), 1); }
+    for (int s = 0; s < C8::VST; ++s) { mbar_init(v_full(s), 1); mbar_init(v_empty(s), 1); }
     *abortf = 0;
     fence_barrier_init();
     prefetch_tensormap(&tmQ);
@@ -147,8 +156,8 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   }
   if (warp == 1) { tmem_alloc(sbase + C8::OFF_BAR + 768, kTmemCols); tmem_relinquish(); }
   // constant operand rows: E4M3 1.0 (0x38) in every byte
-  for (int i = threadIdx.x; i < C8::NST * (C8::ONES_BYTES / 4); i += kAttnThreads)
-    reinterpret_cast<uint32_t*>(sgen + C8::OFF_STAGE + (i / (C8::ONES_BYTES / 4)) * C8::STAGE_BYTES + C::K_BYTES + C8::V_BYTES)[i % (C8::ONES_BYTES / 4)] = 0x38383838u;
+  for (int i = threadIdx.x; i < C8::VST * (C8::ONES_BYTES / 4); i += kAttnThreads)
+    reinterpret_cast<uint32_t*>(sgen + C8::OFF_V + (i / (C8::ONES_BYTES / 4)) * C8::VST_BYTES + C8::V_BYTES)[i % (C8::ONES_BYTES / 4)] = 0x38383838u;
   fence_proxy_async_smem();
   tc_fence_before();
   __syncthreads();
@@ -161,6 +170,9 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     fill_skipped<D>(seq, p, qtiles);
   }
   const int n_my = items_of_cta<CAUSAL>(CAUSAL && p.sorted ? seq->first[p.B] : p.n_items);   // this CTA's items: item_at(0 .. n_my - 1)
+  ItemRec* const tab = reinterpret_cast<ItemRec*>(sgen + C8::OFF_ITEMS);
+  if (CAUSAL) build_item_table<true, false>(tab, n_my, p, qtiles, seq);
+  auto work = [&](int i) { return CAUSAL ? item_of_cta<true>(i, tab, p, qtiles, seq) : decode_item<false>(item_at<false>(i), p, qtiles, seq); };
 
   // Every role walks the same schedule.  Phase ph (0 .. n_my) carries the first sweep ("A": scores -> row maxima) of
   // item ph and the second sweep ("B": scores -> bytes -> PV) of item ph - 1, stage by stage, in the order
@@ -170,15 +182,13 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   // warps of a scheduler are never all in the same kind of work.
   if (warp == 0) {
     // ===================================================================== TMA producer
-    int s = 0, ph = 0;
-    uint32_t gs = 0;
-    uint32_t st = sbase + C8::OFF_STAGE;
+    int s = 0, ph = 0, sv = 0, phv = 0;
     bool ok = true;
     for (int phs = 0; ok && phs <= n_my; ++phs) {
       WorkItem wa = {}, wb = {};
       int TA = 0, TB = 0;
-      if (phs < n_my) { wa = decode_item<CAUSAL>(item_at<CAUSAL>(phs), p, qtiles, seq); TA = wa.T2; }
-      if (phs >= 1) { wb = decode_item<CAUSAL>(item_at<CAUSAL>(phs - 1), p, qtiles, seq); TB = wb.T2; }
+      if (phs < n_my) { wa = work(phs); TA = wa.T2; }
+      if (phs >= 1) { wb = work(phs - 1); TB = wb.T2; }
       if (phs < n_my) {
         const int qb = phs & 1;
         if (phs >= 2) ok = mbar_wait<false>(bar(B8_QFREE0 + qb), ((phs >> 1) - 1) & 1, abort_at);
@@ -196,24 +206,29 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           const int kind = j ^ (s2 & 1);                            // 0: A-step of item phs, 1: B-step of item phs - 1
           if (s2 >= (kind ? TB : TA)) continue;
           const WorkItem& wi = kind ? wb : wa;
-          if (gs >= (uint32_t)C8::NST) ok = mbar_wait<false>(bar_empty(s), ph ^ 1, abort_at);
+          ok = mbar_wait<false>(k_empty(s), ph ^ 1, abort_at);      // (a fresh barrier passes)
+          if (ok && kind) ok = mbar_wait<false>(v_empty(sv), phv ^ 1, abort_at);
           if (!ok) break;
-          const uint32_t fb = bar_full(s);
+          const uint32_t fb = k_full(s), st = sbase + C8::OFF_K + s * C8::KST_BYTES;
           if (elect_one()) {
-            mbar_arrive_expect_tx(fb, C::K_BYTES + C::KSF_BYTES + (kind ? C8::V_BYTES : 0));
+            mbar_arrive_expect_tx(fb, C::K_BYTES + C::KSF_BYTES);
             tma_load_2d(st, &tmK, 0, wi.kvh * p.N + s2 * BS, fb);
-            if (kind) tma_load_2d(st + C::K_BYTES, &tmV, s2 * BS, wi.kvh * D, fb);
-            bulk_load_1d(st + C8::OFF_KSF, p.k_sf + ((size_t)wi.kvh * qtiles + s2) * C::KSF_BYTES, C::KSF_BYTES, fb);
+            bulk_load_1d(st + C::K_BYTES, p.k_sf + ((size_t)wi.kvh * qtiles + s2) * C::KSF_BYTES, C::KSF_BYTES, fb);
+            if (kind) {
+              mbar_arrive_expect_tx(v_full(sv), C8::V_BYTES);
+              tma_load_2d(sbase + C8::OFF_V + sv * C8::VST_BYTES, &tmV, s2 * BS, wi.kvh * D, v_full(sv));
+            }
           }
-          ++gs;
-          st += C8::STAGE_BYTES;
-          if (++s == C8::NST) { s = 0; ph ^= 1; st = sbase + C8::OFF_STAGE; }
+          if (++s == C8::KST) { s = 0; ph ^= 1; }
+          if (kind && ++sv == C8::VST) { sv = 0; phv ^= 1; }
         }
       }
     }
     if (*abortf && lane == 0) {
-      for (int r = 0; r < C8::NST; ++r)
-        for (int spin = 0; spin < (1 << 12) && !mbar_try_wait(bar_full(r), 0) && !mbar_try_wait(bar_full(r), 1); ++spin) {}
+      for (int r = 0; r < C8::KST; ++r)
+        for (int spin = 0; spin < (1 << 12) && !mbar_try_wait(k_full(r), 0) && !mbar_try_wait(k_full(r), 1); ++spin) {}
+      for (int r = 0; r < C8::VST; ++r)
+        for (int spin = 0; spin < (1 << 12) && !mbar_try_wait(v_full(r), 0) && !mbar_try_wait(v_full(r), 1); ++spin) {}
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -221,13 +236,13 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     constexpr uint32_t kIdQK0 = NV ? make_idesc_fp4(BM, BS, false, 0, 0) : make_idesc_fp4(BM, BS, true, 0, 0);
     constexpr uint32_t kIdQK1 = NV ? make_idesc_fp4(BM, BS, false, 0, 0) : make_idesc_fp4(BM, BS, true, 2, 2);
     int sq = 0, phq = 0;
-    uint32_t stq = sbase + C8::OFF_STAGE;
+    uint32_t stq = sbase + C8::OFF_K;
     uint32_t g = 0;                                             // steps issued so far (both kinds, all items)
     bool ok = true;
     for (int phs = 0; ok && phs <= n_my; ++phs) {
       int TA = 0, TB = 0;
-      if (phs < n_my) TA = decode_item<CAUSAL>(item_at<CAUSAL>(phs), p, qtiles, seq).T2;
-      if (phs >= 1) TB = decode_item<CAUSAL>(item_at<CAUSAL>(phs - 1), p, qtiles, seq).T2;
+      if (phs < n_my) TA = work(phs).T2;
+      if (phs >= 1) TB = work(phs - 1).T2;
       if (phs < n_my) {
         const int qb = phs & 1;
         ok = mbar_wait<false>(bar(B8_QFULL0 + qb), (phs >> 1) & 1, abort_at);
@@ -249,7 +264,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           const int qb = (kind ? phs - 1 : phs) & 1;              // the Q buffer of the step's item
           const int pr = g & 1;
           const uint32_t m = g >> 1;
-          ok = mbar_wait<false>(bar_full(sq), phq, abort_at);
+          ok = mbar_wait<false>(k_full(sq), phq, abort_at);
           if (ok && m > 0) ok = mbar_wait<false>(bar(B8_SEMPTY0 + pr), (m - 1) & 1, abort_at);   // both teams have read the slot
           if (!ok) break;
           tc_fence_after();
@@ -260,7 +275,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           const uint64_t dK0 = at(kDescQK, stq);
           if (elect_one()) {
 #pragma unroll
-            for (int a = 0; a < C::CTQ; ++a) tc_cp_32x128b_warpx4(tSFK + 4 * a, at(kDescSF, stq + C8::OFF_KSF + 512 * a));
+            for (int a = 0; a < C::CTQ; ++a) tc_cp_32x128b_warpx4(tSFK + 4 * a, at(kDescSF, stq + C::K_BYTES + 512 * a));
             if (NV) {
               tc_mma_fp4_4x(tS, dQ0, dK0, kIdQK0, tSFQ, tSFK, 0);
               if (C::KBLK == 2) tc_mma_fp4_4x(tS, dQ0 + 2, dK0 + 2, kIdQK1, tSFQ + 4, tSFK + 4, 1);
@@ -269,13 +284,13 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
               if (C::KBLK == 2) tc_mma_fp4_2x(tS, dQ0 + 2, dK0 + 2, kIdQK1, tSFQ, tSFK, 1);
             }
             tc_commit(bar(B8_SFULL0 + pr));
-            if (kind == 0) tc_commit(bar_empty(sq));              // first sweep: nothing else reads the stage
+            tc_commit(k_empty(sq));                               // K back to the producer
             if (kind == 1 && s2 == TB - 1) tc_commit(bar(B8_QFREE0 + qb));   // the item's Q buffer may take the item after next
           }
           __syncwarp();
           ++g;
-          stq += C8::STAGE_BYTES;
-          if (++sq == C8::NST) { sq = 0; phq ^= 1; stq = sbase + C8::OFF_STAGE; }
+          stq += C8::KST_BYTES;
+          if (++sq == C8::KST) { sq = 0; phq ^= 1; stq = sbase + C8::OFF_K; }
         }
       }
     }
@@ -285,13 +300,14 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     // ===================================================================== PV issuer (B-steps)
     constexpr uint32_t kIdPV = make_idesc_f8(BM, C::DN);
     const uint32_t tO = tmem + kColO;
-    uint32_t g = 0;                                             // steps so far (both kinds): ring slot and team pair of a step
+    uint32_t g = 0;                                             // steps so far (both kinds): team pair of a step
+    int sv = 0, phv = 0;
     uint32_t nb[2] = {0, 0};                                    // B-steps served so far, per team pair
     bool ok = true;
     for (int phs = 0; ok && phs <= n_my; ++phs) {
       int TA = 0, TB = 0;
-      if (phs < n_my) TA = decode_item<CAUSAL>(item_at<CAUSAL>(phs), p, qtiles, seq).T2;
-      if (phs >= 1) TB = decode_item<CAUSAL>(item_at<CAUSAL>(phs - 1), p, qtiles, seq).T2;
+      if (phs < n_my) TA = work(phs).T2;
+      if (phs >= 1) TB = work(phs - 1).T2;
       if (phs >= 2) ok = mbar_wait<false>(bar(B8_OFREE), (phs - 2) & 1, abort_at);   // epilogue of item phs - 2 has read O
       const int TM = TA > TB ? TA : TB;
       for (int s2 = 0; ok && s2 < TM; ++s2) {
@@ -302,22 +318,22 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           if (kind == 0) { ++g; continue; }                       // an A-step: only its slot is counted
           const int pr = g & 1;
           ok = mbar_wait<false>(bar(B8_SMDONE0 + pr), (pr ? nb[1] : nb[0]) & 1, abort_at);   // bytes of both tiles are in tensor memory
+          if (ok) ok = mbar_wait<false>(v_full(sv), phv, abort_at);
           if (!ok) break;
           if (pr) ++nb[1]; else ++nb[0];
           tc_fence_after();
-          const uint32_t sp = g % C8::NST;
-          const uint32_t stp = sbase + C8::OFF_STAGE + sp * C8::STAGE_BYTES;
-          const uint64_t dV = at(kDescV, stp + C::K_BYTES);
+          const uint64_t dV = at(kDescV, sbase + C8::OFF_V + sv * C8::VST_BYTES);
           if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)                         // 32 keys per product: 8 columns of P, 32 bytes along V8^T's rows
               tc_mma_f8_ta(tO, tmem + k8ColP + 32 * pr + 8 * kk, dV + 2 * kk, kIdPV, (s2 > 0 || kk > 0) ? 1u : 0u);
-            tc_commit(bar_empty(sp));
+            tc_commit(v_empty(sv));                               // V back to the producer
             tc_commit(bar(B8_PFREE0 + pr));
             if (s2 == TB - 1) tc_commit(bar(B8_OFULL));
           }
           __syncwarp();
           ++g;
+          if (++sv == C8::VST) { sv = 0; phv ^= 1; }
         }
       }
     }
@@ -330,7 +346,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const uint32_t tO = tmem + ((uint32_t)(quarter * 32) << 16) + kColO;
     bool ok = true;
     for (int k = 0; ok && k < n_my; ++k) {
-      const WorkItem wi = decode_item<CAUSAL>(item_at<CAUSAL>(k), p, qtiles, seq);
+      const WorkItem wi = work(k);
       ok = mbar_wait<false>(bar(B8_OFULL), k & 1, abort_at);
       if (!ok) break;
       tc_fence_after();
@@ -408,8 +424,8 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     for (int phs = 0; ok && phs <= n_my; ++phs) {
       WorkItem wa = {}, wb = {};
       int TA = 0, TB = 0;
-      if (phs < n_my) { wa = decode_item<CAUSAL>(item_at<CAUSAL>(phs), p, qtiles, seq); TA = wa.T2; }
-      if (phs >= 1) { wb = decode_item<CAUSAL>(item_at<CAUSAL>(phs - 1), p, qtiles, seq); TB = wb.T2; }
+      if (phs < n_my) { wa = work(phs); TA = wa.T2; }
+      if (phs >= 1) { wb = work(phs - 1); TB = wb.T2; }
       const int va = CAUSAL ? tile_keys(wa) : 64, vb = CAUSAL ? tile_keys(wb) : 64;
       float smax = -INFINITY;                                   // this team's share of the maxima of item phs
       const int TM = TA > TB ? TA : TB;

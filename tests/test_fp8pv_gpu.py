@@ -152,6 +152,27 @@ def test_fp8_pv_padded_sequences_match_oracle_on_the_rows_that_exist(name, kw, l
     assert torch.equal(O1, O2) and torch.equal(L1, L2)           # full lengths: the bits of the call without seq_len
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("N,causal", [(128, False), (384, True), (1152, False)])
+def test_rings_carry_over_from_item_to_item(N, causal, d):
+    """300 to 450 items, up to four a CTA, of one to nine stages: the rings of K and of V wrap at different stages of every item.
+    The bits are those of each head alone, whose CTAs take one item each."""
+    from paper_2609_04105_b200 import binding as Bd
+    H = {128: 450, 384: 150, 1152: 40}[N]
+    w = I.shrink(I.WORKLOADS["cfg1"], H=H, N=N, d=d)
+    q, k, v = (_dev(t) for t in I.make_qkv(w))
+
+    def run(h):
+        x = [t[:, h].contiguous() for t in (q, k, v)]
+        return Bd.fp4attn_fwd(Bd.fp4attn_quantize(x[0], 0, Bd.ROLE_Q), Bd.fp4attn_quantize(x[1], 0, Bd.ROLE_K), Bd.fp4attn_quantize_v_e4m3(x[2]),
+                              causal=causal)
+
+    O, L = run(slice(0, H))
+    for h in (0, 1, H // 2, H - 1):
+        O1, L1 = run(slice(h, h + 1))
+        assert torch.equal(O[:, h], O1[:, 0]) and torch.equal(L[:, h], L1[:, 0]), h
+
+
 def test_fp8_pv_rejects_the_fp4_only_options():
     from paper_2609_04105_b200 import binding as Bd
     w = I.shrink(I.WORKLOADS["cfg1"], N=128)
