@@ -169,7 +169,7 @@ __device__ __forceinline__ void fill_skipped(const SeqTable* st, const AttnParam
     const int r = seq_segment(st->skipped, j), n = qtiles - st->T[r], rem = j - st->skipped[r], h = rem / n;
     const size_t row0 = ((size_t)st->b[r] * p.H + h) * p.N + (size_t)(st->T[r] + rem - h * n) * BM;
     uint4* o = reinterpret_cast<uint4*>(p.O + row0 * D);
-    for (int k = threadIdx.x; k < BM * D / 8; k += kAttnThreads) o[k] = make_uint4(0u, 0u, 0u, 0u);
+    for (int k = threadIdx.x; k < BM * D / 8; k += blockDim.x) o[k] = make_uint4(0u, 0u, 0u, 0u);
     if (p.LSE && threadIdx.x < BM) p.LSE[row0 + threadIdx.x] = 0.f;
   }
 }
@@ -262,7 +262,7 @@ __device__ __forceinline__ float unit_score_constant(const AttnParams& p, const 
 // all threads; ends with a barrier
 template <bool MASKED, bool UNIT_CONSTANT>
 __device__ __forceinline__ void build_item_table(ItemRec* tab, int n_my, const AttnParams& p, int qtiles, const SeqTable* st) {
-  for (int i = threadIdx.x >> 5; i < min(n_my, kItemTable); i += kAttnThreads / 32) {
+  for (int i = threadIdx.x >> 5; i < min(n_my, kItemTable); i += (int)blockDim.x / 32) {
     ItemRec r;
     r.w = decode_item<MASKED>(item_at<MASKED>(i), p, qtiles, st);
     r.c = UNIT_CONSTANT ? unit_score_constant(p, r.w) : 0.f;

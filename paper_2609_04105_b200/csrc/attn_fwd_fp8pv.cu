@@ -17,20 +17,20 @@
 // kernel), so that SFU-heavy and SFU-free visits alternate on every team.
 //
 //   warp 0        TMA producer: Q tile per item; a ring of {K, K scales} for all steps and one of V8^T for B-steps
-//   warp 1        QK issuer (both kinds of step)
+//   warps 1, 23   QK issuers (both kinds of step), one per team pair
 //   warp 2        PV issuer (B-steps): four K32 products per 128-key stage, A operand from tensor memory
 //   warps 3-6     epilogue: O = O_hw / (L_hw G_V), LSE
 //   warps 7-22    softmax teams as in attn_fwd.cu (team 2p + h: h-th 64 keys of the steps with parity p)
 //
 // The row sum is column d of the accumulator: sixteen rows of E4M3 1.0 follow V8^T in every stage.
 // Tensor memory: S slots 0..255 | O 256..399 | Q scales 400..415 | K scales 416..431 | P bytes 432..495 (per step
-// parity 32 columns: 128 keys x 8 bits per row).
+// parity 32 columns: 128 keys x 8 bits per row) | Q scales of the second QK issuer 496..511.
 #include "attn_common.cuh"
 
 namespace fp4attn {
 using namespace ptx;
 
-constexpr uint32_t k8ColP = 432;
+constexpr uint32_t k8ColP = 432, k8ColSFQ1 = 496;
 constexpr float kP8Shift = 8.0f;
 
 template <int D, bool NV>
@@ -39,12 +39,12 @@ struct Cfg8 {
   static constexpr int V_BYTES = D * BS;                              // V8^T: d rows x 128 bytes
   static constexpr int ONES_BYTES = kOnesRows * BS;                   // rows of E4M3 1.0
   // Two rings: a slot of K is handed back by the score product, one of V8^T by the PV product some two steps later, and only
-  // every other step needs V.  Attention alone (B=2, H=16, N=8192, d=128 | causal | d=64 | B=16, H=16, N=1024, d=128), us: one
-  // ring of 5 slots (d=64: 8) 749 | 402 | 719 | 110; K and V slots 8 and 4 736 | 396 | 717 | 102; 8 and 3 723 | 397 | 704 |
-  // 104; 4 and 3 723 | 398 | - | 104; 8 and 5 736; 8 and 2 902 | 480 | 853 | 120.
+  // every other step needs V.  Attention alone, us, d=128 N=8192 | d=128 N=1024 | causal N=8192 | d=64 N=8192: one ring of 5 slots
+  // (d=64: 8) 748 | 110 | 402 | 718, K and V slots 8 and 3 722 | 104 | 397 | 703.  With the issuers and visits as they are now: V
+  // slots 3 680 | 104 | 381 | 646, 4 682 | 97 | 381 | 679; K slots 4, 6, 8 686, 684, 680; a third Q buffer 690 | 95 | 379 | 646.
   static constexpr int KST_BYTES = (C1::K_BYTES + C1::KSF_BYTES + 1023) / 1024 * 1024;   // K, K scales
   static constexpr int VST_BYTES = V_BYTES + ONES_BYTES;
-  static constexpr int KST = 8, VST = 3;
+  static constexpr int KST = 8, VST = (D == 128) ? 4 : 3;
   static constexpr int OFF_Q = 0;                                     // two buffers
   static constexpr int OFF_QSF = OFF_Q + 2 * C1::Q_BYTES;             // two buffers of 1 KB
   static constexpr int OFF_RMAX = OFF_QSF + 2048;                     // [item parity][first-sweep team][row] float
@@ -60,7 +60,7 @@ struct Cfg8 {
 };
 
 enum { B8_QFULL0 = 0, B8_QFREE0 = 2, B8_OFULL = 4, B8_OFREE = 5, B8_SFULL0 = 6, B8_SEMPTY0 = 8, B8_PFREE0 = 10,
-       B8_SMDONE0 = 12, B8_DRAIN0 = 14, B8_MURDY0 = 16, B8_RING = 18 };
+       B8_SMDONE0 = 12, B8_DRAIN0 = 14, B8_MURDY0 = 16, B8_DRAIN2 = 18, B8_RING = 19 };
 
 struct Fp8Params {
   AttnParams a;
@@ -106,8 +106,9 @@ __device__ __forceinline__ void fp8_p_block(const uint32_t* sraw, uint64_t c2, f
   }
 }
 
+constexpr int kFp8Threads = kAttnThreads + 32;                 // and the second QK issuer
 template <int D, int NV, bool CAUSAL>
-__global__ void __launch_bounds__(kAttnThreads, 1)
+__global__ void __launch_bounds__(kFp8Threads, 1)
 attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                       const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
                       const Fp8Params pp) {
@@ -135,7 +136,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   if (threadIdx.x == 0) {
     for (int b = 0; b < 2; ++b) {
       mbar_init(bar(B8_QFULL0 + b), 1);
-      mbar_init(bar(B8_QFREE0 + b), 1);
+      mbar_init(bar(B8_QFREE0 + b), 2);        // both QK issuers
       mbar_init(bar(B8_SFULL0 + b), 1);
       mbar_init(bar(B8_SEMPTY0 + b), 8);       // the two teams of the pair, four warps each
       mbar_init(bar(B8_SMDONE0 + b), 8);
@@ -143,6 +144,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       mbar_init(bar(B8_MURDY0 + b), 4 * kTeams);   // every softmax warp, once per item (slot by item parity)
       mbar_init(bar(B8_DRAIN0 + b), 1);
     }
+    mbar_init(bar(B8_DRAIN2), 1);
     mbar_init(bar(B8_OFULL), 1);
     mbar_init(bar(B8_OFREE), 4);
     for (int s = 0; s < C8::KST; ++s) { mbar_init(k_full(s), 1); mbar_init(k_empty(s), 1); }
@@ -156,7 +158,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   }
   if (warp == 1) { tmem_alloc(sbase + C8::OFF_BAR + 768, kTmemCols); tmem_relinquish(); }
   // constant operand rows: E4M3 1.0 (0x38) in every byte
-  for (int i = threadIdx.x; i < C8::VST * (C8::ONES_BYTES / 4); i += kAttnThreads)
+  for (int i = threadIdx.x; i < C8::VST * (C8::ONES_BYTES / 4); i += kFp8Threads)
     reinterpret_cast<uint32_t*>(sgen + C8::OFF_V + (i / (C8::ONES_BYTES / 4)) * C8::VST_BYTES + C8::V_BYTES)[i % (C8::ONES_BYTES / 4)] = 0x38383838u;
   fence_proxy_async_smem();
   tc_fence_before();
@@ -231,13 +233,20 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         for (int spin = 0; spin < (1 << 12) && !mbar_try_wait(v_full(r), 0) && !mbar_try_wait(v_full(r), 1); ++spin) {}
     }
     __syncwarp();
-  } else if (warp == 1) {
-    // ===================================================================== QK issuer (both sweeps)
+  } else if (warp == 1 || warp == kFirstSoftmaxWarp + 4 * kTeams) {
+    // ===================================================================== QK issuers (both sweeps), one for the steps of either team pair
+    // A pair waits for a score product after each of its A-visits, which are short, so what counts here is the time from the
+    // last read of a slot to the next product into it.  One warp for both pairs takes some 550 clocks from issue to issue and
+    // serves them in step order; two each wait for their own pair (the second on the scheduler that had no issuing warp).
+    // With the visits as they are below: 745 -> 680 us at d=128, N=8192, 706 -> 646 at d=64.
     constexpr uint32_t kIdQK0 = NV ? make_idesc_fp4(BM, BS, false, 0, 0) : make_idesc_fp4(BM, BS, true, 0, 0);
     constexpr uint32_t kIdQK1 = NV ? make_idesc_fp4(BM, BS, false, 0, 0) : make_idesc_fp4(BM, BS, true, 2, 2);
-    int sq = 0, phq = 0;
-    uint32_t stq = sbase + C8::OFF_K;
-    uint32_t g = 0;                                             // steps issued so far (both kinds, all items)
+    const int pr = warp == 1 ? 0 : 1;
+    static_assert(C8::KST % 2 == 0, "a ring slot's steps belong to one pair");
+    const uint32_t tSFK = tmem + kColSFK + 8 * pr, tS = tmem + kColS + BS * pr, tSFQ0 = tmem + (pr ? k8ColSFQ1 : kColSFQ);
+    int sq = pr, phq = 0;
+    uint32_t stq = sbase + C8::OFF_K + pr * C8::KST_BYTES;
+    uint32_t g = 0, m = 0;                                      // steps so far (both kinds, all items); of this warp's: issued so far
     bool ok = true;
     for (int phs = 0; ok && phs <= n_my; ++phs) {
       int TA = 0, TB = 0;
@@ -251,7 +260,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         if (elect_one()) {
 #pragma unroll
           for (int a = 0; a < C::CTQ; ++a)
-            tc_cp_32x128b_warpx4(tmem + kColSFQ + 8 * qb + 4 * a, at(kDescSF, sbase + C8::OFF_QSF + qb * 1024 + 512 * a));
+            tc_cp_32x128b_warpx4(tSFQ0 + 8 * qb + 4 * a, at(kDescSF, sbase + C8::OFF_QSF + qb * 1024 + 512 * a));
         }
         __syncwarp();
       }
@@ -261,16 +270,13 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         for (int j = 0; j < 2; ++j) {
           const int kind = j ^ (s2 & 1);
           if (s2 >= (kind ? TB : TA)) continue;
+          if ((int)(g & 1) != pr) { ++g; continue; }              // the other warp's step
           const int qb = (kind ? phs - 1 : phs) & 1;              // the Q buffer of the step's item
-          const int pr = g & 1;
-          const uint32_t m = g >> 1;
           ok = mbar_wait<false>(k_full(sq), phq, abort_at);
-          if (ok && m > 0) ok = mbar_wait<false>(bar(B8_SEMPTY0 + pr), (m - 1) & 1, abort_at);   // both teams have read the slot
+          if (ok) ok = mbar_wait<false>(bar(B8_SEMPTY0 + pr), (m & 1) ^ 1, abort_at);   // both teams have read the slot (a fresh barrier passes)
           if (!ok) break;
           tc_fence_after();
-          const uint32_t tSFQ = tmem + kColSFQ + 8 * qb;
-          const uint32_t tSFK = tmem + kColSFK + 8 * pr;
-          const uint32_t tS = tmem + kColS + BS * pr;
+          const uint32_t tSFQ = tSFQ0 + 8 * qb;
           const uint64_t dQ0 = at(kDescQK, sbase + C8::OFF_Q + qb * C::Q_BYTES);
           const uint64_t dK0 = at(kDescQK, stq);
           if (elect_one()) {
@@ -285,16 +291,20 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             }
             tc_commit(bar(B8_SFULL0 + pr));
             tc_commit(k_empty(sq));                               // K back to the producer
-            if (kind == 1 && s2 == TB - 1) tc_commit(bar(B8_QFREE0 + qb));   // the item's Q buffer may take the item after next
           }
           __syncwarp();
           ++g;
-          stq += C8::KST_BYTES;
-          if (++sq == C8::KST) { sq = 0; phq ^= 1; stq = sbase + C8::OFF_K; }
+          ++m;
+          stq += 2 * C8::KST_BYTES;
+          if ((sq += 2) >= C8::KST) { sq = pr; phq ^= 1; stq = sbase + C8::OFF_K + pr * C8::KST_BYTES; }
         }
       }
+      if (ok && phs >= 1) {                                       // this warp's products of item phs - 1 are issued: its Q buffer may take item phs + 1
+        if (elect_one()) tc_commit(bar(B8_QFREE0 + ((phs - 1) & 1)));
+        __syncwarp();
+      }
     }
-    if (*abortf && elect_one()) tc_commit(bar(B8_DRAIN0));
+    if (*abortf && elect_one()) tc_commit(bar(pr ? B8_DRAIN2 : B8_DRAIN0));
     __syncwarp();
   } else if (warp == 2) {
     // ===================================================================== PV issuer (B-steps)
@@ -428,6 +438,21 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       if (phs >= 1) { wb = work(phs - 1); TB = wb.T2; }
       const int va = CAUSAL ? tile_keys(wa) : 64, vb = CAUSAL ? tile_keys(wb) : 64;
       float smax = -INFINITY;                                   // this team's share of the maxima of item phs
+      auto first_sweep_step = [&](bool diag) {                  // scores of item phs: maxima only
+        uint32_t sraw[32];
+        tmem_ld_32x32b_x32(tS, sraw);
+        tmem_wait_ld();
+        if (diag) mask_scores(sraw, va);
+        smax = fmaxf(smax, max32(sraw));
+        tmem_ld_32x32b_x32(tS + 32, sraw);
+        tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sempty);
+        if (diag) mask_scores(sraw, va - 32);
+        smax = fmaxf(smax, max32(sraw));
+      };
+      bool swept = false;                                       // the pair's next A-step is done already
       const int TM = TA > TB ? TA : TB;
       for (int s2 = 0; ok && s2 < TM; ++s2) {
 #pragma unroll
@@ -435,27 +460,15 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           const int kind = j ^ (s2 & 1);
           if (s2 >= (kind ? TB : TA)) continue;
           if ((int)(g & 1) != pr) { ++g; continue; }              // the other pair's step
+          if (kind == 0 && swept) { swept = false; ++g; continue; }
           ok = mbar_wait<false>(sfull, (g >> 1) & 1, abort_at);
           if (!ok) break;
           tc_fence_after();
-          uint32_t sraw[32];
           if (kind == 0) {
-            // ---- first sweep of item phs: maxima only
-            const bool diag = CAUSAL && s2 == TA - 1;
-            tmem_ld_32x32b_x32(tS, sraw);
-            tmem_wait_ld();
-            if (diag) mask_scores(sraw, va);
-            smax = fmaxf(smax, max32(sraw));
-            tmem_ld_32x32b_x32(tS + 32, sraw);
-            tmem_wait_ld();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(sempty);
-            if (diag) mask_scores(sraw, va - 32);
-            smax = fmaxf(smax, max32(sraw));
+            first_sweep_step(CAUSAL && s2 == TA - 1);
           } else {
             // ---- second sweep of item phs - 1: bytes against its final reference
-            uint32_t w[16];
+            uint32_t sraw[32], w[8];
             const bool diag = CAUSAL && s2 == TB - 1;
             tmem_ld_32x32b_x32(tS, sraw);
             tmem_wait_ld();
@@ -466,12 +479,22 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(sempty);
-            fp8_p_block(sraw, c2, b, w + 8);
-            if (diag) mask_bytes(w + 8, vb - 32);
             // the pair's probability slot was last read by the PV product of this team's previous B-visit
             if (nbt > 0) ok = mbar_wait<false>(pfree, (nbt - 1) & 1, abort_at);
             if (!ok) break;
-            tmem_st_32x32b_x16(tP, w);
+            tmem_st_32x32b_x8(tP, w);
+            fp8_p_block(sraw, c2, b, w);
+            if (diag) mask_bytes(w, vb - 32);
+            // The pair's next step is an A-step, whose scores may be there by now: they are reduced first, so that the product
+            // after them, which the pair then waits for (580 of the 3080 clocks of an A- and a B-visit), starts a tail of this
+            // visit earlier: 686 -> 680 us, d=64 677 -> 646.  The first half's bytes are in tensor memory by then: with all
+            // sixteen words held the unmasked kernels spill 28 bytes and take 734 us.
+            if (s2 + 1 < min(TA, TB) && mbar_test(sfull, ((g >> 1) + 1) & 1)) {
+              tc_fence_after();
+              first_sweep_step(CAUSAL && s2 + 1 == TA - 1);
+              swept = true;
+            }
+            tmem_st_32x32b_x8(tP + 8, w);
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
@@ -503,8 +526,8 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   if (*abortf && threadIdx.x == 0 && p.status) *p.status = FP4ATTN_ERR_TIMEOUT;
   if (warp == 1) {
     if (*abortf && lane == 0) {
-      for (int r = 0; r < 2; ++r)
-        for (int spin = 0; spin < (1 << 14) && !mbar_try_wait(bar(B8_DRAIN0 + r), 0); ++spin) {}
+      for (int r = 0; r < 3; ++r)
+        for (int spin = 0; spin < (1 << 14) && !mbar_try_wait(bar(r == 2 ? B8_DRAIN2 : B8_DRAIN0 + r), 0); ++spin) {}
     }
     __syncwarp();
     tc_fence_after();
@@ -528,7 +551,7 @@ static int launch_fp8(const fp4attn_operands* ops, int B, int H, int N, const Fp
   const CUtensorMap* tm = attention_tensor_maps_fp8v(D, ops, prm.a.O, B, H, prm.a.Hkv, N);
   if (!tm) return FP4ATTN_ERR_CUDA;
   const unsigned grid = (unsigned)(prm.a.n_items < sms ? prm.a.n_items : sms);
-  launch_overlapped(attn_fwd_fp8pv_kernel<D, NV, CAUSAL>, dim3(grid), kAttnThreads, C8::SMEM_BYTES, st, tm[0], tm[1], tm[2], tm[3], prm);
+  launch_overlapped(attn_fwd_fp8pv_kernel<D, NV, CAUSAL>, dim3(grid), kFp8Threads, C8::SMEM_BYTES, st, tm[0], tm[1], tm[2], tm[3], prm);
   return cudaGetLastError() == cudaSuccess ? FP4ATTN_OK : FP4ATTN_ERR_CUDA;
 }
 
