@@ -190,7 +190,8 @@ enum { FP4ATTN_PSCALE_CEIL = 0,    /* E_B = ceil(max y): nothing saturates      
                                       tensor and the one-query schedule only; about twice the conversions per block */
 
 /* how query tiles are assigned to thread blocks (Section "Two-query execution model") */
-enum { FP4ATTN_SCHEDULE_ONE_QUERY = 0,   /* one 128-row query tile per thread block: every shape                 */
+enum { FP4ATTN_SCHEDULE_ONE_QUERY = 0,   /* every shape: one 128-row query tile per thread block, or two where they
+                                            exist and are faster (affine map, exact_pairs 0x5555)                  */
        FP4ATTN_SCHEDULE_TWO_QUERY = 1 }; /* two query tiles of a head share every K / V stage and run as two
                                             independent chains with an accumulator each.  Exists where tensor
                                             memory holds two accumulators beside the score slots without overlays:

@@ -1139,6 +1139,29 @@ def test_two_query_schedule_matches_oracle_and_the_one_query_schedule(name, kw, 
     check_heads(O2, L2, Oo, Lo, heads, rows)
 
 
+@pytest.mark.parametrize("H,N,group", [(74, 256, 1), (74, 256, 2), (37, 512, 1), (90, 256, 1), (10, 1920, 1)])
+@pytest.mark.parametrize("fmt,okw", [(0, dict(p_map=1)), (1, dict(p_map=1, p_scale_rule=1)), (1, dict(p_map=2, exact_pairs=0x5555))])
+def test_default_schedule_has_the_bits_of_one_query_tile(fmt, okw, H, N, group):
+    """d = 64 with the affine or the mixed map: launches that the default gives to the two-query kernel (and two with one round or an odd
+    number of tiles too many for it) against each unit by itself, which is too small for it."""
+    from paper_2609_04105_b200 import binding as Bd
+    B, d = 2, 64
+    w = I.shrink(I.WORKLOADS["cfg1"], B=B, H=H, N=N, d=d)
+    q, k, v = (_dev(t) for t in I.make_qkv(w))
+    k, v = k[:, :H // group].contiguous(), v[:, :H // group].contiguous()
+    ops = [Bd.fp4attn_quantize(q, fmt, Bd.ROLE_Q), Bd.fp4attn_quantize(k, fmt, Bd.ROLE_K), Bd.fp4attn_quantize(v, 0, Bd.ROLE_V)]
+    O, L = Bd.fp4attn_fwd(*ops, **okw)
+
+    def unit(o, heads, n):
+        units = B * heads
+        return Bd.QuantizedOperand(o.packed.view(units, -1)[n].contiguous(), o.scales.view(units, -1)[n].contiguous(), o.G, o.fmt, o.role, (1, 1, N, d))
+
+    for b, h in ((0, 0), (0, H - 1), (1, H // 2), (1, H - 1)):
+        n, nk = b * H + h, b * (H // group) + h // group
+        O1, L1 = Bd.fp4attn_fwd(unit(ops[0], H, n), unit(ops[1], H // group, nk), unit(ops[2], H // group, nk), **okw)
+        assert torch.equal(O[b, h], O1[0, 0]) and torch.equal(L[b, h], L1[0, 0]), (b, h)
+
+
 def test_two_query_schedule_grouped_kv_heads_and_config3_full_size():
     """Grouped K/V heads under the two-query schedule, and config 3 (B8 H16 N8192 d64) at full size: bit-identical to
     the one-query launch."""
