@@ -684,8 +684,9 @@ int launch_attn_two_query(const fp4attn_operands* ops, int B, int H, int N, int 
 // many, make no more rounds over the SMs: a stage of K and V, a trip of the producer and of the issuers and an item boundary serve
 // 256 rows instead of 128.  us, one | two query tiles, MXFP4, NVFP4: B=64, H=16, N=256 21.2 | 18.6, 22.1 | 19.1; 32,
 // 512 29.4 | 26.9, 30.8 | 27.4; 16, 1024 46.1 | 43.9, 48.9 | 44.4; 8, 2048 80.1 | 77.7, 85.0 | 78.3; 8, 8192 1115 | 1109,
-// 1184 | 1113; the mix 19.8 | 18.4 ... 1413 | 1378; exact codes 34.7 | 35.4 ... 1697 | 1729, which stay.  Where they make more: B=1, H=40, N=4096 (9 against 10 half rounds) 96 | 105, B=1, H=3, N=16384 (3, 4) 122 |
-// 161, B=1, H=16, N=1024 (1, 2) 6.1 | 8.8.
+// 1184 | 1113; the mix 19.8 | 18.4 ... 1413 | 1378; exact codes 34.7 | 35.4 ... 1697 | 1729, which stay.  Where they make
+// more: B=1, H=40, N=4096 (9 against 10 half rounds) 96 | 105, B=1, H=3, N=16384 (3, 4) 122 | 161, B=1, H=16, N=1024 (1, 2)
+// 6.1 | 8.8.
 static bool two_queries_faster(int N, int items) {
   if (N % (2 * BM) != 0) return false;
   int dev = 0, sms = 0;
