@@ -32,6 +32,12 @@ using namespace ptx;
 
 constexpr uint32_t k8ColP = 432, k8ColSFQ1 = 496;
 constexpr float kP8Shift = 8.0f;
+// The row references go from the teams to the epilogue through one slot an item and no barrier of their own.  A slot is written
+// when the item's first sweep ends and read after its last product.  Writers: a team of EITHER pair, with the same values, for
+// the products of an item of one stage come from one pair alone, and only that pair's visits are ordered before the epilogue.
+// Slots: item k + 4 is written after the second sweeps of items k + 1, k + 2 and k + 3, two of which share a pair; that pair's
+// later visit awaited a product of item k + 1 or later, and that product awaited that the epilogue had read item k.
+constexpr int kMuSlots = 4;
 
 template <int D, bool NV>
 struct Cfg8 {
@@ -48,8 +54,8 @@ struct Cfg8 {
   static constexpr int OFF_Q = 0;                                     // two buffers
   static constexpr int OFF_QSF = OFF_Q + 2 * C1::Q_BYTES;             // two buffers of 1 KB
   static constexpr int OFF_RMAX = OFF_QSF + 2048;                     // [item parity][first-sweep team][row] float
-  static constexpr int OFF_MU = OFF_RMAX + 2 * 4 * BM * 4;            // [item parity][row] int
-  static constexpr int OFF_K = (OFF_MU + 2 * BM * 4 + 1023) / 1024 * 1024;
+  static constexpr int OFF_MU = OFF_RMAX + 2 * 4 * BM * 4;            // [item % kMuSlots][row] int
+  static constexpr int OFF_K = (OFF_MU + kMuSlots * BM * 4 + 1023) / 1024 * 1024;
   static constexpr int OFF_V = OFF_K + KST * KST_BYTES;
   static constexpr int OFF_OUT = OFF_V + VST * VST_BYTES;
   static constexpr int OFF_BAR = OFF_OUT + C1::OUT_BYTES;
@@ -360,7 +366,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       ok = mbar_wait<false>(bar(B8_OFULL), k & 1, abort_at);
       if (!ok) break;
       tc_fence_after();
-      const int mu = reinterpret_cast<const int*>(sgen + C8::OFF_MU)[(k & 1) * BM + row];   // written before any PV of the item
+      const int mu = reinterpret_cast<const volatile int*>(sgen + C8::OFF_MU)[(k % kMuSlots) * BM + row];
       float Lhw;
       {
         uint32_t r16[16];
@@ -517,7 +523,7 @@ attn_fwd_fp8pv_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         const float ymax = fminf(fmaxf(__fmul_rn(mall, c32), -2097152.0f), 2097152.0f);
         const float tt = __fadd_ru(ymax, 12582912.0f);          // ceil, exact for |y| < 2^22
         b = __fsub_rn(kP8Shift, __fsub_rn(tt, 12582912.0f));
-        if (team == 0) reinterpret_cast<int*>(sgen + C8::OFF_MU)[(phs & 1) * BM + row] = (int)(__float_as_uint(tt) - 0x4B400000u);
+        if (h == 0) reinterpret_cast<volatile int*>(sgen + C8::OFF_MU)[(phs % kMuSlots) * BM + row] = (int)(__float_as_uint(tt) - 0x4B400000u);
       }
     }
   }
