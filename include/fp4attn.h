@@ -190,14 +190,16 @@ enum { FP4ATTN_PSCALE_CEIL = 0,    /* E_B = ceil(max y): nothing saturates      
                                       tensor and the one-query schedule only; about twice the conversions per block */
 
 /* how query tiles are assigned to thread blocks (Section "Two-query execution model") */
-enum { FP4ATTN_SCHEDULE_ONE_QUERY = 0,   /* every shape: one 128-row query tile per thread block, or two where they
-                                            exist and are faster (affine map, exact_pairs 0x5555)                  */
-       FP4ATTN_SCHEDULE_TWO_QUERY = 1 }; /* two query tiles of a head share every K / V stage and run as two
+enum { FP4ATTN_SCHEDULE_ONE_QUERY = 0,   /* one 128-row query tile per thread block: every shape                 */
+       FP4ATTN_SCHEDULE_TWO_QUERY = 1,   /* two query tiles of a head share every K / V stage and run as two
                                             independent chains with an accumulator each.  Exists where tensor
                                             memory holds two accumulators beside the score slots without overlays:
                                             d = 64, N a multiple of 256, noncausal, one NVFP4 factor per tensor;
                                             anything else returns FP4ATTN_ERR_UNSUPPORTED_SHAPE.  Same results, bit
                                             for bit, as FP4ATTN_SCHEDULE_ONE_QUERY                                */
+       FP4ATTN_SCHEDULE_AUTO = 2 };      /* two where they exist and are known to be faster (affine map, exact_pairs
+                                            0x5555), else one: every shape, and every option that the one-query
+                                            schedule takes                                                        */
 
 /* format of the probabilities and of V in the second product */
 enum { FP4ATTN_PV_MXFP4 = 0,   /* Direct-P: E2M1 codes with E8M0 block scales for P and V (the path of this library)   */
@@ -227,7 +229,7 @@ typedef struct {
                                        B*H factors and k_G B*kv_heads, one per (batch, head) unit
                                        (fp4attn_quantize_nvfp4_per_head); with the ideal and the
                                        affine map, not with FP4ATTN_PMAP_HYBRID                 */
-  int schedule;                     /* FP4ATTN_SCHEDULE_ONE_QUERY (0, default) or _TWO_QUERY */
+  int schedule;                     /* FP4ATTN_SCHEDULE_ONE_QUERY (0), _TWO_QUERY or _AUTO     */
   int pv_fmt;                       /* FP4ATTN_PV_MXFP4 (0, default) or FP4ATTN_PV_E4M3: then v holds E4M3 bytes of V^T
                                        [B, kv_heads, d, N] from fp4attn_quantize_v_e4m3, v_sf is ignored, v_G is required;
                                        with the ideal map, the ceiling rule and the one-query schedule only          */

@@ -26,7 +26,7 @@ FMT_MXFP4, FMT_NVFP4 = 0, 1
 ROLE_Q, ROLE_K, ROLE_V = 0, 1, 2
 PMAP_IDEAL, PMAP_AFFINE, PMAP_HYBRID = 0, 1, 2
 PSCALE_CEIL, PSCALE_THR16, PSCALE_MSE = 0, 1, 2
-SCHEDULE_ONE_QUERY, SCHEDULE_TWO_QUERY = 0, 1
+SCHEDULE_ONE_QUERY, SCHEDULE_TWO_QUERY, SCHEDULE_AUTO = 0, 1, 2
 PV_MXFP4, PV_E4M3 = 0, 1
 QSCALE_CEIL, QSCALE_THR16, QSCALE_FLOOR, QSCALE_MSE = 0, 1, 2, 3
 (OK, ERR_INVALID_ARG, ERR_UNSUPPORTED_SHAPE, ERR_UNSUPPORTED_ARCH, ERR_ALIGNMENT, ERR_WORKSPACE, ERR_CUDA,
@@ -210,10 +210,11 @@ def fp4attn_fwd(q: QuantizedOperand, k: QuantizedOperand, v: QuantizedOperand, s
                 out: Optional[torch.Tensor] = None, lse: Optional[torch.Tensor] = None,
                 status: Optional[torch.Tensor] = None, p_map: int = PMAP_IDEAL, affine_a: float = 0.0,
                 affine_b: float = 0.0, p_scale_rule: int = PSCALE_CEIL, causal: bool = False,
-                exact_pairs: int = 0, schedule: int = SCHEDULE_ONE_QUERY,
+                exact_pairs: int = 0, schedule: int = SCHEDULE_AUTO,
                 seq_len: Optional[torch.Tensor] = None, fixed_reference: Optional[int] = None) -> Tuple[torch.Tensor, torch.Tensor]:
     """Direct-P attention forward on quantized operands -> (O bf16 [B,H,N,d], LSE fp32 [B,H,N]).
     p_map selects the exact code map or the affine classifier (affine_a = 0: A = 1.5, B = 1.2).
+    schedule: the faster of one and two query tiles per thread block, or one of them; the results are the same bits.
     seq_len: optional CUDA int32 tensor [B], the token count of every batch entry (padded to N).
     fixed_reference: None - running row reference; an integer - that constant row reference (the shiftless path)."""
     return (_native_module or _native()).fwd(q, k, v, softmax_scale, out, lse, status, p_map, affine_a, affine_b, p_scale_rule, causal,

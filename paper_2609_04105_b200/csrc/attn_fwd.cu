@@ -719,8 +719,9 @@ extern "C" int fp4attn_fwd(const fp4attn_operands* ops, int B, int H, int N, int
   }
   if (ops->p_scale_rule != FP4ATTN_PSCALE_CEIL && ops->p_scale_rule != FP4ATTN_PSCALE_THR16 && ops->p_scale_rule != FP4ATTN_PSCALE_MSE)
     return FP4ATTN_ERR_INVALID_ARG;
+  const bool may_take_one_query = ops->schedule == FP4ATTN_SCHEDULE_ONE_QUERY || ops->schedule == FP4ATTN_SCHEDULE_AUTO;
   if (ops->p_scale_rule == FP4ATTN_PSCALE_MSE &&
-      (ops->p_map != FP4ATTN_PMAP_IDEAL || ops->g_per_head || ops->schedule != FP4ATTN_SCHEDULE_ONE_QUERY || ops->pv_fmt != FP4ATTN_PV_MXFP4))
+      (ops->p_map != FP4ATTN_PMAP_IDEAL || ops->g_per_head || !may_take_one_query || ops->pv_fmt != FP4ATTN_PV_MXFP4))
     return FP4ATTN_ERR_INVALID_ARG;                                 // ideal map, one factor per tensor, one-query schedule
   if (ops->g_per_head != 0 && ops->g_per_head != 1) return FP4ATTN_ERR_INVALID_ARG;
   if (ops->g_per_head && ops->p_map == FP4ATTN_PMAP_HYBRID) return FP4ATTN_ERR_INVALID_ARG;   // ideal and affine maps only
@@ -760,15 +761,15 @@ extern "C" int fp4attn_fwd(const fp4attn_operands* ops, int B, int H, int N, int
   prm.c_mx2 = twice(nonzero(c_mx));
   prm.ca_mx2 = twice(nonzero(prm.aff_a * c_mx));
   prm.thr16 = ops->p_scale_rule == FP4ATTN_PSCALE_THR16;
-  if (ops->schedule != FP4ATTN_SCHEDULE_ONE_QUERY && ops->schedule != FP4ATTN_SCHEDULE_TWO_QUERY) return FP4ATTN_ERR_INVALID_ARG;
+  if (!may_take_one_query && ops->schedule != FP4ATTN_SCHEDULE_TWO_QUERY) return FP4ATTN_ERR_INVALID_ARG;
   if (ops->pv_fmt != FP4ATTN_PV_MXFP4 && ops->pv_fmt != FP4ATTN_PV_E4M3) return FP4ATTN_ERR_INVALID_ARG;
-  if (ops->seq_len && ops->schedule != FP4ATTN_SCHEDULE_ONE_QUERY) return FP4ATTN_ERR_INVALID_ARG;
+  if (ops->seq_len && !may_take_one_query) return FP4ATTN_ERR_INVALID_ARG;
   if (((uintptr_t)ops->seq_len & 3) != 0) return FP4ATTN_ERR_ALIGNMENT;
   if (ops->row_reference != FP4ATTN_REFERENCE_RUNNING && ops->row_reference != FP4ATTN_REFERENCE_FIXED) return FP4ATTN_ERR_INVALID_ARG;
   prm.ref_fixed = ops->fixed_reference;
   if (ops->row_reference == FP4ATTN_REFERENCE_FIXED) {
     // the shiftless path: ideal or affine map, ceiling rule, one factor per tensor, one query tile, FP4 P and V
-    if (pmap > 1 || ops->p_scale_rule != FP4ATTN_PSCALE_CEIL || ops->g_per_head || ops->schedule != FP4ATTN_SCHEDULE_ONE_QUERY ||
+    if (pmap > 1 || ops->p_scale_rule != FP4ATTN_PSCALE_CEIL || ops->g_per_head || !may_take_one_query ||
         ops->pv_fmt != FP4ATTN_PV_MXFP4 || ops->fixed_reference < -1000 || ops->fixed_reference > 1000)
       return FP4ATTN_ERR_INVALID_ARG;
     const int sel = (d == 128 ? 8 : 0) | (nv ? 4 : 0) | (pmap ? 2 : 0) | (masked ? 1 : 0);
@@ -792,7 +793,8 @@ extern "C" int fp4attn_fwd(const fp4attn_operands* ops, int B, int H, int N, int
     }
   }
   if (ops->pv_fmt == FP4ATTN_PV_E4M3) return launch_attn_fp8pv(ops, B, H, N, d, prm, st);
-  if (ops->schedule == FP4ATTN_SCHEDULE_TWO_QUERY || (d == 64 && (pmap == 1 || pmap == 3) && !masked && !ops->g_per_head && two_queries_faster(N, prm.n_items)))
+  if (ops->schedule == FP4ATTN_SCHEDULE_TWO_QUERY ||
+      (ops->schedule == FP4ATTN_SCHEDULE_AUTO && d == 64 && (pmap == 1 || pmap == 3) && !masked && !ops->g_per_head && two_queries_faster(N, prm.n_items)))
     return launch_attn_two_query(ops, B, H, N, d, pmap, prm, st);
   if (ops->p_scale_rule == FP4ATTN_PSCALE_MSE) {
     const int sel = (d == 128 ? 4 : 0) | (nv ? 2 : 0) | (masked ? 1 : 0);

@@ -565,7 +565,7 @@ static int launch_fp8(const fp4attn_operands* ops, int B, int H, int N, const Fp
 int launch_attn_fp8pv(const fp4attn_operands* ops, int B, int H, int N, int d, AttnParams prm, cudaStream_t st) {
   if (!ops->v_G) return FP4ATTN_ERR_INVALID_ARG;
   if (ops->p_map != FP4ATTN_PMAP_IDEAL || ops->p_scale_rule != FP4ATTN_PSCALE_CEIL || ops->g_per_head ||
-      ops->schedule != FP4ATTN_SCHEDULE_ONE_QUERY)
+      ops->schedule == FP4ATTN_SCHEDULE_TWO_QUERY)
     return FP4ATTN_ERR_INVALID_ARG;                               // the code maps and block rules belong to the FP4 probability path
   Fp8Params pp{prm, ops->v_G};
   const bool nv = ops->qk_fmt == FP4ATTN_FMT_NVFP4;

@@ -1123,7 +1123,7 @@ def test_two_query_schedule_matches_oracle_and_the_one_query_schedule(name, kw, 
     from paper_2609_04105_b200 import binding as Bd
     w = I.shrink(I.WORKLOADS[name], **kw)
     q, k, v = I.make_qkv(w)
-    O1, L1 = run_gpu_general(w, q, k, v, **okw)
+    O1, L1 = run_gpu_general(w, q, k, v, schedule=Bd.SCHEDULE_ONE_QUERY, **okw)
     O2, L2 = run_gpu_general(w, q, k, v, schedule=Bd.SCHEDULE_TWO_QUERY, **okw)
     assert np.array_equal(O1, O2) and np.array_equal(L1, L2)
     qd, kd, vd = oracle_operands(w, q, k, v)
@@ -1169,15 +1169,76 @@ def test_two_query_schedule_grouped_kv_heads_and_config3_full_size():
     w = I.shrink(I.WORKLOADS["cfg3"], B=1, H=6, N=512)
     q, k, v = I.make_qkv(w)
     k, v = k[:, :2], v[:, :2]
-    O1, L1 = run_gpu_general(w, q, k, v)
+    O1, L1 = run_gpu_general(w, q, k, v, schedule=Bd.SCHEDULE_ONE_QUERY)
     O2, L2 = run_gpu_general(w, q, k, v, schedule=Bd.SCHEDULE_TWO_QUERY)
     assert np.array_equal(O1, O2) and np.array_equal(L1, L2)
     w = I.WORKLOADS["cfg3"]
     q, k, v = I.make_qkv(w)
     for okw in (dict(), dict(p_map=Bd.PMAP_AFFINE)):
-        O1, L1 = run_gpu_general(w, q, k, v, **okw)
+        O1, L1 = run_gpu_general(w, q, k, v, schedule=Bd.SCHEDULE_ONE_QUERY, **okw)
         O2, L2 = run_gpu_general(w, q, k, v, schedule=Bd.SCHEDULE_TWO_QUERY, **okw)
         assert np.array_equal(O1, O2) and np.array_equal(L1, L2)
+
+
+def _captured_kernels(graph):
+    """Mangled names of a captured graph's kernels."""
+    import ctypes
+
+    class KernelNodeParams(ctypes.Structure):
+        _fields_ = [("func", ctypes.c_void_p), ("sizes", ctypes.c_uint * 7), ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                    ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+    cu, g, n = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(graph), ctypes.c_size_t()
+    assert cu.cuGraphGetNodes(g, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert cu.cuGraphGetNodes(g, nodes, ctypes.byref(n)) == 0
+    names = []
+    for node in nodes:
+        kind, p, name = ctypes.c_int(), KernelNodeParams(), ctypes.c_char_p()
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value == 0:                                      # a kernel node
+            assert cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)) == 0
+            get, handle = (cu.cuFuncGetName, p.func) if p.func else (cu.cuKernelGetName, p.kern)
+            assert get(ctypes.byref(name), ctypes.c_void_p(handle)) == 0
+            names.append(name.value.decode())
+    return names
+
+
+@pytest.mark.parametrize("schedule,two", [(None, True), ("SCHEDULE_AUTO", True), ("SCHEDULE_ONE_QUERY", False), ("SCHEDULE_TWO_QUERY", True)])
+def test_a_schedule_that_is_asked_for_is_the_one_that_runs(schedule, two):
+    """A launch that the default gives to the two-query kernel (affine map, d = 64, one query tile per SM twice over): the kernel by
+    its name in the captured graph."""
+    from paper_2609_04105_b200 import binding as Bd
+    H, N, d = torch.cuda.get_device_properties(0).multi_processor_count, 256, 64
+    x = torch.zeros((1, H, N, d), dtype=torch.bfloat16, device="cuda")
+    ops = [Bd.fp4attn_quantize(x, 0, role) for role in (Bd.ROLE_Q, Bd.ROLE_K, Bd.ROLE_V)]
+    kw = {} if schedule is None else {"schedule": getattr(Bd, schedule)}
+    fwd = lambda: Bd.fp4attn_fwd(*ops, p_map=Bd.PMAP_AFFINE, **kw)
+    fwd()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        fwd()
+    name, = _captured_kernels(g.raw_cuda_graph())
+    assert ("attn_fwd_2q_kernel" in name) == two and ("attn_fwd_kernel" in name) != two, name
+
+
+@pytest.mark.parametrize("kw", [dict(p_scale_rule=2), dict(fixed_reference=0), dict(causal=True), dict(padded=True), dict(v8=True)])
+def test_options_of_the_one_query_schedule_take_the_default_and_the_one_query_value(kw):
+    from paper_2609_04105_b200 import binding as Bd
+    w = I.shrink(I.WORKLOADS["cfg1"], N=256, d=64)
+    q, k, v = (_dev(t) for t in I.make_qkv(w))
+    kw = dict(kw)
+    if kw.pop("padded", False):
+        kw["seq_len"] = torch.tensor([200], dtype=torch.int32, device="cuda")
+    ops = [Bd.fp4attn_quantize(q, 0, Bd.ROLE_Q), Bd.fp4attn_quantize(k, 0, Bd.ROLE_K),
+           Bd.fp4attn_quantize_v_e4m3(v) if kw.pop("v8", False) else Bd.fp4attn_quantize(v, 0, Bd.ROLE_V)]
+    O, L = Bd.fp4attn_fwd(*ops, **kw)
+    for schedule in (Bd.SCHEDULE_ONE_QUERY, Bd.SCHEDULE_AUTO):
+        O1, L1 = Bd.fp4attn_fwd(*ops, schedule=schedule, **kw)
+        assert torch.equal(O, O1) and torch.equal(L, L1)
+    for schedule in (Bd.SCHEDULE_TWO_QUERY, 3, -1):
+        with pytest.raises(Bd.Fp4AttnError):
+            Bd.fp4attn_fwd(*ops, schedule=schedule, **kw)
 
 
 def test_two_query_schedule_rejects_what_it_does_not_cover():
