@@ -434,7 +434,7 @@ def run_cuda(args, w):
         del g
     # algorithmic bytes per element: bf16 in, 4-bit codes and scale bytes out; NVFP4 reads the tensor twice
     q_bpe = (2 + 0.5 + 1.0 / 32) if w.qk_fmt == I.FMT_MXFP4 else (2 + 2 + 0.5 + 1.0 / 16)
-    q_kernel = "quant_mx_rows_kernel" if w.qk_fmt == I.FMT_MXFP4 else "amax_partials_kernel + nv_encode_factor_kernel + quant_nv_rows_kernel"
+    q_kernel = "quant_mx_rows_kernel" if w.qk_fmt == I.FMT_MXFP4 else "amax_partials_kernel + quant_nv_rows_kernel"
     q_bytes = B * H * N * d * q_bpe
     v_bytes = B * H * N * d * (2 + 0.5 + 1.0 / 32)
 
@@ -474,7 +474,7 @@ def run_cuda(args, w):
             rule = pscale if (pscale != Bd.PSCALE_MSE or name == "ideal") else Bd.PSCALE_CEIL     # the MSE rule exists for the ideal map
             if "fixed_reference" in kw:
                 rule = Bd.PSCALE_CEIL                                # the fixed reference comes with the ceiling rule
-            fn = lambda: Bd.fp4attn_fwd(qd0, kd0, vd0, out=O_alt, status=status, p_scale_rule=rule, **kw)
+            fn = lambda: Bd.fp4attn_fwd(qd0, kd0, vd0, out=O_alt, status=status, p_scale_rule=rule, schedule=Bd.SCHEDULE_ONE_QUERY, **kw)
             for _ in range(3):
                 fn()
             ms_map = statistics.median(timed_launches(fn, 10, flush, E, torch.cuda.synchronize))
@@ -605,6 +605,8 @@ def run_cuda(args, w):
                 variants.append(("length_mix_", dict(seq_len=sl), sum(float(n) * n for n in mix) / (ww.B * float(ww.N) ** 2)))
                 rec["length_mix_tokens"] = mix
             for key, kw, share in variants:
+                if kw is not None:
+                    kw = {"schedule": Bd.SCHEDULE_ONE_QUERY, **kw}       # one query tile per thread block unless the variant says two
                 fn = (lambda: Bd.fp4attn_fwd(sq, sk, sv8, out=so, status=status)) if kw is None else \
                      (lambda: Bd.fp4attn_fwd(sq, sk, sv, out=so, status=status, **kw))
                 for _ in range(3):
