@@ -811,29 +811,36 @@ def test_many_small_heads_more_items_than_one_wave():
     check_heads(Og, Lg, Oo, Lo, heads)
 
 
-@pytest.mark.parametrize("per_head,causal,padded", [(True, False, False), (False, True, False), (True, True, True)])
-def test_items_beyond_those_a_cta_decodes_ahead(per_head, causal, padded):
-    """9600 work items, up to 65 a CTA: one more than are decoded when it starts.  The bits are those of the two halves of the
-    batch, whose CTAs decode all of theirs ahead."""
+@pytest.mark.parametrize("per_head,causal,padded,fp8", [(True, False, False, False), (False, True, False, False), (False, False, True, False),
+                                                        (True, True, True, False), (False, True, False, True), (False, False, True, True)])
+def test_items_beyond_those_a_cta_decodes_ahead(per_head, causal, padded, fp8):
+    """More than 65 work items a CTA, of which 64 are decoded when it starts.  The bits are those of the two halves of the batch,
+    whose CTAs decode all of theirs ahead."""
     from paper_2609_04105_b200 import binding as Bd
-    B, H, N, d = 10, 480, 256, 64
+    B, N, d = 10, 256, 64
+    tokens = [256, 1, 129, 200, 256, 128, 77, 250, 256, 33] if padded else [N] * B
+    tiles = [(n + 127) // 128 for n in tokens]                   # query tiles beyond a length are no items
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    H = 2 * (65 * sms // (2 * sum(tiles)) + 1)
+    assert sum(tiles) * H > 65 * sms and max(sum(tiles[:B // 2]), sum(tiles[B // 2:])) * H <= 64 * sms
     gen = torch.Generator(device="cuda")
     gen.manual_seed(7)
     draw = lambda h: torch.randn((B, h, N, d), generator=gen, device="cuda").to(torch.bfloat16)
     q, k, v = draw(H), draw(H // 2), draw(H // 2)
-    lens = torch.tensor([256, 1, 129, 200, 256, 128, 77, 250, 256, 33], dtype=torch.int32, device="cuda") if padded else None
+    lens = torch.tensor(tokens, dtype=torch.int32, device="cuda") if padded else None
 
     def run(part):
         quant = (lambda x, r: Bd.fp4attn_quantize_nvfp4_per_head(x, r)) if per_head else (lambda x, r: Bd.fp4attn_quantize(x, 0, r))
         x = [t[part].contiguous() for t in (q, k, v)]
-        return Bd.fp4attn_fwd(quant(x[0], Bd.ROLE_Q), quant(x[1], Bd.ROLE_K), Bd.fp4attn_quantize(x[2], Bd.FMT_MXFP4, Bd.ROLE_V),
-                              causal=causal, seq_len=lens[part].contiguous() if padded else None)
+        v8 = Bd.fp4attn_quantize_v_e4m3(x[2]) if fp8 else Bd.fp4attn_quantize(x[2], Bd.FMT_MXFP4, Bd.ROLE_V)
+        return Bd.fp4attn_fwd(quant(x[0], Bd.ROLE_Q), quant(x[1], Bd.ROLE_K), v8, causal=causal,
+                              seq_len=lens[part].contiguous() if padded else None)
 
     O, L = run(slice(0, B))
     for part in (slice(0, B // 2), slice(B // 2, B)):
         O1, L1 = run(part)
         for b in range(B // 2):
-            n = int(lens[part][b]) if padded else N
+            n = tokens[part][b]
             assert torch.equal(O[part][b, :, :n], O1[b, :, :n]) and torch.equal(L[part][b, :, :n], L1[b, :, :n]), (part, b)
 
 
