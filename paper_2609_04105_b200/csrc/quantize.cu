@@ -459,7 +459,9 @@ __device__ __forceinline__ void nv_code_chunk(const uint32_t (&raw)[kLoads][8], 
   constexpr uint32_t LPR = D / 16;                 // lanes per row
   constexpr uint32_t CT = (D / 16 + 3) / 4;
   const uint32_t seg = threadIdx.x % LPR;
-  const bool plain = G < 1.2676506e30f;            // 2^100: a * G is then finite (a of a NaN tensor apart, which any quotient leaves one)
+  // a * G is at most about 2688 for any finite G.  An infinite one (tensors below 2^-116) makes it infinite, which the division
+  // by 6 keeps and the remainder in sixth() would turn into a NaN.
+  const bool plain = G < INFINITY;
 #pragma unroll
   for (int k = 0; k < kLoads; ++k) {
     const float aG = __fmul_rn(__uint_as_float(absmax_bf16x16(raw[k]) << 16), G);

@@ -246,13 +246,16 @@ def test_nvfp4_one_launch_and_two_launch_sizes(B, H, N, d, offset):
     _check_operand(Bd.fp4attn_quantize(t, Bd.FMT_NVFP4, Bd.ROLE_K), Qz.quantize_qk(bits, "nv"), Bd.ROLE_K)
 
 
-@pytest.mark.parametrize("exponent", [60, 0, -85, -95, -110])        # encode factors of 2^-51 ... 2^119; from 2^100 on a block's scale is divided for
+@pytest.mark.filterwarnings("ignore:overflow")
+@pytest.mark.parametrize("exponent", [60, 0, -85, -95, -110, -121])  # encode factors of 2^-51 ... 2^119, and an infinite one
 @pytest.mark.parametrize("kw", [dict(B=1, H=2, N=128, d=64), dict(B=1, H=20, N=2048)])     # one launch, two launches
 def test_nvfp4_of_very_small_and_large_tensors_matches_oracle(exponent, kw):
     from paper_2609_04105_b200 import binding as Bd
     w = I.shrink(I.WORKLOADS["cfg1"], **kw)
     q, _, _ = I.make_qkv(w)
     bits = I.f32_to_bf16_bits(np.ldexp(I.bf16_bits_to_f32(q), exponent))
+    bits[(bits & 0x7FFF) == 0] += 1                              # (0 times an infinite factor is no number)
+    assert np.isinf(Qz.nv_tensor_scale(I.bf16_bits_to_f32(bits))) == (exponent == -121)
     _check_operand(Bd.fp4attn_quantize(_dev(bits), Bd.FMT_NVFP4, Bd.ROLE_Q), Qz.quantize_qk(bits, "nv"), Bd.ROLE_Q)
     got, want = Bd.fp4attn_quantize_nvfp4_per_head(_dev(bits), Bd.ROLE_Q), Qz.quantize_qk(bits, "nv", per_head=True)
     assert np.array_equal(got.G.cpu().numpy().reshape(w.B, w.H), want["G"])
