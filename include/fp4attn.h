@@ -197,8 +197,8 @@ enum { FP4ATTN_SCHEDULE_ONE_QUERY = 0,   /* one 128-row query tile per thread bl
                                             d = 64, N a multiple of 256, noncausal, one NVFP4 factor per tensor;
                                             anything else returns FP4ATTN_ERR_UNSUPPORTED_SHAPE.  Same results, bit
                                             for bit, as FP4ATTN_SCHEDULE_ONE_QUERY                                */
-       FP4ATTN_SCHEDULE_AUTO = 2 };      /* two where they exist and are known to be faster (affine map, exact_pairs
-                                            0x5555), else one: every shape, and every option that the one-query
+       FP4ATTN_SCHEDULE_AUTO = 2 };      /* two where they exist and are known to be faster (with the affine map and
+                                            exact_pairs 0x5555), else one: every shape, and every option that the one-query
                                             schedule takes                                                        */
 
 /* format of the probabilities and of V in the second product */

@@ -679,20 +679,27 @@ static int launch_attn(const fp4attn_operands* ops, int B, int H, int N, AttnPar
 
 int launch_attn_two_query(const fp4attn_operands* ops, int B, int H, int N, int d, int pmap, AttnParams prm, cudaStream_t st);
 
-// The affine map and the even mix (8 of 16 pairs exact) at d = 64 without a mask: the two-query kernel gives the same bits, and
-// with few exponentials in the map, where the hand-offs set the pace, it is faster wherever its items, twice as long and half as
-// many, make no more rounds over the SMs: a stage of K and V, a trip of the producer and of the issuers and an item boundary serve
-// 256 rows instead of 128.  us, one | two query tiles, MXFP4, NVFP4: B=64, H=16, N=256 21.2 | 18.6, 22.1 | 19.1; 32,
-// 512 29.4 | 26.9, 30.8 | 27.4; 16, 1024 46.1 | 43.9, 48.9 | 44.4; 8, 2048 80.1 | 77.7, 85.0 | 78.3; 8, 8192 1115 | 1109,
-// 1184 | 1113; the mix 19.8 | 18.4 ... 1413 | 1378; exact codes 34.7 | 35.4 ... 1697 | 1729, which stay.  Where they make
-// more: B=1, H=40, N=4096 (9 against 10 half rounds) 96 | 105, B=1, H=3, N=16384 (3, 4) 122 | 161, B=1, H=16, N=1024 (1, 2)
-// 6.1 | 8.8.
-static bool two_queries_faster(int N, int items) {
-  if (N % (2 * BM) != 0) return false;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return false;
+// FP4ATTN_SCHEDULE_AUTO, d = 64, no mask: the two-query kernel gives the same bits; its items are twice as long and half as many,
+// and a stage of K and V, a trip of the producer and an item boundary serve 256 rows instead of 128.  Attention alone from a
+// graph, us, one | two query tiles (rounds over the SMs in front):
+//   rounds, shape          affine MXFP4   NVFP4          0x5555 MXFP4   NVFP4          0x1111 MXFP4   NVFP4          exact MXFP4
+//   14|7   1024 x N=256    21.1 | 18.5    21.7 | 18.6    19.8 | 18.2    19.9 | 18.5    19.6 | 18.4    20.0 | 18.8    22.2 | 21.4
+//   4|2    16 x N=4096     44.8 | 43.9    47.3 | 44.0    54.5 | 54.2    55.0 | 54.4    46.0 | 46.4    48.5 | 46.7    64.8 | 65.9
+//   56|28  128 x N=8192    1117 | 1108    1187 | 1112    1404 | 1373    1416 | 1380    1154 | 1181    1220 | 1186    1687 | 1718
+//   4|2    148 x N=512     10.5 | 9.9     11.1 | 10.0    10.9 | 11.0    11.2 | 11.0
+//   2|1    148 x N=256     5.3 | 5.3      5.6 | 5.5      5.4 | 5.7      5.7 | 5.8      5.3 | 5.4      5.6 | 5.5       5.8 | 6.2
+//   2|1    37 x N=1024     9.2 | 9.0      9.7 | 9.1      10.2 | 10.4    10.4 | 10.5
+//   9|5    40 x N=4096     96.2 | 105     102 | 105      118 | 128      119 | 129      98.9 | 111     104 | 112       140 | 160
+//   51|26  471 x N=2048    284 | 280      300 | 280      340 | 335      341 | 337      288 | 294      304 | 297       399 | 417
+//   59|30  136 x N=8192    1177 | 1187    1249 | 1191    1480 | 1471    1492 | 1477    1217 | 1266    1285 | 1270     1777 | 1841
+// So it is taken where it is no slower in either format: the affine map, and the even mix from four rounds on, in no more rounds
+// than one query tile needs.  (Left out though faster: NVFP4 affine at odd numbers of rounds from about twenty on, 0x1111 with
+// NVFP4 at even ones, N = 256 with any map.)
+static bool two_queries_faster(int N, int items, int pmap) {
+  const int sms = device_sms();
+  if (N % (2 * BM) != 0 || !sms) return false;
   const long long one = ((long long)items + sms - 1) / sms, two = ((long long)items / 2 + sms - 1) / sms;
-  return 2 * two <= one;
+  return 2 * two <= one && (pmap == 1 || (pmap == 3 && one >= 4));
 }
 int launch_attn_fp8pv(const fp4attn_operands* ops, int B, int H, int N, int d, AttnParams prm, cudaStream_t st);
 
@@ -794,7 +801,7 @@ extern "C" int fp4attn_fwd(const fp4attn_operands* ops, int B, int H, int N, int
   }
   if (ops->pv_fmt == FP4ATTN_PV_E4M3) return launch_attn_fp8pv(ops, B, H, N, d, prm, st);
   if (ops->schedule == FP4ATTN_SCHEDULE_TWO_QUERY ||
-      (ops->schedule == FP4ATTN_SCHEDULE_AUTO && d == 64 && (pmap == 1 || pmap == 3) && !masked && !ops->g_per_head && two_queries_faster(N, prm.n_items)))
+      (ops->schedule == FP4ATTN_SCHEDULE_AUTO && d == 64 && !masked && !ops->g_per_head && two_queries_faster(N, prm.n_items, pmap)))
     return launch_attn_two_query(ops, B, H, N, d, pmap, prm, st);
   if (ops->p_scale_rule == FP4ATTN_PSCALE_MSE) {
     const int sel = (d == 128 ? 4 : 0) | (nv ? 2 : 0) | (masked ? 1 : 0);

@@ -121,5 +121,6 @@ cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, unsigned thr
 constexpr int kMaxDevices = 64;      // per-device host-side caches are arrays of this length
 
 int check_device_sm100();            // FP4ATTN_OK or FP4ATTN_ERR_UNSUPPORTED_ARCH / _CUDA
+int device_sms();                    // SMs of the current device, kept per device; 0 if the runtime does not tell
 
 }  // namespace fp4attn

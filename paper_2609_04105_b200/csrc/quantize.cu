@@ -633,7 +633,7 @@ static void launch_mx_v(const uint4* xs, int n_tiles, int N, void* packed, void*
                     (uint8_t*)scales, N, n_tiles);
 }
 
-static int device_sms() {                          // 0 if the runtime does not tell
+int device_sms() {
   static std::atomic<int> sm_count[kMaxDevices];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;

@@ -1146,7 +1146,7 @@ def test_two_query_schedule_matches_oracle_and_the_one_query_schedule(name, kw, 
     check_heads(O2, L2, Oo, Lo, heads, rows)
 
 
-@pytest.mark.parametrize("H,N,group", [(74, 256, 1), (74, 256, 2), (37, 512, 1), (90, 256, 1), (10, 1920, 1)])
+@pytest.mark.parametrize("H,N,group", [(74, 256, 1), (74, 256, 2), (37, 512, 1), (90, 256, 1), (10, 1920, 1), (148, 256, 2)])
 @pytest.mark.parametrize("fmt,okw", [(0, dict(p_map=1)), (1, dict(p_map=1, p_scale_rule=1)), (1, dict(p_map=2, exact_pairs=0x5555))])
 def test_default_schedule_has_the_bits_of_one_query_tile(fmt, okw, H, N, group):
     """d = 64 with the affine or the mixed map: launches that the default gives to the two-query kernel (and two with one round or an odd
@@ -1211,16 +1211,20 @@ def _captured_kernels(graph):
     return names
 
 
-@pytest.mark.parametrize("schedule,two", [(None, True), ("SCHEDULE_AUTO", True), ("SCHEDULE_ONE_QUERY", False), ("SCHEDULE_TWO_QUERY", True)])
-def test_a_schedule_that_is_asked_for_is_the_one_that_runs(schedule, two):
-    """A launch that the default gives to the two-query kernel (affine map, d = 64, one query tile per SM twice over): the kernel by
-    its name in the captured graph."""
+@pytest.mark.parametrize("schedule,heads,okw,two", [(None, 1, dict(p_map=1), True), ("SCHEDULE_AUTO", 1, dict(p_map=1), True),
+                                                    ("SCHEDULE_ONE_QUERY", 1, dict(p_map=1), False), ("SCHEDULE_TWO_QUERY", 1, dict(p_map=1), True),
+                                                    (None, 1, dict(p_map=2, exact_pairs=0x5555), False),      # two rounds: slower with two tiles
+                                                    (None, 2, dict(p_map=2, exact_pairs=0x5555), True),       # four rounds
+                                                    (None, 2, dict(p_map=2, exact_pairs=0x1111), False), (None, 2, dict(), False)])
+def test_a_schedule_that_is_asked_for_is_the_one_that_runs(schedule, heads, okw, two):
+    """Two query tiles per head and `heads` heads per SM, d = 64: the kernel by its name in the captured graph, for every schedule on a
+    launch that the default gives to the two-query kernel, and for the default with other maps."""
     from paper_2609_04105_b200 import binding as Bd
-    H, N, d = torch.cuda.get_device_properties(0).multi_processor_count, 256, 64
+    H, N, d = heads * torch.cuda.get_device_properties(0).multi_processor_count, 256, 64
     x = torch.zeros((1, H, N, d), dtype=torch.bfloat16, device="cuda")
     ops = [Bd.fp4attn_quantize(x, 0, role) for role in (Bd.ROLE_Q, Bd.ROLE_K, Bd.ROLE_V)]
     kw = {} if schedule is None else {"schedule": getattr(Bd, schedule)}
-    fwd = lambda: Bd.fp4attn_fwd(*ops, p_map=Bd.PMAP_AFFINE, **kw)
+    fwd = lambda: Bd.fp4attn_fwd(*ops, **okw, **kw)
     fwd()
     g = torch.cuda.CUDAGraph(keep_graph=True)
     with torch.cuda.graph(g):
