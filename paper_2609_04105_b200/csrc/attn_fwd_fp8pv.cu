@@ -48,6 +48,7 @@ struct Cfg8 {
   // every other step needs V.  Attention alone, us, d=128 N=8192 | d=128 N=1024 | causal N=8192 | d=64 N=8192: one ring of 5 slots
   // (d=64: 8) 748 | 110 | 402 | 718, K and V slots 8 and 3 722 | 104 | 397 | 703.  With the issuers and visits as they are now: V
   // slots 3 680 | 104 | 381 | 646, 4 682 | 97 | 381 | 679; K slots 4, 6, 8 686, 684, 680; a third Q buffer 690 | 95 | 379 | 646.
+  // (Short sequences at d = 64 were not timed with more than three.)
   static constexpr int KST_BYTES = (C1::K_BYTES + C1::KSF_BYTES + 1023) / 1024 * 1024;   // K, K scales
   static constexpr int VST_BYTES = V_BYTES + ONES_BYTES;
   static constexpr int KST = 8, VST = (D == 128) ? 4 : 3;

@@ -17,6 +17,7 @@ import json
 import multiprocessing as mp
 import os
 import sys
+import tempfile
 import time
 
 import numpy as np
@@ -87,6 +88,25 @@ def _fp8_head(Og, Lg, qd, kd, v8, chunk=1024, n=None):
     return st
 
 
+def _launch(args, lens, path):
+    """The configuration's launch on the device, as bench.py launches it; O (fp32), LSE -> `path`."""
+    import torch
+    from paper_2609_04105_b200 import binding as Bd
+    w = I.WORKLOADS[args.workload]
+    q, k, v = I.make_qkv(w)
+    dev = lambda a: torch.from_numpy(a.view(np.int16)).cuda().view(torch.bfloat16)
+    qg = Bd.fp4attn_quantize(dev(q), w.qk_fmt, Bd.ROLE_Q)
+    kg = Bd.fp4attn_quantize(dev(k), w.qk_fmt, Bd.ROLE_K)
+    vg = Bd.fp4attn_quantize_v_e4m3(dev(v)) if args.route == "fp8" else Bd.fp4attn_quantize(dev(v), Bd.FMT_MXFP4, Bd.ROLE_V)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rule = {"ceil": Bd.PSCALE_CEIL, "thr16": Bd.PSCALE_THR16, "mse": Bd.PSCALE_MSE}[args.p_scale]
+    O, L = Bd.fp4attn_fwd(qg, kg, vg, status=status, p_map=Bd.PMAP_AFFINE if args.p_map == "affine" else Bd.PMAP_IDEAL,
+                          p_scale_rule=rule, seq_len=None if lens is None else torch.tensor(lens, dtype=torch.int32, device="cuda"))
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    np.savez(path, O=O.float().cpu().numpy(), L=L.cpu().numpy())
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("workload", choices=sorted(I.WORKLOADS))
@@ -98,39 +118,32 @@ def main():
     ap.add_argument("--workers", type=int, default=max(1, len(os.sched_getaffinity(0)) - 2))
     ap.add_argument("--units", default=None, help="begin:end slice of the (batch, head) units, default all")
     args = ap.parse_args()
-    import torch
     from oracle import quantize as Qz
-    from paper_2609_04105_b200 import binding as Bd
     w = I.WORKLOADS[args.workload]
-    q, k, v = I.make_qkv(w)
-    dev = lambda a: torch.from_numpy(a.view(np.int16)).cuda().view(torch.bfloat16)
-    qg = Bd.fp4attn_quantize(dev(q), w.qk_fmt, Bd.ROLE_Q)
-    kg = Bd.fp4attn_quantize(dev(k), w.qk_fmt, Bd.ROLE_K)
-    vg = Bd.fp4attn_quantize_v_e4m3(dev(v)) if args.route == "fp8" else Bd.fp4attn_quantize(dev(v), Bd.FMT_MXFP4, Bd.ROLE_V)
-    status = torch.zeros(1, dtype=torch.int32, device="cuda")
     lens = None
     if args.length_mix:
         assert w.B >= 4, "the length mix needs four batch entries"
         lens = [w.N, w.N * 5 // 8 - 120, w.N // 2 + 1, 300] + [w.N] * (w.B - 4)
-    rule = {"ceil": Bd.PSCALE_CEIL, "thr16": Bd.PSCALE_THR16, "mse": Bd.PSCALE_MSE}[args.p_scale]
     assert args.route == "fp4" or args.p_scale == "ceil", "the FP8 P/V route has one rule"
-    O, L = Bd.fp4attn_fwd(qg, kg, vg, status=status, p_map=Bd.PMAP_AFFINE if args.p_map == "affine" else Bd.PMAP_IDEAL,
-                          p_scale_rule=rule, seq_len=None if lens is None else torch.tensor(lens, dtype=torch.int32, device="cuda"))
-    torch.cuda.synchronize()
-    assert int(status.item()) == 0
-    _G.update(lens=lens, route=args.route, w=w, q=q, k=k, v=v, O=O.float().cpu().numpy(), L=L.cpu().numpy(), Gq=None, Gk=None,
-              okw=dict(p_map=args.p_map, p_scale=args.p_scale))
+    with tempfile.TemporaryDirectory() as tmp:                   # CUDA in a process of its own: this one forks the oracle's workers
+        path = os.path.join(tmp, "launch.npz")
+        child = mp.get_context("spawn").Process(target=_launch, args=(args, lens, path))
+        child.start()
+        child.join()
+        assert child.exitcode == 0, "the launch failed"
+        res = np.load(path)
+        O, L = res["O"], res["L"]
+    q, k, v = I.make_qkv(w)
+    _G.update(lens=lens, route=args.route, w=w, q=q, k=k, v=v, O=O, L=L, Gq=None, Gk=None, okw=dict(p_map=args.p_map, p_scale=args.p_scale))
     if w.qk_fmt == I.FMT_NVFP4:
         _G["Gq"] = Qz.nv_tensor_scale(Qz.bf16_bits_to_f64(q))
         _G["Gk"] = Qz.nv_tensor_scale(Qz.bf16_bits_to_f64(k))
-    del qg, kg, vg, O, L
-    torch.cuda.empty_cache()
     units = [(b, h) for b in range(w.B) for h in range(w.H)]
     if args.units:
         lo, hi = (int(x) for x in args.units.split(":"))
         units = units[lo:hi]
     t0 = time.perf_counter()
-    with mp.get_context("fork").Pool(args.workers) as pool:        # workers inherit the arrays; they never touch CUDA
+    with mp.get_context("fork").Pool(args.workers) as pool:        # workers inherit the arrays
         res = []
         for st in pool.imap_unordered(_unit, units):
             print(json.dumps(st), flush=True)
