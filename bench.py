@@ -18,8 +18,8 @@ clock-normalised figure beside the raw one.
 
 Rooflines: `roofline` holds the attention kernel against the tensor roof (measured bf16 burst x 4);
 `roofline_softmax_arith` holds the same kernel against what its softmax arithmetic alone allows on this device
-(the kernel's score -> code instruction stream run by itself, four warps per scheduler: with exact codes the
-special-function unit binds it); `roofline_quantize` the quantizers against the measured copy bandwidth.
+(the kernel's score -> code instruction stream run by itself, four warps per scheduler: dispatch binds it, with
+no unit above three quarters busy); `roofline_quantize` the quantizers against the measured copy bandwidth.
 
 N > 1 is launched with torch.distributed.run (one rank per GPU); every rank runs the same
 workload on its own batch (independent (batch, head) units, no data-path collective), so the
